@@ -90,10 +90,10 @@ typedef enum {
  * Create an engine for fixed sizes on the current CUDA device.
  *   nstation N >= 1, npol P in {1, 2}, nfreq F >= 1 (at most 65535),
  *   ntime T >= 1.
- * Allocates the workspace: a ring of tensor-core operand tiles for the
- * channels in flight (about 1.6 x 152 / (blocks per channel) + 4 channel
- * slots, at most 256 MiB; 60 MiB for N=256 x 2 pols, T=1000, sized to stay
- * in L2), plus counters and a status word.  Small arrays (N*P <= 64) have k
+ * Allocates the workspace: a ring of tensor-core operand tiles (60 to 120 MiB,
+ * or the whole operand set if that is less, so that it stays in L2; at least
+ * one channel),
+ * plus counters and a status word.  Small arrays (N*P <= 64) have k
  * consecutive channels correlated together in one tensor-core block (k the
  * largest divisor of F with k*N*P <= 128); this is internal and changes
  * neither layouts nor results.  Returns NULL on error; the reason is in
@@ -227,8 +227,9 @@ enum { XC_PREC_FP16 = 0, XC_PREC_HILO = 1, XC_PREC_FP8 = 2 };
  *   XC_TILE_AUTO: XC_TILE_SMALL where it applies (see
  *     xc_small_engine_channels; an input pointer that is not 16-byte aligned
  *     keeps the planar engine), else
- *     XC_TILE_128, the fastest planar shape measured on the Large-N
- *     workload.  A batch handle takes the shape xc_batch_tune chose
+ *     the planar shape measured fastest: XC_TILE_WIDE for 8-bit input with
+ *     fp16 operands, nstation * npol > 896 and ntime > 4032, XC_TILE_128 for
+ *     the rest.  A batch handle takes the shape xc_batch_tune chose
  *     (XC_TILE_AUTO restores the default). */
 enum { XC_TILE_AUTO = 0, XC_TILE_128 = 1, XC_TILE_PAIR = 2, XC_TILE_WIDE = 3, XC_TILE_SMALL = 4 };
 /* Engines:
@@ -348,10 +349,10 @@ int xc_small_engine_channels(int nstation, int npol);
  * Its scratch is a static device array of XC_NOALLOC_SCRATCH_BYTES that
  * every GPU loading the library holds until the process exits.  The planar
  * engine keeps in it the kernel's counters, the scale pre-pass maxima
- * (nfreq*npol*nstation words for float input) and as many operand-ring
- * channel slots as fit; one slot is 2*P*N rows (rounded up to 128) x ntime
- * (rounded up to 64) x 2 bytes.  A size where not even one slot fits is
- * rejected with XC_ERR_UNSUPPORTED (message in xc_last_error_message()).
+ * (nfreq*npol*nstation words for float input) and as much of the operand
+ * ring as fits.  A size where not even one channel's operands fit (2*P*N rows,
+ * rounded up to 128, x ntime, rounded up to 64, x 2 bytes) is rejected with
+ * XC_ERR_UNSUPPORTED (message in xc_last_error_message()).
  * The small-array engine uses only the status word.
  *
  *   sizes, in_dtype, in, out: as for xc_create / xc_correlate.

@@ -79,11 +79,10 @@ struct BatchSub {
   xc::Geometry g{};
   xc::Geometry pg{};   // planar engine's geometry: `pack` channels per virtual channel
   int pack = 1;
-  int slots_unpacked = 0;  // ring depth 1x without channel packing (pack > 1 only)
+  xc::PlanarRing ring1{}, ring1_unpacked{};  // ring depth 1x, with and without channel packing
   size_t in_bytes = 0, out_bytes = 0;
   void* ring = nullptr;
-  int slots_base = 0;  // ring depth 1x (xc::planar_ring_slots)
-  int max_slots = 0;   // slots the region holds (for the 2x candidate)
+  size_t ring_bytes = 0;  // the region's size (for the 2x candidate)
   unsigned* counters = nullptr;
   unsigned* amax = nullptr;
 };
@@ -119,9 +118,9 @@ struct xc_handle {
   void* ring = nullptr;
   int ring_slots = 0;
   unsigned* counters = nullptr;
-  unsigned* chan_amax = nullptr;  // [F] per-channel max |x| (planar engine)
+  unsigned* chan_amax = nullptr;  // [F][nseg] max |x| per channel segment (planar engine)
   CUtensorMap ring_tmap;     // interleaved form: {Tp, R, ring_slots}
-  int planar_slots = 0;       // planar form: xc::planar_slot_bytes() per slot
+  xc::PlanarRing pring{};     // planar form
   // Planar engine geometry: small arrays pack `pack` consecutive channels into
   // one virtual channel (xc::planar_geometry); pg is that virtual geometry.
   xc::Geometry pg{};
@@ -170,12 +169,12 @@ xc_status encode_operand_map(CUtensorMap* map, void* base, int64_t R, int64_t Tp
 void batch_drop_graph(BatchState* b);
 
 // Planar tile shape for an XC_TILE_* option value (-1: not available).
-int planar_shape(int tile, const xc::Geometry& pg, int fmt) {
+int planar_shape(int tile, const xc::Geometry& pg, int in_dtype, int fmt) {
   switch (tile) {
     case XC_TILE_128: return xc::kPlanar128;
     case XC_TILE_PAIR: return xc::kPlanarPair;
     case XC_TILE_WIDE: return fmt == XC_PREC_HILO ? -1 : xc::kPlanarWide;
-    default: return xc::planar_default_shape(pg, fmt);
+    default: return xc::planar_default_shape(pg, in_dtype, fmt);
   }
 }
 
@@ -301,7 +300,8 @@ xc_status launch_one(xc_handle* h, const void* in, void* out, cudaStream_t s) {
     X.out = out;
     X.accumulate = h->accumulate;
     X.ring = h->ring;
-    X.ring_slots = h->planar_slots;
+    X.ring_slots = h->pring.slots;
+    X.ring_seg_kb = h->pring.seg_kb;
     X.counters = h->counters;
     X.amax = h->chan_amax;
     X.gains = gains;
@@ -321,7 +321,7 @@ xc_status launch_one(xc_handle* h, const void* in, void* out, cudaStream_t s) {
       im = &in_map;
     }
     if (tm) tm->nkern = 1;
-    const int shape = planar_shape(h->tile, h->pg, X.in_dtype == 0 ? 0 : h->precision);
+    const int shape = planar_shape(h->tile, h->pg, X.in_dtype, h->precision);
     if (shape < 0) return fail(XC_ERR_UNSUPPORTED, "hi/lo operands do not run on XC_TILE_WIDE");
     e = xc::launch_planar(im, X, shape, s);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core X-engine launch");
@@ -646,16 +646,16 @@ xc_handle* xc_create(int nstation, int npol, int nfreq, int ntime, xc_dtype in_d
   }
   h->ring_slots = xc::xengine_ring_slots(h->g);
   h->pg = xc::planar_geometry(h->g, &h->pack);
-  h->planar_slots = xc::planar_ring_slots(h->pg, h->num_sms, XC_PREC_FP16);
-  const int slots = std::max({h->ring_slots, h->planar_slots, xc::kMaxRingSlots});
+  h->pring = xc::planar_ring(h->pg, in_dtype, XC_PREC_FP16, h->num_sms);
+  const int slots = std::max({h->ring_slots, h->pring.slots, xc::kMaxRingSlots});
   h->ring_bytes = std::max(static_cast<size_t>(h->ring_slots) * R * Tp * 2,
-                           static_cast<size_t>(h->planar_slots) *
-                               xc::planar_slot_bytes(h->pg, XC_PREC_FP16));
+                           static_cast<size_t>(h->pring.slots) * h->pring.slot_bytes);
   e = cudaMalloc(&h->ring, h->ring_bytes);
   if (e == cudaSuccess)
     e = cudaMalloc(reinterpret_cast<void**>(&h->counters), 2 * sizeof(unsigned) * slots);
   if (e == cudaSuccess)
-    e = cudaMalloc(reinterpret_cast<void**>(&h->chan_amax), sizeof(unsigned) * nfreq);
+    e = cudaMalloc(reinterpret_cast<void**>(&h->chan_amax),
+                   sizeof(unsigned) * static_cast<size_t>(nfreq) * h->pring.nseg);
   if (e == cudaSuccess && in_dtype != XC_CI8)
     e = cudaMalloc(reinterpret_cast<void**>(&h->in_amax),
                    sizeof(unsigned) * static_cast<size_t>(nfreq) * nstation * npol);
@@ -710,8 +710,8 @@ xc_status xc_set_option(xc_handle* h, int key, long long value) {
       if (h->dtype == XC_CI8 && value == XC_PREC_HILO)
         return fail(XC_ERR_UNSUPPORTED, "8-bit input is exact in fp16; hi/lo applies to float input");
       const int fmt = static_cast<int>(value);
-      const int slots = xc::planar_ring_slots(h->pg, h->num_sms, fmt);
-      const size_t need = static_cast<size_t>(slots) * xc::planar_slot_bytes(h->pg, fmt);
+      const xc::PlanarRing pr = xc::planar_ring(h->pg, h->dtype, fmt, h->num_sms);
+      const size_t need = static_cast<size_t>(pr.slots) * pr.slot_bytes;
       if (need > h->ring_bytes) {
         // Work already queued may still use the ring.
         cudaError_t e = cudaDeviceSynchronize();
@@ -728,7 +728,7 @@ xc_status xc_set_option(xc_handle* h, int key, long long value) {
         h->ring_bytes = need;
       }
       h->precision = fmt;
-      h->planar_slots = slots;
+      h->pring = pr;
       return succeed();
     }
     case XC_OPT_TILE:
@@ -739,7 +739,7 @@ xc_status xc_set_option(xc_handle* h, int key, long long value) {
         return fail(XC_ERR_UNSUPPORTED, "batched launches run on the planar engine");
       if (h->batch) {
         h->batch->shape = value == XC_TILE_AUTO ? h->batch->shape_default
-                                                : planar_shape(static_cast<int>(value), h->pg, 0);
+                                                : planar_shape(static_cast<int>(value), h->pg, XC_CI8, XC_PREC_FP16);
         batch_drop_graph(h->batch);
       }
       h->tile = static_cast<int>(value);
@@ -1127,7 +1127,11 @@ xc_status batch_prepare(xc_handle* h, const void* const* in, void* const* out,
     X.out = out[i];
     X.accumulate = h->accumulate;
     X.ring = s.ring;
-    X.ring_slots = std::min(s.max_slots, (packed ? s.slots_base : s.slots_unpacked) * depth);
+    const xc::PlanarRing& pr = packed ? s.ring1 : s.ring1_unpacked;
+    X.ring_slots = static_cast<int>(std::min<int64_t>(
+        {static_cast<int64_t>(s.ring_bytes) / pr.slot_bytes, static_cast<int64_t>(pr.slots) * depth,
+         std::max<int64_t>(xc::kMaxRingSlots, pr.slots)}));
+    X.ring_seg_kb = pr.seg_kb;
     X.counters = s.counters;
     X.amax = s.amax;
     X.gains = nullptr;
@@ -1207,26 +1211,25 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
     s.in_bytes = static_cast<size_t>(ntime[i]) * nfreq[i] * nstation[i] * npol * 2;
     s.out_bytes = static_cast<size_t>(nfreq[i]) * s.g.NB * npol * npol * 2 * 4;
     s.pg = xc::planar_geometry(s.g, &s.pack);
-    const int64_t slot_bytes = xc::planar_slot_bytes(s.pg, XC_PREC_FP16);
-    s.slots_base = xc::planar_ring_slots(s.pg, h->num_sms, XC_PREC_FP16);
-    const int64_t cap2 = std::max<int64_t>(s.slots_base, (512ll << 20) / std::max<int64_t>(slot_bytes, 1));
-    s.max_slots = static_cast<int>(std::min<int64_t>(
-        {static_cast<int64_t>(xc::kMaxRingSlots), static_cast<int64_t>(s.pg.F), 2ll * s.slots_base, cap2}));
-    s.max_slots = std::max(s.max_slots, s.slots_base);
-    if (s.pack > 1) {
-      // Unpacked, the same channel slot size (one 128-input block) serves
-      // pack times as many channels.
-      s.slots_unpacked = std::min(s.max_slots, xc::planar_ring_slots(s.g, h->num_sms, XC_PREC_FP16));
-    }
+    s.ring1 = xc::planar_ring(s.pg, XC_CI8, XC_PREC_FP16, h->num_sms);
+    s.ring1_unpacked = xc::planar_ring(s.g, XC_CI8, XC_PREC_FP16, h->num_sms);
+    // Depth 2x may not take more than 512 MiB.
+    const size_t one = std::max(static_cast<size_t>(s.ring1.slots) * s.ring1.slot_bytes,
+                                static_cast<size_t>(s.ring1_unpacked.slots) * s.ring1_unpacked.slot_bytes);
+    s.ring_bytes = std::max(one, std::min<size_t>(2 * one, 512u << 20));
     ring_off[i] = ring_total;
-    ring_total += static_cast<size_t>(s.max_slots) * slot_bytes;
+    ring_total += (s.ring_bytes + 255) / 256 * 256;
     in_total += s.in_bytes;
     out_total += s.out_bytes;
   }
   h->in_bytes = in_total;
   h->out_bytes = out_total;
   size_t ctr_words = 0;
-  for (int i = 0; i < nsub; ++i) ctr_words += 2 * xc::kMaxRingSlots + b->sub[i].g.F;
+  auto ctr_of = [](const BatchSub& s) {  // ready and done counters of the deepest ring
+    return 2 * static_cast<size_t>(std::max({xc::kMaxRingSlots, s.ring1.slots, s.ring1_unpacked.slots}));
+  };
+  for (int i = 0; i < nsub; ++i)
+    ctr_words += ctr_of(b->sub[i]) + static_cast<size_t>(b->sub[i].g.F) * b->sub[i].ring1.nseg;
   cudaError_t e = cudaMalloc(&b->ring_all, ring_total);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&b->ctr_all), ctr_words * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
@@ -1240,15 +1243,15 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
     BatchSub& s = b->sub[i];
     s.ring = static_cast<char*>(b->ring_all) + ring_off[i];
     s.counters = c;
-    c += 2 * xc::kMaxRingSlots;
+    c += ctr_of(s);
     s.amax = c;
-    c += s.g.F;
+    c += static_cast<size_t>(s.g.F) * s.ring1.nseg;
     b->order[i] = i;
   }
   b->depth = 1;
   // The larger shape pays when some subarray has more than one block row.
   for (int i = 0; i < nsub; ++i)
-    b->shape_default = std::max(b->shape_default, xc::planar_default_shape(b->sub[i].pg, 0));
+    b->shape_default = std::max(b->shape_default, xc::planar_default_shape(b->sub[i].pg, XC_CI8, XC_PREC_FP16));
   b->shape = b->shape_default;
   succeed();
   return h;

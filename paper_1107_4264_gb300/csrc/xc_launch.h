@@ -37,9 +37,10 @@ struct XeLaunch {
   void* out;
   int accumulate;
   void* ring;
-  int ring_slots;
+  int ring_slots;      // planar engine: segment slots
+  int ring_seg_kb = 0; // planar engine: K-blocks per ring segment
   unsigned* counters;  // 2 * ring_slots, zeroed by the launcher on `s`
-  unsigned* amax;      // [F] per-channel max |x| (planar engine, 8-bit input)
+  unsigned* amax;      // [F][segments] max |x| (planar engine, 8-bit input)
   const void* gains;   // cf32 [N][P] applied to float input (planar engine), or NULL
   // Planar engine, float input:
   int fmt = 0;              // operand format: 0 fp16, 1 split hi/lo fp16, 2 e4m3
@@ -56,7 +57,7 @@ struct XeLaunch {
 };
 cudaError_t launch_xengine(const CUtensorMap* tmap, const XeLaunch& p, cudaStream_t s);
 // Planar complex form (separate real/imaginary fp16 planes, 4 MMAs per step
-// into D_re/D_im).  The ring holds planar_slot_bytes() per channel slot;
+// into D_re/D_im).  The ring holds PlanarRing::slot_bytes per segment slot;
 // `in_map` (8-bit input with R % 16 == 0, else NULL) is {R, F, T} int8 in
 // 128 x 1 x 64 boxes.  shape: kPlanar128 (128 x 128 blocks on single CTAs),
 // kPlanarPair (two blocks sharing a column block on a CTA pair, tcgen05
@@ -64,13 +65,22 @@ cudaError_t launch_xengine(const CUtensorMap* tmap, const XeLaunch& p, cudaStrea
 // N = 256 MMAs).
 enum : int { kPlanar128 = 0, kPlanarPair = 1, kPlanarWide = 2 };
 cudaError_t launch_planar(const CUtensorMap* in_map, const XeLaunch& p, int shape, cudaStream_t s);
-// The default shape for a (virtual) geometry and operand format.
-int planar_default_shape(const Geometry& g, int fmt);
-constexpr int kMaxRingSlots = 256;
+// The default shape for a (virtual) geometry, input type and operand format.
+int planar_default_shape(const Geometry& g, int in_dtype, int fmt);
+constexpr int kMaxRingSlots = 1024;
 // Samples per converter unit of the planar engine (8-bit input arrives by TMA
 // in 128-row x 1 x kPlanarUnitT boxes).
 constexpr int kPlanarUnitT = 64;
-int planar_ring_slots(const Geometry& g, int grid, int fmt);
+// The planar engine's operand ring: a channel's K-blocks are split into nseg
+// segments of seg_kb (the last one shorter), and a slot holds one segment's
+// operand tiles.
+struct PlanarRing {
+  int seg_kb, nseg, slots;
+  int64_t slot_bytes;
+};
+PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid);
+// The same with one segment per channel (the least memory that works: one slot).
+PlanarRing planar_ring_whole(const Geometry& g, int fmt);
 // Small arrays (n = N P <= 64 inputs): k consecutive channels, k the largest
 // divisor of F with k n <= 128, are correlated as one virtual channel of k N
 // stations.  The input [T][F][n] is the same memory as [T][F / k][k n], so
@@ -85,7 +95,6 @@ Geometry planar_geometry(const Geometry& g, int* pack);
 // of two in [16, 4096]; taps NULL needs ntaps = 1.
 cudaError_t launch_fengine(const void* in, int in_dtype, void* out, int out_dtype, int n, int F,
                            int T, float scale, const float* taps, int ntaps, cudaStream_t s);
-int64_t planar_slot_bytes(const Geometry& g, int fmt);
 
 // One planar launch over up to kMaxSub subarrays (same input type and
 // format; every subarray with its own ring region, counters and buffers).

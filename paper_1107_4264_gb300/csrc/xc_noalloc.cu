@@ -16,9 +16,9 @@
 // (it needs no scratch), else the planar engine (same tile shape, same
 // operand formation and scaling, same exact chunks for 8-bit input), so its
 // visibilities are identical to xc_correlate's.  The planar scratch
-// holds, in order: the status word, the ring counters, the per-channel and
-// per-(channel, input) maxima of the scale pre-pass, and then as many
-// operand-ring channel slots as fit.  All work is queued on the caller's
+// holds, in order: the status word, the per-(channel, input) maxima of the
+// scale pre-pass, the ring counters, the per-segment maxima of 8-bit input,
+// and then as many operand-ring slots as fit.  All work is queued on the caller's
 // stream.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -155,25 +155,35 @@ extern "C" xc_status xc_correlate_noalloc(int nstation, int npol, int nfreq, int
   const xc::Geometry pg = xc::planar_geometry(g, &pack);
   const int64_t n = static_cast<int64_t>(pg.N) * pg.P;
 
-  // Scratch plan: status | counters | per-channel max |x| | per-(channel,
-  // input) maxima (float input) | ring slots.
-  const int64_t off_ctr = 256;
-  const int64_t off_amax = off_ctr + round256(2LL * xc::kMaxRingSlots * 4);
-  const int64_t off_inamax = off_amax + round256(static_cast<int64_t>(pg.F) * 4);
-  const int64_t off_ring =
-      off_inamax + (in_dtype == XC_CI8 ? 0 : round256(static_cast<int64_t>(pg.F) * n * 4));
-  const int64_t slot_bytes = xc::planar_slot_bytes(pg, XC_PREC_FP16);
-  const int64_t room = static_cast<int64_t>(XC_NOALLOC_SCRATCH_BYTES) - off_ring;
-  if (room < slot_bytes)
+  // Scratch plan: status | per-(channel, input) maxima (float input) | ring
+  // counters | per-segment max |x| | ring slots.  The least that works is one
+  // whole channel: sizes for which not even that fits are refused (the bound
+  // counts fixed room for the counters and per-channel maxima).
+  const int64_t inamax_bytes = in_dtype == XC_CI8 ? 0 : round256(static_cast<int64_t>(pg.F) * n * 4);
+  xc::PlanarRing ring = xc::planar_ring_whole(pg, XC_PREC_FP16);
+  const int64_t fixed = 256 + 2048 + round256(static_cast<int64_t>(pg.F) * 4) + inamax_bytes;
+  if (static_cast<int64_t>(XC_NOALLOC_SCRATCH_BYTES) - fixed < ring.slot_bytes)
     return record_error(XC_ERR_UNSUPPORTED,
                         "the static scratch (%u bytes) cannot hold one channel's operands (%lld "
                         "bytes: 2*npol*nstation rows x ntime rounded up to 64 x 2 bytes) after its "
                         "%lld bytes of counters and scales",
-                        XC_NOALLOC_SCRATCH_BYTES, static_cast<long long>(slot_bytes),
-                        static_cast<long long>(off_ring));
-
-  const int slots = static_cast<int>(
-      std::min<int64_t>(xc::planar_ring_slots(pg, s.num_sms, XC_PREC_FP16), room / slot_bytes));
+                        XC_NOALLOC_SCRATCH_BYTES, static_cast<long long>(ring.slot_bytes),
+                        static_cast<long long>(fixed));
+  const int64_t off_inamax = 256;
+  const int64_t off_ctr = off_inamax + inamax_bytes;
+  // Slots that fit, with two counters each, beside nseg maxima per channel.
+  auto slots_for = [&](const xc::PlanarRing& r) {
+    const int64_t room = static_cast<int64_t>(XC_NOALLOC_SCRATCH_BYTES) - off_ctr - 256 -
+                         static_cast<int64_t>(pg.F) * r.nseg * 4;
+    return std::min<int64_t>(r.slots, room / (r.slot_bytes + 8));
+  };
+  xc::PlanarRing segs = xc::planar_ring(pg, in_dtype, XC_PREC_FP16, s.num_sms);
+  if (slots_for(segs) >= segs.nseg) {
+    ring = segs;
+    ring.slots = static_cast<int>(slots_for(segs));
+  }
+  const int64_t off_amax = off_ctr + 2LL * ring.slots * 4;
+  const int64_t off_ring = round256(off_amax + static_cast<int64_t>(pg.F) * ring.nseg * 4);
   xc::XeLaunch X;
   X.g = pg;
   X.pack = pack;
@@ -182,7 +192,8 @@ extern "C" xc_status xc_correlate_noalloc(int nstation, int npol, int nfreq, int
   X.out = out;
   X.accumulate = 0;
   X.ring = s.scratch + off_ring;
-  X.ring_slots = slots;
+  X.ring_slots = ring.slots;
+  X.ring_seg_kb = ring.seg_kb;
   X.counters = reinterpret_cast<unsigned*>(s.scratch + off_ctr);
   X.amax = reinterpret_cast<unsigned*>(s.scratch + off_amax);
   X.gains = nullptr;
@@ -203,7 +214,7 @@ extern "C" xc_status xc_correlate_noalloc(int nstation, int npol, int nfreq, int
   // Kernel parameter block on the stack: nothing is allocated, host or device.
   xc::PlanarKernel k;
   const CUtensorMap* maps[1] = {im};
-  cudaError_t e = xc::planar_prepare(&X, maps, 1, &k, xc::planar_default_shape(pg, XC_PREC_FP16));
+  cudaError_t e = xc::planar_prepare(&X, maps, 1, &k, xc::planar_default_shape(pg, in_dtype, XC_PREC_FP16));
   if (e == cudaSuccess && k.grid > 0) e = xc::planar_setup(&X, 1, st);
   if (e == cudaSuccess) e = xc::planar_launch(k, st);
   if (e != cudaSuccess) {

@@ -72,6 +72,11 @@ __global__ void __launch_bounds__(128) input_amax_kernel(const void* __restrict_
 int fmt_kt(int fmt) { return fmt == kFmtHiLo ? 2 : 1; }
 int fmt_tile_bytes(int fmt) { return fmt == kFmtF8 ? (1 << 13) : (1 << 14); }
 
+// fast_div's magic of a divisor (0 for a divisor of 0, which nothing divides by).
+unsigned div_magic(int d) {
+  return d <= 0 ? 0u : d == 1 ? 0xffffffffu : static_cast<unsigned>((1ull << 32) / static_cast<unsigned>(d));
+}
+
 // Kernel parameters of one subarray.
 Params sub_params(const XeLaunch& L, int shape) {
   Params p;
@@ -87,7 +92,9 @@ Params sub_params(const XeLaunch& L, int shape) {
   p.nkb = L.g.Tp / kBK;
   p.is_int = L.in_dtype == 0 ? 1 : 0;
   const int fmt = p.is_int ? (L.fmt == kFmtF8 ? kFmtF8 : kFmtF16) : L.fmt;
-  p.nkt = fmt_kt(fmt) * p.nkb;
+  p.seg_kb = std::max(1, L.ring_seg_kb);
+  p.nseg = (p.nkb + p.seg_kb - 1) / p.seg_kb;
+  p.nkt = fmt_kt(fmt) * p.seg_kb;
   p.amax = L.amax;
   p.gains = static_cast<const float2*>(L.gains);
   p.in_amax = p.is_int ? nullptr : L.in_amax;
@@ -98,8 +105,9 @@ Params sub_params(const XeLaunch& L, int shape) {
   p.ring_slots = L.ring_slots;
   p.ready = L.counters;
   p.done = L.counters + L.ring_slots;
-  p.row_units = 2 * p.nib;
-  p.units_per_chan = p.row_units * p.nkb * (kBK / kUnitT);
+  p.seg_units = 2 * p.nib * p.seg_kb;
+  p.mag_kb = div_magic(p.seg_kb);
+  p.mag_slots = div_magic(p.ring_slots);
   p.tma_in = 0;
   p.timeout_ns = L.timeout_ns;
   p.status = L.status;
@@ -112,11 +120,6 @@ Params sub_params(const XeLaunch& L, int shape) {
 }
 
 }  // namespace
-
-int64_t planar_slot_bytes(const Geometry& g, int fmt) {
-  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
-  return 2 * fmt_kt(fmt) * (g.Tp / kBK) * nib * fmt_tile_bytes(fmt);
-}
 
 Geometry planar_geometry(const Geometry& g, int* pack) {
   int k = 1;
@@ -138,26 +141,61 @@ Geometry planar_geometry(const Geometry& g, int* pack) {
   return v;
 }
 
-int planar_ring_slots(const Geometry& g, int grid, int fmt) {
-  // The persistent CTAs keep about grid / blocks_per_channel channels in
-  // flight; the converters need room ahead of them.
+namespace {
+PlanarRing ring_of(const Geometry& g, int fmt, int seg_kb) {
   const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
-  const int64_t blocks = std::max<int64_t>(1, nib * (nib + 1) / 2);
-  const int64_t inflight = (grid + blocks - 1) / blocks;
-  int64_t n = (inflight * 8 + 4) / 5 + 4;
-  const int64_t cap =
-      std::max<int64_t>(2, (256ll << 20) / std::max<int64_t>(planar_slot_bytes(g, fmt), 1));
-  n = std::max<int64_t>(4, std::min<int64_t>(std::min<int64_t>(kMaxRingSlots, cap), n));
-  return static_cast<int>(std::min<int64_t>(n, g.F));
+  PlanarRing r;
+  r.seg_kb = seg_kb;
+  r.nseg = (g.Tp / kBK + seg_kb - 1) / seg_kb;
+  r.slots = 1;
+  r.slot_bytes = 2 * fmt_kt(fmt) * static_cast<int64_t>(seg_kb) * nib * fmt_tile_bytes(fmt);
+  return r;
+}
+}  // namespace
+
+PlanarRing planar_ring_whole(const Geometry& g, int fmt) { return ring_of(g, fmt, g.Tp / kBK); }
+
+// 128 x 256 items for large arrays with long integrations, whose channels are
+// few and big: a quarter fewer operand bytes per MAC, and no more channels in
+// flight than the ring can feed.  Measured (8-bit input, ms, 128 x 128 / 128 x
+// 256): N=1024 F=16 T=8192 1.39 / 1.23, N=512 F=64 T=4096 0.81 / 0.71, N=256
+// F=64 T=8192 0.59 / 0.60, N=384 F=256 T=2048 0.96 / 0.95, N=1024 F=32 T=1000
+// 0.41 / 0.40, N=256 F=1024 T=1000 0.98 / 1.01.  Float input, whose converters
+// set the pace, stays with 128 x 128 (N=512 F=60 T=2048 0.75 / 0.87).
+int planar_default_shape(const Geometry& g, int in_dtype, int fmt) {
+  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
+  return in_dtype == 0 && fmt == kFmtF16 && nib >= 8 && g.Tp >= 4096 ? kShapeWide : kShape128;
 }
 
-int planar_default_shape(const Geometry& g, int fmt) {
-  // 128 x 128 measured fastest for the Large-N geometry (the larger shapes
-  // move fewer operand bytes per MAC but put more channels in flight than
-  // the L2-resident ring can run ahead of); the batch tuner tries all three.
-  (void)g;
-  (void)fmt;
-  return kShape128;
+// Segments of at most 8 K-blocks (512 samples; half as many with hi/lo
+// operands, which take twice the bytes) and 60 MiB of ring, so that it stays
+// in the 129 MB L2 beside the streams.  Measured (8-bit input, ms):
+//   K-blocks per segment       16     8     4
+//     N=100 F=512  T=1000   0.243 0.207 0.203
+//     N=256 F=1024 T=1000   0.987 0.969 0.988
+//     N=200 F=256  T=512    0.144 0.144 0.150
+//   ring                   50 MiB 60 MiB 75 MiB 90 MiB 120 MiB 250 MiB
+//     N=256 F=1024 T=1000   1.028  0.977  1.044  1.100   1.144
+//     N=256 F=256  T=4096          1.104         1.004   1.061   1.099
+//     N=256 F=64   T=8192          0.671         0.604   0.605   0.602
+//     N=512 F=64   T=4096          0.809         0.822   0.830   0.824
+// So 90 MiB when the channels of a wave take more than 80 MiB (8-bit input:
+// the float converters are too slow to fill it), and 120 MiB on 128 x 256
+// items (N=512 F=64 T=4096 0.708 against 0.777 ms).
+PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid) {
+  const int seg = fmt == kFmtHiLo ? 4 : 8;
+  const int nkb = g.Tp / kBK;
+  const int parts = (nkb + seg - 1) / seg;
+  PlanarRing r = ring_of(g, fmt, (nkb + parts - 1) / parts);
+  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
+  const int64_t wave = std::max<int64_t>(1, grid / (nib * (nib + 1) / 2));
+  int64_t mib = 60;
+  if (in_dtype == 0 && wave * r.nseg * r.slot_bytes > (80ll << 20)) mib = 90;
+  if (planar_default_shape(g, in_dtype, fmt) == kShapeWide) mib = 120;
+  int64_t n = std::min<int64_t>((mib << 20) / r.slot_bytes, kMaxRingSlots);
+  n = std::max<int64_t>(n, std::max<int64_t>(4, r.nseg + 4));
+  r.slots = static_cast<int>(std::min<int64_t>(n, static_cast<int64_t>(g.F) * r.nseg));
+  return r;
 }
 
 cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps, int nsub,
@@ -175,8 +213,8 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
   bool all_tma = true;
   for (int i = 0; i < nsub; ++i) {
     if (subs[i].in_dtype != dt || fmt_of(subs[i]) != fmt) return cudaErrorInvalidValue;
-    if (subs[i].ring_slots < 1 || subs[i].ring_slots > kMaxRingSlots) return cudaErrorInvalidValue;
     b->sub[i] = sub_params(subs[i], shape);
+    if (subs[i].ring_slots < 1) return cudaErrorInvalidValue;
     if (maps && maps[i]) {
       b->maps[i] = *maps[i];
     } else {
@@ -184,9 +222,10 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     }
     b->item_base[i + 1] = b->item_base[i] + (b->sub[i].nkb > 0 ? b->sub[i].nitems : 0);
     b->unit_base[i + 1] = b->unit_base[i] +
-                          (b->sub[i].nkb > 0 ? static_cast<long long>(subs[i].g.F) * b->sub[i].units_per_chan : 0);
+                          static_cast<long long>(subs[i].g.F) * b->sub[i].nseg * b->sub[i].seg_units;
   }
   for (int i = 0; i < nsub; ++i) b->sub[i].tma_in = all_tma ? 1 : 0;
+  const int conv = (fmt == kFmtF8 && dt == 0) ? conv_warps<kFmtF8, 0>() : conv_warps<kFmtF16, 0>();
   const bool pair = shape == kShapePair;
   switch (shape) {
     case kShape128: k->func = select_kernel(dt, fmt, nsub > 1); break;
@@ -226,6 +265,31 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     const long long resident = static_cast<long long>(per_sm) * subs[0].grid;
     k->grid = static_cast<int>(std::min<long long>({items, static_cast<long long>(subs[0].grid), resident}));
   }
+  // A converter warp's step from one run to its next, for its incremental
+  // unit numbers.
+  const long long step = static_cast<long long>(k->grid) * conv * kUnitRun;
+  for (int i = 0; i < nsub; ++i) {
+    Params& p = b->sub[i];
+    p.step_seg = static_cast<int>(step / p.seg_units);
+    p.step_rem = static_cast<int>(step % p.seg_units);
+    p.step_gen = p.step_seg / p.ring_slots;
+    p.step_slot = p.step_seg % p.ring_slots;
+    const int item_step = pair ? k->grid / 2 : k->grid;
+    // Waves: as many channels as there are CTAs (clusters) for their items,
+    // and no more than half the ring's slots.  (N=256 F=64 T=8192 on a 60 MiB
+    // ring: 0.686 ms, and 1.150 ms with one channel to a wave.)
+    p.wave = std::max(1, std::min({item_step / p.ipc, p.ring_slots / 2, p.g.F}));
+    if (p.ipc > item_step && p.ring_slots < p.nseg) return cudaErrorInvalidConfiguration;
+    p.wave_segs = p.wave * p.nseg;
+    p.wave_full = p.g.F / p.wave;
+    p.wave_last = p.g.F - p.wave_full * p.wave;
+    p.last_base = p.wave_full * p.wave_segs;
+    p.mag_wave = div_magic(p.wave);
+    p.mag_wsegs = div_magic(p.wave_segs);
+    p.mag_last = div_magic(p.wave_last);
+    p.it_step_f = item_step / p.ipc;
+    p.it_step_i = item_step % p.ipc;
+  }
   return cudaSuccess;
 }
 
@@ -234,8 +298,10 @@ cudaError_t planar_setup(const XeLaunch* subs, int nsub, cudaStream_t s) {
     const XeLaunch& L = subs[i];
     const int n = L.g.N * L.g.P;
     cudaError_t e = cudaMemsetAsync(L.counters, 0, 2 * sizeof(unsigned) * L.ring_slots, s);
-    if (e == cudaSuccess && L.in_dtype == 0)
-      e = cudaMemsetAsync(L.amax, 0, sizeof(unsigned) * L.g.F, s);
+    if (e == cudaSuccess && L.in_dtype == 0) {
+      const size_t nseg = (L.g.Tp / kBK + std::max(1, L.ring_seg_kb) - 1) / std::max(1, L.ring_seg_kb);
+      e = cudaMemsetAsync(L.amax, 0, sizeof(unsigned) * L.g.F * nseg, s);
+    }
     if (e != cudaSuccess) return e;
     if (L.in_dtype != 0 && L.in_amax) {
       e = cudaMemsetAsync(L.in_amax, 0, sizeof(unsigned) * L.g.F * static_cast<size_t>(n), s);

@@ -45,31 +45,50 @@
 // operands and store only their lower station triangle (Sec. 4.4).
 //
 // Operand formation (Sec. 4.1 input order, Sec. 5 8-bit samples): converter
-// warps form each channel's planes once into a ring of channel slots in
-// global memory that stays in L2; the blocks of a channel read it back with
-// bulk copies.  The ring holds operand tiles exactly as the MMA reads them:
-// per (slot, plane, 64-sample K-block, 128-input block) one 16 KiB tile in
-// the no-swizzle K-major canonical layout, K inside: [8-input group]
-// [8-sample chunk][8 inputs][16 B], so a stage is contiguous tile copies,
-// inputs 0..63 and 64..127 of a tile are its two contiguous halves, and the
-// 8 x 16 B core matrix that four converter lanes write is one whole line.
-// 8-bit input arrives by TMA in 128-row x 64-sample boxes (other types and
-// row counts by direct loads); lane l converts inputs l and l + 32 of a
-// 64-input half block; each converter warp works through its own stream of
-// units.  Ring protocol:
-//   ready[slot] counts converted units (128 rows x 64 samples); channel c
-//     (generation c / slots of slot c % slots) is complete at
-//     ready >= (gen + 1) * units_per_channel;
-//   done[slot] counts blocks whose operands have landed in shared memory;
-//     slot s may take channel c once done >= gen(c) * blocks_per_channel.
-// Dependencies point only to lower channels and all CTAs are co-resident,
-// so the ring cannot deadlock; every wait is bounded regardless.
+// warps form each channel's planes once into a ring in global memory that
+// stays in L2; the blocks of a channel read it back with bulk copies.  The
+// ring's unit is a segment of a channel (seg_kb K-blocks of 64 samples, all
+// its inputs); the channels at work at one time (a wave) are brought a segment
+// each in turn, so the ring's size follows neither the channels' length nor
+// how many of them are in flight (seg_first).
+// The ring holds operand tiles exactly as the MMA reads them: per (slot,
+// K-block, 128-input block) the two planes' tiles of 128 inputs x four 16-byte
+// K chunks (8 KiB) in the no-swizzle K-major canonical layout, K inside:
+// [8-input group][chunk][8 inputs][16 B], so a stage is one contiguous copy
+// per operand, inputs 0..63 and 64..127 of a tile are its two contiguous
+// halves, and the 8 x 16 B core matrix that four converter lanes write is one
+// whole line.  8-bit input arrives by TMA in 128-row x 64-sample boxes (other
+// types likewise, other row counts by direct loads); each converter warp works
+// through its own stream of units.  Ring protocol:
+//   ready[slot] counts converted units (64 inputs x 64 samples); segment G
+//     (generation G / slots of slot G % slots) is complete at
+//     ready >= (gen + 1) * units_per_segment;
+//   done[slot] counts work items whose MMAs have read the segment; slot s may
+//     take segment G once done >= gen(G) * items_per_channel.
+// A segment waits for segments of lower number only, and a work item for
+// segments of its own channel.  All CTAs are co-resident and each has at most
+// one item of a wave, so the items of the lowest number not yet read are at
+// work or come next once the waves before are done: the ring cannot deadlock.
+// (When a channel has more items than there are CTAs, a wave is one channel
+// and the ring holds all its segments.)  Every wait is bounded regardless.
 //
 // CTA roles (persistent, one CTA per SM, channel-major items):
-//   warp 0      producer: 3 stages x (Ar, Ai, Br, Bi) 64-sample tiles (bulk copies)
-//   warp 1      MMA issuer; owns TMEM (2 sets x {D_re, D_im} x 128 columns)
+//   warp 0      producer: 3 stages x (Ar, Ai, Br, Bi) of 64 samples (bulk copies);
+//               releases segments
+//   warp 1      MMA issuer; owns TMEM (2 sets x {D_im, D_re} x 128 columns)
 //   warps 2..5  epilogue
 //   warps 6..9  converters
+// What bounds it: the converters' and the epilogue's stores share the SM's
+// shared-memory path with the MMAs' operand reads.  Alone, the stage copies and
+// MMAs of a 64-sample step take 1050 cycles (1024 is the tensor rate); with 4
+// warps storing 64 KiB of tiles per 6500 cycles 1260-1320, with the epilogue's
+// stores as well 1580.  In the kernel a step takes about 1830 cycles on the
+// 256-station array (2040 when one thread per CTA walked the items, waited and
+// issued four 128 x 128 MMAs per K-step): 1.07 -> 0.97 ms at 1024 channels of
+// 1000 samples, 0.195 -> 0.144 ms for 200 stations, 256 channels of 512, and
+// 1.02 -> 0.62 ms at 2048 channels of 125 samples, where the ring of whole
+// channels was 30 slots deep whatever their size and each item cost every
+// role an FP64 square root and several divisions.
 //
 // CTA pairs (PAIR = true, tcgen05 cta_group::2, clusters of two CTAs): one
 // item is two 128 x 128 blocks sharing their column block b, computed by one
@@ -111,11 +130,10 @@ constexpr int kBK = 64;        // samples per stage
 constexpr int kNumEpiWarps = 4;
 constexpr int kNumConvWarps = 4;
 constexpr int kThreads = 32 * (2 + kNumEpiWarps + kNumConvWarps);
-constexpr int kTileBytes = kBlk * kBK * 2;  // 16 KiB: one plane tile
 constexpr uint32_t kTmemCols = 512;         // 2 sets x (D_re, D_im) x 128
 constexpr int kUnitRows = 128;  // converter unit: 128 real rows (64 inputs) x kUnitT samples
 constexpr int kUnitT = kPlanarUnitT;
-static_assert(kUnitT == 32 || kUnitT == 64, "a unit covers a whole or half 64-sample K-block");
+static_assert(kUnitT == kBK, "a unit covers one 64-sample K-block");
 constexpr uint32_t kCoreBytes = 8 * 16;  // one core matrix: 8 inputs x 16 bytes
 constexpr int kConvBufBytes = kUnitRows * kUnitT;  // int8 staging per converter warp
 
@@ -143,6 +161,26 @@ constexpr int threads_of() {
   return 32 * (2 + kNumEpiWarps + conv_warps<FMT, DT>());
 }
 
+// Operand formats.  A tile holds kChunks 16-byte K chunks of 128 inputs: the
+// 64 samples of a K-block, or half of them for fp16 operands on 128 x 256
+// items, whose two 96 KiB stages would leave little to run ahead with (a
+// stage is one tile per plane; on the other shapes finer stages lose more to
+// a stage's fixed cost in the MMA warp than they give: 128 x 128 on the
+// 256-station array 1.03 against 0.98 ms).
+template <int FMT, int SHAPE>
+struct FmtT {
+  static constexpr int kChunks = FMT == kFmtF8 || SHAPE == kShapeWide ? 4 : 8;
+  static constexpr int kTile = kBlk * 16 * kChunks;
+  static constexpr int kSplit = (FMT == kFmtF8 ? 4 : 8) / kChunks;  // tiles per plane and K-block
+  static constexpr int kHalves = FMT == kFmtHiLo ? 3 : 1;  // operand pairs per K-block (H H, L H, H L)
+  static constexpr int kSteps = kHalves * kSplit;          // stages per K-block
+  // A K-block of one input block in the ring: [kSplit][plane] tiles.
+  static constexpr int kKbBytes = kSplit * 2 * kTile;
+  // Bytes between 8-input groups of a tile (the descriptor's stride offset);
+  // core matrices adjacent in K are kCoreBytes apart (its leading offset).
+  static constexpr uint32_t kSbo = kChunks * kCoreBytes;
+};
+
 // Shared-memory plan per shape and operand format: stages of (Ar, Ai, Br,
 // Bi) tiles; (Ar, Ai, half Br, half Bi) on pairs; (Ar, Ai, Br Br', Bi Bi')
 // for 128 x 256; then the converters' staging buffers and the barriers.
@@ -152,9 +190,9 @@ template <int SHAPE, int FMT, int DT>
 struct Cfg {
   static constexpr bool kF8 = f8_int8_plan<FMT, DT>();
   static constexpr int kStages = kF8 ? (SHAPE == kShapePair ? 7 : (SHAPE == kShapeWide ? 3 : 5))
-                                     : (SHAPE == kShapePair ? 4 : (SHAPE == kShapeWide ? 2 : 3));
+                                     : (SHAPE == kShapePair ? 4 : (SHAPE == kShapeWide ? 4 : 3));
   static constexpr int kStageBytes =
-      (SHAPE == kShapePair ? 3 : (SHAPE == kShapeWide ? 6 : 4)) * (kF8 ? kTileBytes / 2 : kTileBytes);
+      (SHAPE == kShapePair ? 3 : (SHAPE == kShapeWide ? 6 : 4)) * FmtT<FMT, SHAPE>::kTile;
   static constexpr int kConvOff = kStages * kStageBytes;
   static constexpr int kBarOff = kConvOff + conv_warps<FMT, DT>() * kConvBufBytes;
   // full, empty (and pfull) per stage; accf, acce x 2; drain; one per converter
@@ -165,24 +203,13 @@ struct Cfg {
   static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
-// Operand formats: tile size (log2 bytes), 16-byte K chunks per tile and
-// MMA steps per 64-sample block (ring K-tiles per block: fmt_kt()).
-template <int FMT>
-struct FmtT {
-  static constexpr int kTileShift = FMT == kFmtF8 ? 13 : 14;
-  static constexpr int kTile = 1 << kTileShift;
-  static constexpr int kChunks = FMT == kFmtF8 ? 4 : 8;
-  static constexpr int kSteps = FMT == kFmtHiLo ? 3 : 1;
-  // Bytes between 8-input groups of a tile (the descriptor's stride offset);
-  // core matrices adjacent in K are kCoreBytes apart (its leading offset).
-  static constexpr uint32_t kSbo = kChunks * kCoreBytes;
-};
-
-// Byte offset of (input row, 16-byte K chunk) in a tile.
-template <int FMT>
+// Byte offset of (input row, 16-byte K chunk of the K-block) from the K-block's
+// first tile of a plane.
+template <int FMT, int SHAPE>
 __device__ __forceinline__ uint32_t tile_off(int row, int chunk) {
-  return static_cast<uint32_t>(row >> 3) * FmtT<FMT>::kSbo + static_cast<uint32_t>(chunk) * kCoreBytes +
-         static_cast<uint32_t>(row & 7) * 16u;
+  return static_cast<uint32_t>(chunk / FmtT<FMT, SHAPE>::kChunks) * (2 * FmtT<FMT, SHAPE>::kTile) +
+         static_cast<uint32_t>(row >> 3) * FmtT<FMT, SHAPE>::kSbo +
+         static_cast<uint32_t>(chunk % FmtT<FMT, SHAPE>::kChunks) * kCoreBytes + static_cast<uint32_t>(row & 7) * 16u;
 }
 
 struct Params {
@@ -196,19 +223,29 @@ struct Params {
   long long nitems;    // ipc * F
   int nkb;             // Tp / 64
   int is_int;          // 8-bit input: exact chunks from the channel's max |x|
-  unsigned* amax;      // [F] max |x| per channel (8-bit input), zeroed by the host
+  unsigned* amax;      // [F][nseg] max |x| per channel segment (8-bit input), zeroed by the host
   const float2* gains; // [n] complex gains applied to float input (y = g x), or NULL
   const unsigned* in_amax;  // [F][n] max component of g x (float bits), float input
   double* acc64;       // FP64 block sums: running visibility sums (output layout), or NULL
   int f_chunk_kb;      // float input: K-blocks per fp32 accumulation chunk
-  uint8_t* ring;       // tiles [slots][2][nkt][nib][chunks][128][16 B]
-  int nkt;             // K-tiles per plane per input block of a slot (nkb or 2 nkb)
+  uint8_t* ring;       // tiles [slots][nkt][nib][split][2][chunks][128][16 B]
+  int nkt;             // K-tiles per plane per input block of a slot (seg_kb or 2 seg_kb)
   int nib;             // 128-input blocks per channel
-  int ring_slots;
-  unsigned* ready;
-  unsigned* done;
-  int row_units;       // 64-input half blocks per channel = 2 * nib
-  int units_per_chan;  // row_units * Tp / 64
+  int seg_kb, nseg;    // K-blocks per ring segment; segments per channel
+  int ring_slots;      // segment slots, at least nseg
+  unsigned* ready;     // [ring_slots]
+  unsigned* done;      // [ring_slots]
+  int seg_units;       // converter units per segment = 2 * nib * seg_kb
+  // Channels go through the ring in waves of `wave` (the last one of
+  // wave_last, from segment number last_base on): see seg_first.
+  int wave, wave_segs, wave_full, wave_last, last_base;
+  unsigned mag_kb, mag_wave, mag_wsegs, mag_last, mag_slots;  // fast_div magics
+  // From one of a converter warp's runs to its next (kUnitRun * converter
+  // warps units on): step_seg segments and step_rem units, and step_seg as
+  // ring generations and slots.
+  int step_seg, step_rem, step_gen, step_slot;
+  // From one of a CTA's (cluster's) items to its next: channels and items.
+  int it_step_f, it_step_i;
   int tma_in;          // 8-bit input staged by TMA (else direct loads)
   unsigned long long timeout_ns;
   int* status;
@@ -295,12 +332,64 @@ __device__ __noinline__ bool wait_counter(const unsigned* p, unsigned target, co
   }
 }
 
-__device__ __forceinline__ void item_coords(long long it, int ntiles, int* f, int* bx, int* by) {
-  *f = static_cast<int>(it / ntiles);
-  int64_t x, y;
-  tri_coords(it % ntiles, &x, &y);
-  *bx = static_cast<int>(x);
+// Is a wait that began at t0 over (another role gave up, or the time is up)?
+// For loops that do something else in between.
+__device__ __noinline__ bool wait_given_up(const Params& prm, uint64_t t0, volatile int* abort_flag) {
+  if (*abort_flag) return true;
+  const bool late = ptx::globaltimer() - t0 > prm.timeout_ns;
+  if (!late && *reinterpret_cast<volatile int*>(prm.status) == 0) return false;
+  *abort_flag = 1;
+  if (late) atomicOr(prm.status, kStatusTimeout);
+  return true;
+}
+
+// A work item: its number in the launch, its subarray, channel and number in
+// the channel.  Stepped from item to item without divisions (and the block
+// coordinates below come from a float square root: the FP64 one of
+// tri_coords cost every role some thousand cycles per item).
+struct Item {
+  long long it;
+  int sb, f, i;
+};
+template <bool MULTI>
+__device__ __forceinline__ void item_locate(const Batch& bt, Item& x) {
+  x.sb = advance_sub<MULTI>(bt.item_base, bt.nsub, x.it, x.sb);
+  const Params& p = bt.sub[x.sb];
+  const long long v = x.it - bt.item_base[x.sb];
+  x.f = static_cast<int>(v / p.ipc);
+  x.i = static_cast<int>(v - static_cast<long long>(x.f) * p.ipc);
+}
+template <bool MULTI>
+__device__ __forceinline__ Item item_start(const Batch& bt, long long it, long long nitems) {
+  Item x = {it, 0, 0, 0};
+  if (it < nitems) item_locate<MULTI>(bt, x);
+  return x;
+}
+template <bool MULTI>
+__device__ __forceinline__ void item_step(const Batch& bt, Item& x, long long step, long long nitems) {
+  x.it += step;
+  if (x.it >= nitems) return;
+  if (MULTI && x.it >= bt.item_base[x.sb + 1]) {
+    item_locate<MULTI>(bt, x);
+    return;
+  }
+  const Params& p = bt.sub[x.sb];
+  x.f += p.it_step_f;
+  x.i += p.it_step_i;
+  if (x.i >= p.ipc) {
+    x.i -= p.ipc;
+    ++x.f;
+  }
+}
+
+// Lower block i of a channel: row by, column bx (Sec. 4.2's inverse map, the
+// float estimate corrected with exact integers).
+__device__ __forceinline__ void block_coords(int i, int* bx, int* by) {
+  long long y = static_cast<long long>((__fsqrt_rn(8.f * static_cast<float>(i) + 1.f) - 1.f) * 0.5f);
+  while (y * (y + 1) / 2 > i) --y;
+  while ((y + 1) * (y + 2) / 2 <= i) ++y;
   *by = static_cast<int>(y);
+  *bx = static_cast<int>(i - y * (y + 1) / 2);
 }
 
 // This CTA's share of work item `it` (local to its subarray): channel f,
@@ -313,20 +402,18 @@ struct Blk {
   bool idle;
 };
 template <int SHAPE>
-__device__ __forceinline__ Blk item_block(const Params& p, long long it, uint32_t rank) {
+__device__ __forceinline__ Blk item_block(const Params& p, const Item& x, uint32_t rank) {
   Blk k;
+  k.f = x.f;
   k.b2 = -1;
   k.idle = false;
   if constexpr (SHAPE == kShape128) {
-    int bx, by;
-    item_coords(it, p.ntiles, &k.f, &bx, &by);
-    k.a = by;
-    k.b = bx;
+    block_coords(x.i, &k.b, &k.a);
+    (void)p;
     (void)rank;
   } else {
-    k.f = static_cast<int>(it / p.ipc);
     int a0, a1, b, single;
-    pair_coords(static_cast<int>(it % p.ipc), p.nib, &a0, &a1, &b, &single);
+    pair_coords(x.i, p.nib, &a0, &a1, &b, &single);
     if constexpr (SHAPE == kShapePair) {
       k.a = rank ? a1 : a0;
       k.b = b;
@@ -343,22 +430,53 @@ __device__ __forceinline__ Blk item_block(const Params& p, long long it, uint32_
   return k;
 }
 
-// K-blocks per exact fp32 accumulation chunk for channel f (all K-blocks for
-// float input).  Called after the channel is known to be fully converted.
-__device__ __forceinline__ int chunk_kblocks(const Params& p, int f) {
-  if (!p.is_int) return p.f_chunk_kb;
-  const unsigned m = *reinterpret_cast<volatile const unsigned*>(p.amax + f);
-  if (m == 0) return p.nkb;
-  const unsigned long long per_block = 2ull * m * m * kBK;  // |partial| growth per K-block
-  const unsigned long long kb = (1ull << 24) / per_block;
-  return static_cast<int>(kb < 1 ? 1 : (kb > static_cast<unsigned long long>(p.nkb) ? p.nkb : kb));
+// x / d for a run-time d, with mag = floor(2^32 / d) (2^32 - 1 for d = 1):
+// the product's high word is the quotient or one less.
+__device__ __forceinline__ int fast_div(int x, int d, unsigned mag) {
+  const int q = static_cast<int>(__umulhi(static_cast<unsigned>(x), mag));
+  return x - q * d >= d ? q + 1 : q;
 }
 
-// Wait (bounded) until channel f is fully converted into its ring slot.
-__device__ __forceinline__ bool channel_ready(const Params& p, int f, volatile int* abort_flag) {
-  const unsigned gen = static_cast<unsigned>(f / p.ring_slots);
-  return wait_counter(p.ready + f % p.ring_slots, (gen + 1) * static_cast<unsigned>(p.units_per_chan),
-                      p, abort_flag);
+// Segments are numbered (and take ring slots, in turn) wave by wave, within a
+// wave segment by segment, within a segment channel by channel: the channels
+// that are worked on at the same time arrive together, a segment each, so the
+// ring need not hold whole channels of a long integration.  Channel f's
+// segments are numbers first, first + *width, first + 2 *width, ...
+// A wave holds no more work items than there are CTAs (or is one channel), so
+// all its items are at work at the same time and none waits for a segment
+// whose slot is held for an item that has yet to start.
+__device__ __forceinline__ int seg_first(const Params& p, int f, int* width) {
+  const int w = fast_div(f, p.wave, p.mag_wave);
+  *width = w < p.wave_full ? p.wave : p.wave_last;
+  return w * p.wave_segs + f - w * p.wave;
+}
+
+// 8-bit input: how much a partial sum can grow over one K-block of segment G
+// (its number in the subarray), from the segment's max |x|; at most 2^21.
+// Called after the segment is known to be converted.  A chunk is exact in
+// fp32 while its K-blocks' growths sum to at most kExactSum.
+constexpr unsigned kExactSum = 1u << 24;
+__device__ __forceinline__ unsigned kblock_growth(const Params& p, int G) {
+  const unsigned m = *reinterpret_cast<volatile const unsigned*>(p.amax + G);
+  return 2u * m * m * kBK;
+}
+
+// First K-block after the exact chunk that starts at kb0 of the channel whose
+// segments are G0, G0 + width, ...: the same walk as the producer's (which
+// tells the MMA warp).  Every segment of the channel has been converted.
+__device__ __forceinline__ int exact_chunk_end(const Params& p, int G0, int width, int kb0) {
+  int seg = kb0 / p.seg_kb, left = p.seg_kb - (kb0 - seg * p.seg_kb);
+  unsigned sum = 0, grow = kblock_growth(p, G0 + seg * width);
+  for (int kb = kb0; kb < p.nkb; ++kb) {
+    if (left == 0) {
+      grow = kblock_growth(p, G0 + ++seg * width);
+      left = p.seg_kb;
+    }
+    if (kb > kb0 && sum + grow > kExactSum) return kb;
+    sum += grow;
+    --left;
+  }
+  return p.nkb;
 }
 
 // -------------------------------------------------------------- converter
@@ -374,11 +492,13 @@ __device__ __forceinline__ uint32_t pair_i8(uint32_t a, uint32_t b, uint32_t j) 
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// Byte address of tile (slot, plane, K-tile kt, ib) in the ring.
-template <int FMT>
+// Byte address of the first tile of (slot, plane, K-tile kt, ib) in the ring: a
+// K-tile is a K-block's tiles, [kSplit][plane], so that the two planes of a
+// stage lie side by side (one copy brings both).
+template <int FMT, int SHAPE>
 __device__ __forceinline__ uint8_t* ring_tile(const Params& p, int slot, int plane, int kt, int ib) {
-  return p.ring + ((((static_cast<int64_t>(slot) * 2 + plane) * p.nkt + kt) * p.nib + ib)
-                   << FmtT<FMT>::kTileShift);
+  return p.ring + ((static_cast<int64_t>(slot) * p.nkt + kt) * p.nib + ib) * FmtT<FMT, SHAPE>::kKbBytes +
+         plane * FmtT<FMT, SHAPE>::kTile;
 }
 
 // Power-of-two scale exponent e for an input whose largest component is
@@ -395,47 +515,126 @@ __device__ __forceinline__ int scale_exp(unsigned bits) {
 }
 __device__ __forceinline__ float exp2i(int e) { return __int_as_float((127 + e) << 23); }
 
-// A unit: 64 inputs (half block hb) x kUnitT samples (unit ku along K) of
-// channel c, units numbered channel-major with K fastest; it fills 8-sample
-// chunks cbase .. cbase + kUnitT/8 - 1 of the tiles of K-block kb.
+// A converter unit: 64 inputs (half block hb) x one K-block (k of its
+// segment) of segment number G.  Units are numbered segment by
+// segment, half block by half block, K fastest; every segment has seg_units
+// numbers, of which those past the channel's last K-block stand for nothing.
 struct Unit {
-  int c, slot, hb, ku, kb, cbase;
+  long long u;      // global number
+  int sb;           // subarray
+  int G, c, seg;    // segment number in the subarray; channel, segment of it
+  int slot;         // G % ring_slots
+  unsigned gen;     // G / ring_slots
+  int w, hb, k;     // unit in the segment
 };
 
-__device__ __forceinline__ Unit unit_of(const Params& p, long long u) {
-  Unit x;
-  x.c = static_cast<int>(u / p.units_per_chan);
-  const int w = static_cast<int>(u % p.units_per_chan);
-  x.slot = x.c % p.ring_slots;
-  const int nku = p.nkb * (kBK / kUnitT);
-  x.hb = w / nku;
-  x.ku = w % nku;
-  x.kb = x.ku * kUnitT / kBK;
-  x.cbase = (x.ku * kUnitT % kBK) / 8;
-  return x;
+// Converter warps take their units in runs of kUnitRun consecutive units
+// (always of one segment, whose unit count is even): one slot claim and one
+// publish (fence + release of the whole count) per run instead of per unit.
+// Warp gw of nw takes runs gw, gw + nw, gw + 2 nw, ... of the global unit
+// list.
+constexpr int kUnitRun = 2;
+
+// Unit u by division (a warp's first one, and the first in another subarray).
+template <bool MULTI>
+__device__ __forceinline__ void unit_locate(const Batch& bt, Unit& x) {
+  x.sb = advance_sub<MULTI>(bt.unit_base, bt.nsub, x.u, x.sb);
+  const Params& p = bt.sub[x.sb];
+  const long long v = x.u - bt.unit_base[x.sb];
+  x.G = static_cast<int>(v / p.seg_units);
+  x.w = static_cast<int>(v - static_cast<long long>(x.G) * p.seg_units);
+  x.gen = static_cast<unsigned>(x.G / p.ring_slots);
+  x.slot = x.G - static_cast<int>(x.gen) * p.ring_slots;
 }
 
-// Before a warp first writes channel c into its slot: the slot's previous
-// channel (c - ring_slots) must have been read by all of its blocks.
-__device__ __forceinline__ bool claim_slot_warp(const Params& p, int c, int lane,
+// Next number of the warp; false at the end of the list.  The precomputed
+// steps replace four divisions per unit: together with their dependent chains
+// they were about a quarter of a converter warp's time per unit.
+template <bool MULTI>
+__device__ __forceinline__ bool unit_step(const Batch& bt, Unit& x, long long nw, long long total) {
+  if ((x.u & (kUnitRun - 1)) != kUnitRun - 1) {
+    ++x.u;
+    ++x.w;
+    return true;
+  }
+  x.u += 1 + (nw - 1) * kUnitRun;
+  if (x.u >= total) return false;
+  if (MULTI && x.u >= bt.unit_base[x.sb + 1]) {
+    unit_locate<MULTI>(bt, x);
+    return true;
+  }
+  const Params& p = bt.sub[x.sb];
+  x.w += p.step_rem - (kUnitRun - 1);
+  const int carry = x.w >= p.seg_units ? 1 : 0;
+  x.w -= carry ? p.seg_units : 0;
+  x.G += p.step_seg + carry;
+  x.gen += static_cast<unsigned>(p.step_gen);
+  x.slot += p.step_slot + carry;
+  if (x.slot >= p.ring_slots) {
+    x.slot -= p.ring_slots;
+    ++x.gen;
+  }
+  return true;
+}
+
+// Channel, segment, half block and K-block of a number; false if it stands for
+// nothing.
+__device__ __forceinline__ bool unit_decode(const Params& p, Unit& x) {
+  const bool last = x.G >= p.last_base;
+  const int wv = last ? p.wave_full : fast_div(x.G, p.wave_segs, p.mag_wsegs);
+  const int r = x.G - wv * p.wave_segs, width = last ? p.wave_last : p.wave;
+  x.seg = fast_div(r, width, last ? p.mag_last : p.mag_wave);
+  x.c = wv * p.wave + r - x.seg * width;
+  x.hb = fast_div(x.w, p.seg_kb, p.mag_kb);
+  x.k = x.w - x.hb * p.seg_kb;
+  return x.seg * p.seg_kb + x.k < p.nkb;
+}
+
+template <bool MULTI>
+__device__ __forceinline__ bool unit_first(const Batch& bt, Unit& x, long long gw, long long nw,
+                                           long long total) {
+  x.u = gw * kUnitRun;
+  x.sb = 0;
+  if (x.u >= total) return false;
+  unit_locate<MULTI>(bt, x);
+  while (!unit_decode(bt.sub[x.sb], x))
+    if (!unit_step<MULTI>(bt, x, nw, total)) return false;
+  return true;
+}
+template <bool MULTI>
+__device__ __forceinline__ bool unit_next(const Batch& bt, Unit& x, long long nw, long long total) {
+  do {
+    if (!unit_step<MULTI>(bt, x, nw, total)) return false;
+  } while (!unit_decode(bt.sub[x.sb], x));
+  return true;
+}
+
+// What unit x adds to its segment's ready counter: one, and for the last
+// K-block of a half block in a short segment also its missing units, so that
+// every segment counts seg_units.
+__device__ __forceinline__ unsigned unit_weight(const Params& p, const Unit& x) {
+  return x.seg * p.seg_kb + x.k == p.nkb - 1 ? static_cast<unsigned>(p.seg_kb - x.k) : 1u;
+}
+
+// Before a warp first writes segment G into its slot: the slot's previous
+// segment (G - ring_slots) must have been read by all of its channel's items.
+__device__ __forceinline__ bool claim_slot_warp(const Params& p, const Unit& x, int lane,
                                                 volatile int* abort_flag) {
-  const unsigned gen = static_cast<unsigned>(c / p.ring_slots);
   bool ok = true;
-  if (gen > 0 && lane == 0)
-    ok = wait_counter(p.done + (c % p.ring_slots), gen * static_cast<unsigned>(p.ipc), p, abort_flag);
-  // No proxy fence here: every bulk read of the slot's previous channel has
-  // completed (its data sat in shared memory before the MMA thread released
+  if (x.gen > 0 && lane == 0)
+    ok = wait_counter(p.done + x.slot, x.gen * static_cast<unsigned>(p.ipc), p, abort_flag);
+  // No proxy fence here: every bulk read of the slot's previous segment has
+  // completed (its data sat in shared memory before the producer released
   // done[slot]), so the generic writes that follow cannot reach it.
   return __all_sync(0xffffffffu, ok);
 }
 
-// Would a claim of channel c's slot have to wait for the slot's previous
-// channel?  (Checked before a warp waits while it holds an unpublished unit.)
-__device__ __forceinline__ bool slot_busy(const Params& p, int c, int lane) {
-  const unsigned gen = static_cast<unsigned>(c / p.ring_slots);
+// Would a claim of segment G's slot have to wait for the slot's previous
+// segment?  (Checked before a warp waits while it holds an unpublished unit.)
+__device__ __forceinline__ bool slot_busy(const Params& p, const Unit& x, int lane) {
   bool busy = false;
-  if (gen > 0 && lane == 0)
-    busy = ld_acquire(p.done + (c % p.ring_slots)) < gen * static_cast<unsigned>(p.ipc);
+  if (x.gen > 0 && lane == 0)
+    busy = ld_acquire(p.done + x.slot) < x.gen * static_cast<unsigned>(p.ipc);
   return __any_sync(0xffffffffu, busy);
 }
 
@@ -449,16 +648,6 @@ __device__ __forceinline__ void publish_unit(const Params& p, int slot, int lane
   fence_proxy_async_global();
   __syncwarp();
   if (lane == 0) red_release_add(p.ready + slot, n);
-}
-
-// Converter warps take their units in runs of kUnitRun consecutive units
-// (the same channel except at channel ends): one slot claim and one publish
-// (fence + release of the whole count) per run instead of per unit.  Warp gw
-// of nw takes runs gw, gw + nw, gw + 2 nw, ... of the global unit list.
-constexpr int kUnitRun = 2;
-__device__ __forceinline__ long long first_unit(long long gw) { return gw * kUnitRun; }
-__device__ __forceinline__ long long next_unit(long long u, long long nw) {
-  return (u % kUnitRun != kUnitRun - 1) ? u + 1 : u + 1 + (nw - 1) * kUnitRun;
 }
 
 // Complex sample (re, im) of input a at sample t, channel c, as fp32.
@@ -499,23 +688,24 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
 // input's power-of-two scale (float input) and writes 16-byte chunks: per
 // (input, plane) two fp16 chunks (8 samples each; HI/LO: two more into the
 // L tile) or one e4m3 chunk (16 samples).
-template <int DT, int FMT, bool MULTI>
+template <int DT, int FMT, bool MULTI, int SHAPE>
 __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int* abort_flag) {
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
-  const long long stride = static_cast<long long>(gridDim.x) * conv_warps<FMT, DT>();
-  int sb = 0, claimed = -1, claimed_sb = -1;
-  for (long long u = static_cast<long long>(blockIdx.x) * conv_warps<FMT, DT>() + cw; u < total; u += stride) {
-    sb = advance_sub<MULTI>(bt.unit_base, bt.nsub, u, sb);
-    const Params& p = bt.sub[sb];
-    const Unit x = unit_of(p, u - bt.unit_base[sb]);
-    if (x.c != claimed || sb != claimed_sb) {
-      if (!claim_slot_warp(p, x.c, lane, abort_flag)) return;
-      claimed = x.c;
-      claimed_sb = sb;
+  const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, DT>();
+  int claimed = -1, claimed_sb = -1;
+  Unit x;
+  bool more = unit_first<MULTI>(bt, x, static_cast<long long>(blockIdx.x) * conv_warps<FMT, DT>() + cw, nw, total);
+  for (; more; more = unit_next<MULTI>(bt, x, nw, total)) {
+    const Params& p = bt.sub[x.sb];
+    if (x.G != claimed || x.sb != claimed_sb) {
+      if (!claim_slot_warp(p, x, lane, abort_flag)) return;
+      claimed = x.G;
+      claimed_sb = x.sb;
     }
     const int ib = x.hb >> 1;
-    uint8_t* tre = ring_tile<FMT>(p, x.slot, 0, x.kb, ib);
-    uint8_t* tim = ring_tile<FMT>(p, x.slot, 1, x.kb, ib);
+    const int t0 = (x.seg * p.seg_kb + x.k) * kBK;  // first sample
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
     const int a0 = x.hb * 64 + lane, a1 = a0 + 32;
     const int row0 = (x.hb & 1) * 64 + lane;
     // y = g x 2^-e (float input; gains are not defined for 8-bit input).
@@ -540,7 +730,7 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
       float2 v0[16], v1[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        const int t = x.ku * kUnitT + g * 16 + i;
+        const int t = t0 + g * 16 + i;
         v0[i] = (a0 < p.n && t < p.g.T) ? load_cx<DT>(p, x.c, a0, t) : make_float2(0.f, 0.f);
         v1[i] = (a1 < p.n && t < p.g.T) ? load_cx<DT>(p, x.c, a1, t) : make_float2(0.f, 0.f);
       }
@@ -558,8 +748,8 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
         }
       }
       if constexpr (FMT == kFmtF8) {
-        const uint32_t off = tile_off<FMT>(row0, x.cbase / 2 + g);
-        const uint32_t off1 = tile_off<FMT>(row0 + 32, x.cbase / 2 + g);
+        const uint32_t off = tile_off<FMT, SHAPE>(row0, g);
+        const uint32_t off1 = tile_off<FMT, SHAPE>(row0 + 32, g);
         uint32_t r0[4], i0[4], r1[4], i1[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -577,8 +767,8 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
       } else {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const uint32_t off = tile_off<FMT>(row0, x.cbase + 2 * g + h);
-          const uint32_t off1 = tile_off<FMT>(row0 + 32, x.cbase + 2 * g + h);
+          const uint32_t off = tile_off<FMT, SHAPE>(row0, 2 * g + h);
+          const uint32_t off1 = tile_off<FMT, SHAPE>(row0 + 32, 2 * g + h);
           uint32_t r0[4], i0[4], r1[4], i1[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -594,8 +784,8 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
           *reinterpret_cast<uint4*>(tre + off1) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
           *reinterpret_cast<uint4*>(tim + off1) = make_uint4(i1[0], i1[1], i1[2], i1[3]);
           if constexpr (FMT == kFmtHiLo) {
-            // Residual tile of the same K-block: K-tile nkb + kb.
-            const int64_t lo_off = static_cast<int64_t>(p.nkb) * p.nib << FmtT<FMT>::kTileShift;
+            // Residual tile of the same K-block: K-tile seg_kb + k.
+            const int64_t lo_off = static_cast<int64_t>(p.seg_kb) * p.nib * FmtT<FMT, SHAPE>::kKbBytes;
             uint32_t l0[4], m0[4], l1[4], m1[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -614,10 +804,10 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
         }
       }
     }
-    if (DT == 0 && lane == 0) atomicMax(p.amax + x.c, 128u);  // no scan: worst case
+    if (DT == 0 && lane == 0) atomicMax(p.amax + x.G, 128u);  // no scan: worst case
     if (DT == 0 && FMT == kFmtF8 && __any_sync(0xffffffffu, unit_over_16) && lane == 0)
       atomicOr(p.status, kStatusRange);  // e4m3 is exact only for |x| <= 16
-    publish_unit(p, x.slot, lane);
+    publish_unit(p, x.slot, lane, unit_weight(p, x));
     if (*abort_flag) return;
   }
 }
@@ -645,25 +835,22 @@ __device__ __forceinline__ void drain_tma(uint32_t bar, uint32_t phase, bool pen
 // stores have drained by the time the proxy fence waits for them; a warp
 // that would have to wait for a slot publishes first (a consumer of the
 // slot's previous channel may need that unit).
-template <int FMT, bool MULTI>
+template <int FMT, bool MULTI, int SHAPE>
 __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int cw, int lane,
                               volatile int* abort_flag) {
   static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
-  int sb_issue = 0;
   bool tma_pending = false;  // a box issued and not yet waited for
-  auto issue = [&](long long u) {
+  auto issue = [&](const Unit& x) {
     tma_pending = true;
-    sb_issue = advance_sub<MULTI>(bt.unit_base, bt.nsub, u, sb_issue);
-    const Unit x = unit_of(bt.sub[sb_issue], u - bt.unit_base[sb_issue]);
     if (lane == 0) {
       ptx::mbar_arrive_expect_tx(bar, kConvBufBytes);
       // The input streams through once: first in line for L2 replacement, so
       // the operand ring it is converted into stays resident.
-      ptx::tma_load_3d_hint(buf, &bt.maps[sb_issue], bar, x.hb * kUnitRows, x.c, x.ku * kUnitT,
-                            ptx::l2_policy_evict_first());
+      ptx::tma_load_3d_hint(buf, &bt.maps[x.sb], bar, x.hb * kUnitRows, x.c,
+                            (x.seg * bt.sub[x.sb].seg_kb + x.k) * kUnitT, ptx::l2_policy_evict_first());
     }
   };
   const uint32_t* src = reinterpret_cast<const uint32_t*>(__cvta_shared_to_generic(static_cast<size_t>(buf)));
@@ -672,28 +859,28 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
   // the lane writes tile rows 2l and 2l + 1 (32 contiguous bytes), so a warp
   // store covers 1 KiB.
   uint32_t phase = 0;
-  int sb = 0, claimed = -1, claimed_sb = -1;
-  // Converted units not yet published: their subarray, slot, channel, count.
+  int claimed = -1, claimed_sb = -1;
+  // Converted units of a run not yet published: their subarray, slot, run, count.
   const Params* pend = nullptr;
-  int pend_slot = 0, pend_c = -1, pend_sb = -1;
+  int pend_slot = 0;
+  long long pend_run = -1;
   unsigned pend_n = 0;
-  long long u = first_unit(static_cast<long long>(blockIdx.x) * conv_warps<FMT, 0>() + cw);
-  if (u < total) issue(u);
-  for (; u < total; u = next_unit(u, nw)) {
-    sb = advance_sub<MULTI>(bt.unit_base, bt.nsub, u, sb);
-    const Params& p = bt.sub[sb];
-    const Unit x = unit_of(p, u - bt.unit_base[sb]);
-    if (x.c != claimed || sb != claimed_sb) {
-      if (pend && slot_busy(p, x.c, lane)) {
+  Unit x;
+  bool more = unit_first<MULTI>(bt, x, static_cast<long long>(blockIdx.x) * conv_warps<FMT, 0>() + cw, nw, total);
+  if (more) issue(x);
+  while (more) {
+    const Params& p = bt.sub[x.sb];
+    if (x.G != claimed || x.sb != claimed_sb) {
+      if (pend && slot_busy(p, x, lane)) {
         publish_unit(*pend, pend_slot, lane, pend_n);
         pend = nullptr;
       }
-      if (!claim_slot_warp(p, x.c, lane, abort_flag)) {
+      if (!claim_slot_warp(p, x, lane, abort_flag)) {
         drain_tma(bar, phase, tma_pending, wc.timeout_ns);
         return;
       }
-      claimed = x.c;
-      claimed_sb = sb;
+      claimed = x.G;
+      claimed_sb = x.sb;
     }
     const bool got = ptx::wait_bounded(bar, phase, wc);
     if (!__all_sync(0xffffffffu, got)) {
@@ -708,17 +895,18 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
     for (int t = 0; t < kUnitT; ++t) w[t] = src[t * (kUnitRows / 4) + lane];
     __syncwarp();
     ptx::fence_proxy_async_smem();
-    const long long un = next_unit(u, nw);
-    if (un < total) issue(un);
-    // A finished run (or the units of another channel) is published now: its
-    // stores have drained during this unit's shared-memory reads.
-    if (pend && (pend_n == kUnitRun || pend_c != x.c || pend_sb != sb)) {
+    Unit nx = x;
+    more = unit_next<MULTI>(bt, nx, nw, total);
+    if (more) issue(nx);
+    // A finished run is published now: its stores have drained during this
+    // unit's shared-memory reads.
+    if (pend && pend_run != x.u / kUnitRun) {
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
     const int ib = x.hb >> 1;
-    uint8_t* tre = ring_tile<FMT>(p, x.slot, 0, x.kb, ib);
-    uint8_t* tim = ring_tile<FMT>(p, x.slot, 1, x.kb, ib);
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
     const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
     // Ring tiles are read back by every block of the channel: keep them in L2.
     const uint64_t pol_last = ptx::l2_policy_evict_last();
@@ -744,7 +932,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       };
 #pragma unroll
       for (int cc = 0; cc < kUnitT / 8; ++cc) {
-        const uint32_t off = tile_off<FMT>(row, x.cbase + cc);
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
         store8(tre + off, w + 8 * cc, 0u, mx[0]);
         store8(tim + off, w + 8 * cc, 1u, mx[1]);
       }
@@ -773,7 +961,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       };
 #pragma unroll
       for (int cc = 0; cc < kUnitT / 16; ++cc) {
-        const uint32_t off = tile_off<FMT>(row, x.cbase / 2 + cc);
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
         const uint32_t* W = w + 16 * cc;
         uint32_t vr[8], vi[8];
 #pragma unroll
@@ -790,18 +978,17 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) {
-      atomicMax(p.amax + x.c, m);
+      atomicMax(p.amax + x.G, m);
       if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
     }
-    if (pend) {
-      ++pend_n;
-    } else {
+    if (!pend) {
       pend = &p;
       pend_slot = x.slot;
-      pend_c = x.c;
-      pend_sb = sb;
-      pend_n = 1;
+      pend_run = x.u / kUnitRun;
+      pend_n = 0;
     }
+    pend_n += unit_weight(p, x);
+    x = nx;
     if (*abort_flag) {
       drain_tma(bar, phase, tma_pending, wc.timeout_ns);
       return;
@@ -814,7 +1001,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
 // gains and scale already applied) into the tiles of one K-block: fp16 (two
 // 8-sample chunks from chunk8), hi/lo (the same in the H tiles plus the
 // residuals in the L tiles) or e4m3 (one 16-sample chunk).
-template <int FMT>
+template <int FMT, int SHAPE>
 __device__ __forceinline__ void store_group16(const Params& p, uint8_t* tre, uint8_t* tim, int row0,
                                               int chunk8, const float2 (&v0)[16],
                                               const float2 (&v1)[16], uint64_t pol) {
@@ -822,8 +1009,8 @@ __device__ __forceinline__ void store_group16(const Params& p, uint8_t* tre, uin
     ptx::st_global_v4_hint(dst, a, b, c, d, pol);
   };
   if constexpr (FMT == kFmtF8) {
-    const uint32_t off = tile_off<FMT>(row0, chunk8 / 2);
-    const uint32_t off1 = tile_off<FMT>(row0 + 32, chunk8 / 2);
+    const uint32_t off = tile_off<FMT, SHAPE>(row0, chunk8 / 2);
+    const uint32_t off1 = tile_off<FMT, SHAPE>(row0 + 32, chunk8 / 2);
     uint32_t r0[4], i0[4], r1[4], i1[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -841,8 +1028,8 @@ __device__ __forceinline__ void store_group16(const Params& p, uint8_t* tre, uin
   } else {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const uint32_t off = tile_off<FMT>(row0, chunk8 + h);
-      const uint32_t off1 = tile_off<FMT>(row0 + 32, chunk8 + h);
+      const uint32_t off = tile_off<FMT, SHAPE>(row0, chunk8 + h);
+      const uint32_t off1 = tile_off<FMT, SHAPE>(row0 + 32, chunk8 + h);
       uint32_t r0[4], i0[4], r1[4], i1[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -858,8 +1045,8 @@ __device__ __forceinline__ void store_group16(const Params& p, uint8_t* tre, uin
       st(tre + off1, r1[0], r1[1], r1[2], r1[3]);
       st(tim + off1, i1[0], i1[1], i1[2], i1[3]);
       if constexpr (FMT == kFmtHiLo) {
-        // Residual tile of the same K-block: K-tile nkb + kb.
-        const int64_t lo_off = static_cast<int64_t>(p.nkb) * p.nib << FmtT<FMT>::kTileShift;
+        // Residual tile of the same K-block: K-tile seg_kb + k.
+        const int64_t lo_off = static_cast<int64_t>(p.seg_kb) * p.nib * FmtT<FMT, SHAPE>::kKbBytes;
         uint32_t l0[4], m0[4], l1[4], m1[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -884,7 +1071,7 @@ __device__ __forceinline__ void store_group16(const Params& p, uint8_t* tre, uin
 // through the warp's one staging buffer, kUnitT / kFBox boxes per unit;
 // while one box is converted the next (of this unit or of the next) is in
 // flight.  Units are taken in runs and published as in converter_tma.
-template <int DT, int FMT, bool MULTI>
+template <int DT, int FMT, bool MULTI, int SHAPE>
 __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar, int cw, int lane,
                                     volatile int* abort_flag) {
   constexpr int kCx = DT == 1 ? 4 : 8;  // bytes per complex sample
@@ -894,50 +1081,51 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, DT>();
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
-  int sb_issue = 0;
   bool tma_pending = false;  // a box issued and not yet waited for
-  auto issue = [&](long long u, int j) {
+  auto issue = [&](const Unit& x, int j) {
     tma_pending = true;
-    sb_issue = advance_sub<MULTI>(bt.unit_base, bt.nsub, u, sb_issue);
-    const Unit x = unit_of(bt.sub[sb_issue], u - bt.unit_base[sb_issue]);
     if (lane == 0) {
       ptx::mbar_arrive_expect_tx(bar, kConvBufBytes);
       // Map elements: one complex fp16 (32-bit) or one fp32 component.
       const int ex = DT == 1 ? x.hb * 64 : x.hb * 128;
-      ptx::tma_load_3d_hint(buf, &bt.maps[sb_issue], bar, ex, x.c, x.ku * kUnitT + j * kFBox,
+      ptx::tma_load_3d_hint(buf, &bt.maps[x.sb], bar, ex, x.c,
+                            (x.seg * bt.sub[x.sb].seg_kb + x.k) * kUnitT + j * kFBox,
                             ptx::l2_policy_evict_first());
     }
   };
   const uint8_t* src = reinterpret_cast<const uint8_t*>(__cvta_shared_to_generic(static_cast<size_t>(buf)));
   const uint64_t pol_last = ptx::l2_policy_evict_last();
   uint32_t phase = 0;
-  int sb = 0, claimed = -1, claimed_sb = -1;
+  int claimed = -1, claimed_sb = -1;
+  // Converted units of a run not yet published: their subarray, slot, run, count.
   const Params* pend = nullptr;
-  int pend_slot = 0, pend_c = -1, pend_sb = -1;
+  int pend_slot = 0;
+  long long pend_run = -1;
   unsigned pend_n = 0;
-  long long u = first_unit(static_cast<long long>(blockIdx.x) * conv_warps<FMT, DT>() + cw);
-  if (u < total) issue(u, 0);
-  for (; u < total; u = next_unit(u, nw)) {
-    sb = advance_sub<MULTI>(bt.unit_base, bt.nsub, u, sb);
-    const Params& p = bt.sub[sb];
-    const Unit x = unit_of(p, u - bt.unit_base[sb]);
-    if (x.c != claimed || sb != claimed_sb) {
-      if (pend && slot_busy(p, x.c, lane)) {
+  Unit x;
+  bool more = unit_first<MULTI>(bt, x, static_cast<long long>(blockIdx.x) * conv_warps<FMT, DT>() + cw, nw, total);
+  if (more) issue(x, 0);
+  while (more) {
+    const Params& p = bt.sub[x.sb];
+    if (x.G != claimed || x.sb != claimed_sb) {
+      if (pend && slot_busy(p, x, lane)) {
         publish_unit(*pend, pend_slot, lane, pend_n);
         pend = nullptr;
       }
-      if (!claim_slot_warp(p, x.c, lane, abort_flag)) {
+      if (!claim_slot_warp(p, x, lane, abort_flag)) {
         drain_tma(bar, phase, tma_pending, wc.timeout_ns);
         return;
       }
-      claimed = x.c;
-      claimed_sb = sb;
+      claimed = x.G;
+      claimed_sb = x.sb;
     }
     const int ib = x.hb >> 1;
-    uint8_t* tre = ring_tile<FMT>(p, x.slot, 0, x.kb, ib);
-    uint8_t* tim = ring_tile<FMT>(p, x.slot, 1, x.kb, ib);
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
     const int a0 = x.hb * 64 + lane, a1 = a0 + 32;
     const int row0 = (x.hb & 1) * 64 + lane;
+    Unit nx = x;
+    more = unit_next<MULTI>(bt, nx, nw, total);
     // y = g x 2^-e.
     float2 g0 = make_float2(1.f, 0.f), g1 = make_float2(1.f, 0.f);
     if (p.gains) {
@@ -972,12 +1160,11 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
       __syncwarp();
       ptx::fence_proxy_async_smem();
       if (j + 1 < kBoxes) {
-        issue(u, j + 1);
-      } else {
-        const long long un = next_unit(u, nw);
-        if (un < total) issue(un, 0);
+        issue(x, j + 1);
+      } else if (more) {
+        issue(nx, 0);
       }
-      if (j == 0 && pend && (pend_n == kUnitRun || pend_c != x.c || pend_sb != sb)) {
+      if (j == 0 && pend && pend_run != x.u / kUnitRun) {
         publish_unit(*pend, pend_slot, lane, pend_n);
         pend = nullptr;
       }
@@ -997,18 +1184,17 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
           v0[i] = make_float2(g0.x * c0.x - g0.y * c0.y, g0.x * c0.y + g0.y * c0.x);
           v1[i] = make_float2(g1.x * c1.x - g1.y * c1.y, g1.x * c1.y + g1.y * c1.x);
         }
-        store_group16<FMT>(p, tre, tim, row0, x.cbase + (j * kFBox + 16 * g16) / 8, v0, v1, pol_last);
+        store_group16<FMT, SHAPE>(p, tre, tim, row0, (j * kFBox + 16 * g16) / 8, v0, v1, pol_last);
       }
     }
-    if (pend) {
-      ++pend_n;
-    } else {
+    if (!pend) {
       pend = &p;
       pend_slot = x.slot;
-      pend_c = x.c;
-      pend_sb = sb;
-      pend_n = 1;
+      pend_run = x.u / kUnitRun;
+      pend_n = 0;
     }
+    pend_n += unit_weight(p, x);
+    x = nx;
     if (*abort_flag) {
       drain_tma(bar, phase, tma_pending, wc.timeout_ns);
       return;
@@ -1019,16 +1205,26 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
 
 // --------------------------------------------------------------- epilogue
 
+// How a piece's fp32 sums become the stored words: as they are (float input)
+// or int32 (8-bit input).
+enum : int { kWordFloat = 0, kWordInt = 1 };
+template <int WORD>
+__device__ __forceinline__ uint32_t out_word(uint32_t u) {
+  if constexpr (WORD == kWordFloat) return u;
+  return static_cast<uint32_t>(__float2int_rn(__uint_as_float(u)));
+}
+
 // Store one 32-column piece: values v_re[j], v_im[j] of V(a, b0 + j).
-template <bool IS_INT>
+template <int WORD>
 __device__ __forceinline__ void store_piece(const uint32_t (&re)[32], const uint32_t (&im)[32],
-                                            const Params& p, int f, int a, int b0, bool add) {
+                                            const Params& p, int f, int a, int b0, bool add, uint64_t pol) {
+  constexpr bool IS_INT = WORD != kWordFloat;
   using T = typename std::conditional<IS_INT, int, float>::type;
   const Geometry& g = p.g;
   T* out = static_cast<T*>(p.out);
   auto val = [&](uint32_t u) -> T {
     if constexpr (IS_INT) {
-      return __float2int_rn(__uint_as_float(u));
+      return static_cast<int>(out_word<WORD>(u));
     } else {
       return __uint_as_float(u);
     }
@@ -1041,7 +1237,7 @@ __device__ __forceinline__ void store_piece(const uint32_t (&re)[32], const uint
   if (!valid && !pairs) return;
   // Real channel, row station and first column station (packed channels:
   // columns of another channel of the pack fall outside 0 <= s2 <= s1).
-  int fr = f, s1 = a / g.P, s2_0 = b0 / g.P;
+  int fr = f, s1 = a >> (g.P - 1), s2_0 = b0 >> (g.P - 1);  // P is 1 or 2
   if (p.pack > 1) {
     const int j = s1 / p.Nr;
     s1 -= j * p.Nr;
@@ -1056,19 +1252,12 @@ __device__ __forceinline__ void store_piece(const uint32_t (&re)[32], const uint
     for (int m = 0; m < 8; ++m) {
       // This lane's products for column stations 2m (A) and 2m + 1 (B) of the piece.
       uint32_t A[4], B[4], rec[8];
-      auto bits = [&](uint32_t u) -> uint32_t {  // the stored word: int32 value or fp32 bits
-        if constexpr (IS_INT) {
-          return static_cast<uint32_t>(val(u));
-        } else {
-          return u;
-        }
-      };
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        A[2 * q] = bits(re[4 * m + q]);
-        A[2 * q + 1] = bits(im[4 * m + q]);
-        B[2 * q] = bits(re[4 * m + 2 + q]);
-        B[2 * q + 1] = bits(im[4 * m + 2 + q]);
+        A[2 * q] = out_word<WORD>(re[4 * m + q]);
+        A[2 * q + 1] = out_word<WORD>(im[4 * m + q]);
+        B[2 * q] = out_word<WORD>(re[4 * m + 2 + q]);
+        B[2 * q + 1] = out_word<WORD>(im[4 * m + 2 + q]);
       }
       // Row p1 = 0 writes baseline 2m, row p1 = 1 baseline 2m + 1; each sends
       // the partner the half it needs.
@@ -1080,7 +1269,7 @@ __device__ __forceinline__ void store_piece(const uint32_t (&re)[32], const uint
       }
       const int s2 = s2_0 + 2 * m + p1;
       if (valid && s2 >= 0 && s2 <= s1)
-        ptx::st_global_v8_hint(o8 + 8 * static_cast<int64_t>(s2), rec, ptx::l2_policy_evict_first());
+        ptx::st_global_v8_hint(o8 + 8 * static_cast<int64_t>(s2), rec, pol);
     }
   } else if (g.P == 2) {
     const int p1 = a & 1;
@@ -1168,13 +1357,13 @@ __device__ __forceinline__ void scale_piece(uint32_t (&re)[32], uint32_t (&im)[3
 // piece; the last chunk of the integration also stores its fp32 rounding.
 __device__ __forceinline__ void store_piece_f64(const uint32_t (&re)[32], const uint32_t (&im)[32],
                                                 const Params& p, int f, int a, int b0, bool first,
-                                                bool last) {
+                                                bool last, uint64_t pol) {
   const int P = p.g.P;
   // Every lane of the warp joins the pairs path's exchanges; rows past n
   // (the ragged last block) only skip their memory accesses.
   const bool valid = a < p.n;
   if (!valid && !(P == 2 && p.pack == 1)) return;
-  int s1 = a / P, joff = 0, fr = f;
+  int s1 = a >> (P - 1), joff = 0, fr = f;
   const int p1 = a - s1 * P;
   if (p.pack > 1) {  // packed channels: real channel and stations
     const int j = s1 / p.Nr;
@@ -1257,7 +1446,7 @@ __device__ __forceinline__ void store_piece_f64(const uint32_t (&re)[32], const 
             rec[2 * k] = __float_as_uint(static_cast<float>(v[k].x));
             rec[2 * k + 1] = __float_as_uint(static_cast<float>(v[k].y));
           }
-          ptx::st_global_v8_hint(out + (krow + s2) * 4, rec, ptx::l2_policy_evict_first());
+          ptx::st_global_v8_hint(out + (krow + s2) * 4, rec, pol);
         }
       }
     }
@@ -1266,7 +1455,7 @@ __device__ __forceinline__ void store_piece_f64(const uint32_t (&re)[32], const 
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     const int b = b0 + j;
-    const int s2v = b / P, p2 = b - s2v * P, s2 = s2v - joff;
+    const int s2v = b >> (P - 1), p2 = b - s2v * P, s2 = s2v - joff;
     if (s2 < 0 || s2 > s1) continue;
     const int64_t idx = (krow + s2) * P * P + p1 * P + p2;
     double2 v = make_double2(static_cast<double>(__uint_as_float(re[j])),
@@ -1286,25 +1475,21 @@ __device__ __forceinline__ void store_piece_f64(const uint32_t (&re)[32], const 
 // entries are the mirror ones, V[b][a] = conj(V[a][b]): baseline
 // (s1, s2) = (s_b, s_a), polarisation product p_b * P + p_a.  Packed
 // channels never occur here (they have one block row).
-template <bool IS_INT>
+template <int WORD>
 __device__ __forceinline__ void store_piece_tr(const uint32_t (&re)[32], const uint32_t (&im)[32],
-                                               const Params& p, int f, int a, int b0, bool add) {
+                                               const Params& p, int f, int a, int b0, bool add,
+                                               uint64_t pol) {
+  constexpr bool IS_INT = WORD != kWordFloat;
   using T = typename std::conditional<IS_INT, int, float>::type;
   const Geometry& g = p.g;
   T* out = static_cast<T*>(p.out);
   const int P = g.P;
-  const int sa = a / P, pa = a - sa * P;
+  const int sa = a >> (P - 1), pa = a - sa * P;
   // The stored word of the conjugate: int32 value or fp32 bits.
-  auto re_bits = [](uint32_t u) -> uint32_t {
-    if constexpr (IS_INT) {
-      return static_cast<uint32_t>(__float2int_rn(__uint_as_float(u)));
-    } else {
-      return u;
-    }
-  };
+  auto re_bits = [](uint32_t u) -> uint32_t { return out_word<WORD>(u); };
   auto im_bits = [](uint32_t u) -> uint32_t {  // of -im
     if constexpr (IS_INT) {
-      return static_cast<uint32_t>(-__float2int_rn(__uint_as_float(u)));
+      return 0u - out_word<WORD>(u);
     } else {
       return u ^ 0x80000000u;
     }
@@ -1343,8 +1528,7 @@ __device__ __forceinline__ void store_piece_tr(const uint32_t (&re)[32], const u
       if (row_ok && sb < g.N) {
         const int64_t rec_idx =
             static_cast<int64_t>(f) * p.NBr + static_cast<int64_t>(sb) * (sb + 1) / 2 + sa;
-        ptx::st_global_v8_hint(reinterpret_cast<uint32_t*>(out) + rec_idx * 8, rec,
-                               ptx::l2_policy_evict_first());
+        ptx::st_global_v8_hint(reinterpret_cast<uint32_t*>(out) + rec_idx * 8, rec, pol);
       }
     }
     return;
@@ -1354,7 +1538,7 @@ __device__ __forceinline__ void store_piece_tr(const uint32_t (&re)[32], const u
   for (int j = 0; j < 32; ++j) {
     const int b = b0 + j;
     if (b >= p.n) continue;
-    const int sb = b / P, pb = b - sb * P;
+    const int sb = b >> (P - 1), pb = b - sb * P;
     const int64_t idx =
         ((static_cast<int64_t>(f) * p.NBr + static_cast<int64_t>(sb) * (sb + 1) / 2 + sa) * P + pb) * P + pa;
     uint32_t w[2] = {re_bits(re[j]), im_bits(im[j])};
@@ -1376,7 +1560,7 @@ __device__ __forceinline__ void store_piece_f64_tr(const uint32_t (&re)[32], con
                                                    bool last) {
   if (a >= p.n) return;
   const int P = p.g.P;
-  const int sa = a / P, pa = a - sa * P;
+  const int sa = a >> (P - 1), pa = a - sa * P;
   const bool load_old = !first || p.accumulate;
   double2* ws = reinterpret_cast<double2*>(p.acc64);
   float2* out = static_cast<float2*>(p.out);
@@ -1384,7 +1568,7 @@ __device__ __forceinline__ void store_piece_f64_tr(const uint32_t (&re)[32], con
   for (int j = 0; j < 32; ++j) {
     const int b = b0 + j;
     if (b >= p.n) continue;
-    const int sb = b / P, pb = b - sb * P;
+    const int sb = b >> (P - 1), pb = b - sb * P;
     const int64_t idx =
         ((static_cast<int64_t>(f) * p.NBr + static_cast<int64_t>(sb) * (sb + 1) / 2 + sa) * P + pb) * P + pa;
     double2 v = make_double2(static_cast<double>(__uint_as_float(re[j])),
@@ -1400,6 +1584,11 @@ __device__ __forceinline__ void store_piece_f64_tr(const uint32_t (&re)[32], con
 }
 
 // ------------------------------------------------------------------ kernel
+
+// stage_acc flags: the step opens an accumulation group (closing the one that
+// is open), or is the last step of its group.
+// A diagonal step has one operand pair (kAccSame).  The MMA's N sits above.
+enum : int { kAccStart = 1, kAccEnd = 2, kAccSame = 4, kAccNShift = 8 };
 
 // Per-launch constants of the item loop: CTA pairs walk the items by
 // cluster, single CTAs by block.
@@ -1418,6 +1607,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   constexpr bool WIDE = SHAPE == kShapeWide;
   using C = Cfg<SHAPE, FMT, DT>;
   constexpr int kStages = C::kStages;
+  constexpr int kSteps = FmtT<FMT, SHAPE>::kSteps;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -1433,13 +1623,13 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   auto conv_bar = [&](int w) { return bar0 + 8u * (kB + 5 + w); };
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + C::kBarOff + C::kNumBars * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  // K-blocks per exact accumulation chunk of the item whose first step stage s
-  // holds: the producer (which has waited for the channel) writes it before the
+  // What stage s's step does to the accumulation (kAccStart, kAccEnd): the
+  // producer (which has waited for the step's segment) writes it before the
   // stage's arrive, so the MMA thread reads it after its wait with no global
   // round trip of its own.
-  volatile int* item_chunk = reinterpret_cast<volatile int*>(tmem_holder + 2);
+  volatile int* stage_acc = reinterpret_cast<volatile int*>(tmem_holder + 2);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known uniform)
   const int lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;
   const bool leader = rank == 0;
@@ -1484,105 +1674,212 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   static_assert(!(kTmemSum && WIDE), "hi/lo operands need TMEM columns 256..511 for their sums");
   // One accumulator set in TMEM (no double buffer) for 128 x 256 items:
   // D_re in columns 0..255, D_im in 256..511.  Other shapes alternate two
-  // sets {D_re, D_im} of 128 + 128 columns.
+  // sets of 128 + 128 columns, {D_im, D_re} for 128 x 128 blocks (one N = 256
+  // MMA, Ai [Br Bi]^T, adds to both) and {D_re, D_im} for pairs.
+  constexpr uint32_t kReCol = SHAPE == kShape128 ? 128 : 0;
+  constexpr uint32_t kImCol = WIDE ? 256 : (SHAPE == kShape128 ? 0 : 128);
   constexpr bool kOneSet = kTmemSum || WIDE;
-  constexpr int TB = FmtT<FMT>::kTile;
+  constexpr int TB = FmtT<FMT, SHAPE>::kTile;
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
   const long long nitems = table_end<MULTI>(bt.item_base, bt.nsub);
   const long long it0 = item_first<SHAPE>(), istep = item_stride<SHAPE>();
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int issued_phase[kStages];
-      for (int s = 0; s < kStages; ++s) issued_phase[s] = -1;
-      bool ok = true;
-      int sb = 0, ready_chan = -1, ready_sb = -1, chan_chunk = 1;
-      const uint64_t pol_last = ptx::l2_policy_evict_last();  // tiles are shared by the channel's blocks
-      for (long long it = it0; ok && it < nitems; it += istep) {
-        sb = advance_sub<MULTI>(bt.item_base, bt.nsub, it, sb);
-        const Params& p = bt.sub[sb];
-        const Blk k = item_block<SHAPE>(p, it - bt.item_base[sb], rank);
-        const int slot = k.f % p.ring_slots;
-        if (k.f != ready_chan || sb != ready_sb) {
-          const unsigned gen = static_cast<unsigned>(k.f / p.ring_slots);
-          if (!wait_counter(p.ready + slot, (gen + 1) * static_cast<unsigned>(p.units_per_chan), p,
-                            abort_flag)) {
-            ok = false;
-            break;
-          }
-          ready_chan = k.f;
-          ready_sb = sb;
-          chan_chunk = chunk_kblocks(p, k.f);  // the channel is converted: its max |x| is final
+    // The whole warp walks the items; lane 0 waits for stages, releases
+    // segments and issues the copies, and the lanes together look at up to 32
+    // segments of a channel at a time (one round trip to L2 for all of them).
+    int stage = 0;
+    uint32_t phase = 0;
+    long long issued = 0;  // stages filled so far
+    // Parity of the phase that stage s's last fill (of any so far) runs in.
+    auto fill_phase = [&](int s) { return s < stage ? phase : phase ^ 1u; };
+    // Lane 0.  Bit s: stage s holds this item's last step of a segment, whose
+    // done counter rel[s] is released once the stage's MMAs have completed.
+    uint32_t rel_mask = 0;
+    unsigned* rel[kStages];
+    auto release = [&](int s) {
+      red_release_add(rel[s], 1u);
+      rel_mask &= ~(1u << s);
+    };
+    bool ok = true;
+    int ready_chan = -1, ready_sb = -1;
+    const uint64_t pol_last = ptx::l2_policy_evict_last();  // tiles are shared by the channel's blocks
+    for (Item x = item_start<MULTI>(bt, it0, nitems); ok && x.it < nitems;
+         item_step<MULTI>(bt, x, istep, nitems)) {
+      const Params& p = bt.sub[x.sb];
+      const Blk k = item_block<SHAPE>(p, x, rank);
+      int width;
+      const int G0 = seg_first(p, k.f, &width);
+      int slot = G0 - fast_div(G0, p.ring_slots, p.mag_slots) * p.ring_slots;
+      const bool new_chan = k.f != ready_chan || x.sb != ready_sb;
+      ready_chan = k.f;
+      ready_sb = x.sb;
+      const bool diag = SHAPE == kShape128 && k.a == k.b;
+      // MMA shape.  128 x 128: M = 128 rows, N trimmed to the block's valid
+      // columns (rounded up to 16), so ragged edge blocks skip the zero
+      // columns.  Pairs: M = 256 (both row blocks), N = 128, 64 per CTA.
+      // 128 x 256: N = 128 + the second block's valid columns (it sits right
+      // after the first in shared memory, whatever their block indices).
+      const bool two = WIDE && k.b2 >= 0;
+      const int mma_n = PAIR ? kBlk : (((two ? kBlk : 0) + min(kBlk, p.n - (two ? k.b2 : k.b) * kBlk) + 15) & ~15);
+      const int64_t kt_step = static_cast<int64_t>(p.nib) * FmtT<FMT, SHAPE>::kKbBytes;  // between K-tiles
+      const int64_t slot_step = p.nkt * kt_step;
+      const int64_t a_off = static_cast<int64_t>(k.a) * FmtT<FMT, SHAPE>::kKbBytes;
+      const int64_t b_off = static_cast<int64_t>(k.b) * FmtT<FMT, SHAPE>::kKbBytes;
+      const uint8_t* slot_base = p.ring + slot * slot_step;
+      unsigned grow = 0, sum = 0;  // 8-bit input: exact-chunk bookkeeping
+      int f_left = 0;              // float input: K-blocks left in the fp32 chunk
+      int seg = 0, kl = 0;         // segment, K-block in it
+      // The window of 32 segments that seg is in: which are known to be
+      // converted, and (lane l: the window's segment l) their growth.
+      uint32_t known = 0;
+      unsigned my_grow = 0;
+      // Segments of the window from seg on.
+      auto look = [&]() {
+        const int s = (seg & ~31) + lane;
+        bool r = s >= seg && s < p.nseg;
+        if (r && new_chan) {
+          const int G = G0 + s * width, gen = fast_div(G, p.ring_slots, p.mag_slots);
+          r = ld_acquire(p.ready + G - gen * p.ring_slots) >=
+              static_cast<unsigned>(gen + 1) * static_cast<unsigned>(p.seg_units);
         }
-        const bool diag = SHAPE == kShape128 && k.a == k.b;
-        for (int st = 0; ok && st < p.nkb * FmtT<FMT>::kSteps; ++st) {
-          // Step st: K-block kb; HI/LO steps j = 0, 1, 2 take (H, H), (L, H), (H, L).
-          const int kb = st / FmtT<FMT>::kSteps, j = st - kb * FmtT<FMT>::kSteps;
-          const int kta = kb + (j == 1 ? p.nkb : 0);
-          const int ktb = kb + (j == 2 ? p.nkb : 0);
-          if (!ptx::wait_bounded(empty_bar(stage), phase ^ 1u, wc)) {
-            ok = false;
-            break;
+        // (A converted segment's max |x| is final.)
+        if (IS_INT && r) my_grow = kblock_growth(p, G0 + s * width);
+        known |= __ballot_sync(0xffffffffu, r);
+        __syncwarp();  // what lane l acquired is ordered before lane 0's copies
+      };
+      for (int kb = 0; ok && kb < p.nkb; ++kb) {
+        if (kl == 0) {
+          // A new segment: wait until it is converted.
+          if ((seg & 31) == 0) {
+            known = 0;
+            look();
           }
+          const uint64_t t0 = (known >> (seg & 31) & 1u) ? 0 : ptx::globaltimer();
+          while (!(known >> (seg & 31) & 1u)) {
+            // Meanwhile, release what has completed.
+            if (lane == 0)
+              for (int s = 0; s < kStages; ++s)
+                if ((rel_mask >> s & 1u) && ptx::mbar_test_wait(empty_bar(s), fill_phase(s))) release(s);
+            __nanosleep(32);
+            look();
+            const bool over = !(known >> (seg & 31) & 1u) && lane == 0 && wait_given_up(p, t0, abort_flag);
+            if (__any_sync(0xffffffffu, over)) {
+              ok = false;
+              break;
+            }
+          }
+          if (!ok) break;
+          if constexpr (IS_INT) grow = __shfl_sync(0xffffffffu, my_grow, seg & 31);
+        }
+        int acc = kb == 0 ? kAccStart : 0;
+        if constexpr (IS_INT) {
+          if (kb > 0 && sum + grow > kExactSum) {
+            acc = kAccStart;
+            sum = 0;
+          }
+          sum += grow;
+        } else {
+          if (f_left == 0) {
+            acc = kAccStart;
+            f_left = p.f_chunk_kb;
+          }
+          --f_left;
+          if (kTmemSum) acc = kAccStart;
+        }
+        const bool acc_end = kb + 1 == p.nkb || (!IS_INT && (kTmemSum || f_left == 0));
+        const bool seg_end = kl + 1 == p.seg_kb || kb + 1 == p.nkb;
+        for (int st = 0; ok && st < kSteps; ++st) {
+          // HI/LO operand pairs j = 0, 1, 2 of a K-block: (H, H), (L, H), (H, L).
+          constexpr int kSpj = FmtT<FMT, SHAPE>::kSplit;
+          const int j = st / kSpj, half = st % kSpj;
+          const uint8_t* ar = slot_base + (kl + (j == 1 ? p.seg_kb : 0)) * kt_step + a_off + half * 2 * TB;
+          const uint8_t* br = slot_base + (kl + (j == 2 ? p.seg_kb : 0)) * kt_step + b_off + half * 2 * TB;
+          const bool jlast = st + 1 == kSteps;
+          const bool same = diag && (FMT != kFmtHiLo || j == 0);
+          const int word = (st == 0 ? acc : 0) | (jlast && acc_end ? kAccEnd : 0) | (same ? kAccSame : 0) |
+                           mma_n << kAccNShift;
           const uint32_t dst = sbase + stage * C::kStageBytes;
           const uint32_t fb = full_bar(stage);
-          if (st == 0) item_chunk[stage] = chan_chunk;  // published by the arrive below
-          if constexpr (PAIR) {
-            // A: this CTA's row block (not needed by an idle CTA); B: this
-            // CTA's half of the column block (always: the leader's MMA reads it).
-            constexpr int HB = TB / 2;
-            ptx::mbar_arrive_expect_tx(fb, k.idle ? 2 * HB : 2 * TB + 2 * HB);
-            if (!k.idle) {
-              ptx::bulk_load_hint(dst, ring_tile<FMT>(p, slot, 0, kta, k.a), TB, fb, pol_last);
-              ptx::bulk_load_hint(dst + TB, ring_tile<FMT>(p, slot, 1, kta, k.a), TB, fb, pol_last);
-            }
-            ptx::bulk_load_hint(dst + 2 * TB, ring_tile<FMT>(p, slot, 0, ktb, k.b) + rank * HB, HB, fb,
-                                pol_last);
-            ptx::bulk_load_hint(dst + 2 * TB + HB, ring_tile<FMT>(p, slot, 1, ktb, k.b) + rank * HB, HB,
-                                fb, pol_last);
-          } else if constexpr (WIDE) {
-            // Ar, Ai; then Br of both column blocks back to back (one 256-row
-            // operand: the second tile starts 16 groups on), and Bi likewise.
-            const bool two = k.b2 >= 0;
-            ptx::mbar_arrive_expect_tx(fb, two ? 6 * TB : 4 * TB);
-            ptx::bulk_load_hint(dst, ring_tile<FMT>(p, slot, 0, kta, k.a), TB, fb, pol_last);
-            ptx::bulk_load_hint(dst + TB, ring_tile<FMT>(p, slot, 1, kta, k.a), TB, fb, pol_last);
-            ptx::bulk_load_hint(dst + 2 * TB, ring_tile<FMT>(p, slot, 0, ktb, k.b), TB, fb, pol_last);
-            ptx::bulk_load_hint(dst + 4 * TB, ring_tile<FMT>(p, slot, 1, ktb, k.b), TB, fb, pol_last);
-            if (two) {
-              ptx::bulk_load_hint(dst + 3 * TB, ring_tile<FMT>(p, slot, 0, ktb, k.b2), TB, fb, pol_last);
-              ptx::bulk_load_hint(dst + 5 * TB, ring_tile<FMT>(p, slot, 1, ktb, k.b2), TB, fb, pol_last);
-            }
-          } else {
-            const bool same = diag && kta == ktb;
-            ptx::mbar_arrive_expect_tx(fb, same ? 2 * TB : 4 * TB);
-            ptx::bulk_load_hint(dst, ring_tile<FMT>(p, slot, 0, kta, k.a), TB, fb, pol_last);
-            ptx::bulk_load_hint(dst + TB, ring_tile<FMT>(p, slot, 1, kta, k.a), TB, fb, pol_last);
-            if (!same) {
-              ptx::bulk_load_hint(dst + 2 * TB, ring_tile<FMT>(p, slot, 0, ktb, k.b), TB, fb, pol_last);
-              ptx::bulk_load_hint(dst + 3 * TB, ring_tile<FMT>(p, slot, 1, ktb, k.b), TB, fb, pol_last);
+          bool got = true;
+          if (lane == 0) {
+            got = ptx::wait_bounded(empty_bar(stage), phase ^ 1u, wc);
+            if (got) {
+              // The MMAs of an item's last step of a segment have read it.
+              if (rel_mask >> stage & 1u) release(stage);
+              stage_acc[stage] = word;  // published by the arrive below
+              if (jlast && seg_end && leader) {
+                rel[stage] = p.done + slot;
+                rel_mask |= 1u << stage;
+              }
+              if constexpr (PAIR) {
+                // A: this CTA's row block (not needed by an idle CTA); B: this
+                // CTA's half of the column block (always: the leader's MMA reads it).
+                constexpr int HB = TB / 2;
+                ptx::mbar_arrive_expect_tx(fb, (k.idle ? 1 : 3) * TB);
+                if (!k.idle) ptx::bulk_load_hint(dst, ar, 2 * TB, fb, pol_last);
+                ptx::bulk_load_hint(dst + 2 * TB, br + rank * HB, HB, fb, pol_last);
+                ptx::bulk_load_hint(dst + 2 * TB + HB, br + TB + rank * HB, HB, fb, pol_last);
+              } else if constexpr (WIDE) {
+                // Ar, Ai; then Br of both column blocks back to back (one 256-row
+                // operand: the second tile starts 16 groups on), and Bi likewise.
+                ptx::mbar_arrive_expect_tx(fb, two ? 6 * TB : 4 * TB);
+                ptx::bulk_load_hint(dst, ar, 2 * TB, fb, pol_last);
+                ptx::bulk_load_hint(dst + 2 * TB, br, TB, fb, pol_last);
+                ptx::bulk_load_hint(dst + 4 * TB, br + TB, TB, fb, pol_last);
+                if (two) {
+                  const uint8_t* br2 = br + static_cast<int64_t>(k.b2 - k.b) * FmtT<FMT, SHAPE>::kKbBytes;
+                  ptx::bulk_load_hint(dst + 3 * TB, br2, TB, fb, pol_last);
+                  ptx::bulk_load_hint(dst + 5 * TB, br2 + TB, TB, fb, pol_last);
+                }
+              } else {
+                constexpr int OB = 2 * TB;  // one operand
+                ptx::mbar_arrive_expect_tx(fb, same ? OB : 2 * OB);
+                ptx::bulk_load_hint(dst, ar, OB, fb, pol_last);
+                if (!same) ptx::bulk_load_hint(dst + OB, br, OB, fb, pol_last);
+              }
             }
           }
-          issued_phase[stage] = static_cast<int>(phase);
+          if (!__all_sync(0xffffffffu, got)) {
+            ok = false;
+            break;
+          }
+          ++issued;
           if (++stage == kStages) {
             stage = 0;
             phase ^= 1u;
           }
         }
+        if (++kl == p.seg_kb) {
+          kl = 0;
+          ++seg;
+          slot += width;
+          while (slot >= p.ring_slots) slot -= p.ring_slots;
+          slot_base = p.ring + slot * slot_step;
+        }
+      }
+    }
+    if (lane == 0) {
+      // The last segments' releases: other CTAs' converters may wait for them.
+      for (int s = 0; ok && s < kStages; ++s) {
+        if (!(rel_mask >> s & 1u)) continue;
+        if (ptx::wait_bounded(empty_bar(s), fill_phase(s), wc))
+          release(s);
+        else
+          ok = false;
       }
       if (!ok) {
         for (int s = 0; s < kStages; ++s) {
-          if (issued_phase[s] < 0) continue;
+          if (issued <= s) continue;
           const uint64_t t0 = ptx::globaltimer();
-          while (!ptx::mbar_try_wait(full_bar(s), static_cast<uint32_t>(issued_phase[s])) &&
+          while (!ptx::mbar_try_wait(full_bar(s), fill_phase(s)) &&
                  ptx::globaltimer() - t0 < wc.timeout_ns) {
           }
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1 && PAIR && !leader) {
     // ------------------------------------------------ peer relay (pairs)
     // Forwards each completed stage of this CTA to the leader's pfull.
@@ -1594,7 +1891,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
       for (long long it = it0; ok && it < nitems; it += istep) {
         sb = advance_sub<MULTI>(bt.item_base, bt.nsub, it, sb);
         const Params& p = bt.sub[sb];
-        for (int st = 0; st < p.nkb * FmtT<FMT>::kSteps; ++st) {
+        for (int st = 0; st < p.nkb * kSteps; ++st) {
           if (!ptx::wait_bounded(full_bar(stage), phase, wc)) {
             ok = false;
             break;
@@ -1609,162 +1906,180 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t u = 0;
-      bool ok = true;
-      bool issued_any = false;
-      int sb = 0;
-      for (long long it = it0; ok && it < nitems; it += istep) {
-        sb = advance_sub<MULTI>(bt.item_base, bt.nsub, it, sb);
-        const Params& p = bt.sub[sb];
-        const Blk k = item_block<SHAPE>(p, it - bt.item_base[sb], rank);
-        const bool diag = SHAPE == kShape128 && k.a == k.b;
-        // MMA shape.  128 x 128: M = 128 rows, N trimmed to the block's valid
-        // columns (rounded up to 16), so ragged edge blocks skip the zero
-        // columns.  Pairs: M = 256 (both row blocks), N = 128, 64 per CTA.
-        // 128 x 256: N = 128 + the second block's valid columns.
-        uint32_t idesc;
+    // The whole warp walks the stages, so that loop state and descriptors are
+    // warp-uniform (uniform registers, which tcgen05.mma takes them from); one
+    // elected lane issues.  What the thread does between the last MMA of a
+    // stage and the first of the next is not hidden by the MMA queue: a stage
+    // cost about 600 cycles more than its MMAs when one lane ran this loop and
+    // worked out each item's coordinates itself.
+    const bool issuer = ptx::elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t u = 0;
+    bool ok = true;
+    int sb = 0;
+    // Accumulation groups: an exact chunk (8-bit input), an fp32 chunk, or one
+    // K-block when the epilogue sums 64-sample fp32 blocks in TMEM (buffer 0
+    // only).  The producer says where they start and, where it knows (not for
+    // 8-bit chunks, whose end depends on the next segment's values), end.
+    auto commit_acc = [&](uint32_t ab) {
+      if (issuer) {
         if constexpr (PAIR) {
-          idesc = ptx::idesc_f16_f32(2 * kBlk, kBlk);
+          ptx::mma_commit_pair_mc(accf_bar(ab), 0x3);
         } else {
-          // (The second column block of a 128 x 256 item sits right after the
-          // first in shared memory, whatever their block indices.)
-          const bool two = WIDE && k.b2 >= 0;
-          const int last_b = two ? k.b2 : k.b;
-          const int ncols = (two ? kBlk : 0) + min(kBlk, p.n - last_b * kBlk);
-          idesc = ptx::idesc_f16_f32(kBlk, (ncols + 15) & ~15);
+          ptx::mma_commit(accf_bar(ab));
         }
-        const uint32_t idesc_negb = idesc | (1u << 14);
-        // The item's first stage (its data and its chunk length).  Waiting for
-        // it again in the step loop returns at once: the stage cannot complete
-        // another phase before these MMAs release it.
-        if (!ptx::wait_bounded(full_bar(stage), phase, wc) ||
-            (PAIR && !ptx::wait_bounded(pfull_bar(stage), phase, wc))) {
-          ok = false;
-          break;
-        }
-        const int chunk_kb = item_chunk[stage];
-        const int nchunks = (p.nkb + chunk_kb - 1) / chunk_kb;
-        // The item's first step needs no second wait.
-        bool waited = true;
-        for (int ch = 0; ok && ch < nchunks; ++ch) {
-          const int kb0 = ch * chunk_kb;
-          const int kb1 = min(p.nkb, kb0 + chunk_kb);
-          // Accumulation groups: the whole chunk, or one K-block per group when
-          // the epilogue sums 64-sample fp32 blocks in TMEM (buffer 0 only).
-          const int gstep = kTmemSum ? 1 : (kb1 - kb0);
-          for (int g0 = kb0; ok && g0 < kb1; g0 += gstep) {
-          const int g1 = min(kb1, g0 + gstep);
-          const uint32_t ab = kOneSet ? 0u : (u & 1u);
-          const uint32_t ap = kOneSet ? (u & 1u) : ((u >> 1) & 1u);
-          if (!ptx::wait_bounded(acce_bar(ab), ap ^ 1u, wc)) {
+      }
+    };
+    // Descriptors of stage 0's Ar; the other operands and stages and the
+    // K-steps add their byte offsets (16-byte units) to the address field,
+    // which cannot carry: every shared-memory address is below 256 KiB.
+    const uint64_t desc0 = ptx::interleave_kmajor_desc(sbase, kCoreBytes, FmtT<FMT, SHAPE>::kSbo);
+    constexpr uint64_t kStageDesc = C::kStageBytes >> 4, kTileDesc = TB >> 4;
+    // The next stage's word, once it is known to be full: looked up while the
+    // MMA queue still holds work, so that little but the issue itself lies
+    // between two stages' MMAs.
+    bool ahead = false;
+    uint32_t word = 0;
+    for (long long it = it0; ok && it < nitems; it += istep) {
+      sb = advance_sub<MULTI>(bt.item_base, bt.nsub, it, sb);
+      const int nsteps = bt.sub[sb].nkb * kSteps;
+      bool open = false;
+      uint32_t ab = 0, d_acc = 0, started = 0;
+      for (int st = 0; st < nsteps; ++st) {
+        if (!ahead) {
+          const bool got = ptx::wait_bounded(full_bar(stage), phase, wc) &&
+                           (!PAIR || ptx::wait_bounded(pfull_bar(stage), phase, wc));
+          if (!__all_sync(0xffffffffu, got)) {
             ok = false;
             break;
           }
-          ptx::tc_fence_after();
-          const uint32_t d_re = tmem + ab * 256;
-          const uint32_t d_im = d_re + (WIDE ? 256 : 128);
-          for (int st = g0 * FmtT<FMT>::kSteps; st < g1 * FmtT<FMT>::kSteps; ++st) {
-            if (!waited && (!ptx::wait_bounded(full_bar(stage), phase, wc) ||
-                            (PAIR && !ptx::wait_bounded(pfull_bar(stage), phase, wc)))) {
-              ok = false;
-              break;
-            }
-            waited = false;
-            const int nstage = stage + 1 == kStages ? 0 : stage + 1;
-            const uint32_t nphase = stage + 1 == kStages ? phase ^ 1u : phase;
-            ptx::tc_fence_after();
-            const uint32_t ar = sbase + stage * C::kStageBytes;
-            const uint32_t ai = ar + TB;
-            uint32_t br, bi;
-            if constexpr (PAIR) {
-              br = ar + 2 * TB;
-              bi = br + TB / 2;
-            } else if constexpr (WIDE) {
-              br = ar + 2 * TB;
-              bi = ar + 4 * TB;
-            } else {
-              const bool same = diag && (FMT != kFmtHiLo || st % 3 == 0);
-              br = same ? ar : ar + 2 * TB;
-              bi = same ? ai : ar + 3 * TB;
-            }
-            // Descriptors of the stage's four operands; K-step kk adds its byte
-            // offset (16-byte units) to the address field, which cannot carry:
-            // every shared-memory address is below 256 KiB.
-            constexpr uint32_t SBO = FmtT<FMT>::kSbo;
-            const uint64_t dar0 = ptx::interleave_kmajor_desc(ar, kCoreBytes, SBO);
-            const uint64_t dai0 = ptx::interleave_kmajor_desc(ai, kCoreBytes, SBO);
-            const uint64_t dbr0 = ptx::interleave_kmajor_desc(br, kCoreBytes, SBO);
-            const uint64_t dbi0 = ptx::interleave_kmajor_desc(bi, kCoreBytes, SBO);
-#pragma unroll
-            for (int kk = 0; kk < FmtT<FMT>::kChunks / 2; ++kk) {
-              const uint32_t acc = (st > g0 * FmtT<FMT>::kSteps || kk > 0) ? 1u : 0u;
-              // K-step kk covers 16-byte chunks 2kk and 2kk + 1 (16 fp16 or 32 e4m3 samples).
-              const uint64_t kd = static_cast<uint64_t>(kk * 2 * kCoreBytes) >> 4;
-              const uint64_t dar = dar0 + kd, dai = dai0 + kd, dbr = dbr0 + kd, dbi = dbi0 + kd;
-
-              if constexpr (PAIR && FMT == kFmtF8) {
-                ptx::mma_f8_ss_pair(d_re, dar, dbr, idesc, acc);       // Re += Ar Br^T
-                ptx::mma_f8_ss_pair(d_re, dai, dbi, idesc, 1u);        // Re += Ai Bi^T
-                ptx::mma_f8_ss_pair(d_im, dai, dbr, idesc, acc);       // Im += Ai Br^T
-                ptx::mma_f8_ss_pair(d_im, dar, dbi, idesc_negb, 1u);   // Im -= Ar Bi^T
-              } else if constexpr (PAIR) {
-                ptx::mma_f16_ss_pair(d_re, dar, dbr, idesc, acc);
-                ptx::mma_f16_ss_pair(d_re, dai, dbi, idesc, 1u);
-                ptx::mma_f16_ss_pair(d_im, dai, dbr, idesc, acc);
-                ptx::mma_f16_ss_pair(d_im, dar, dbi, idesc_negb, 1u);
-              } else if constexpr (FMT == kFmtF8) {
-                ptx::mma_f8_ss(d_re, dar, dbr, idesc, acc);
-                ptx::mma_f8_ss(d_re, dai, dbi, idesc, 1u);
-                ptx::mma_f8_ss(d_im, dai, dbr, idesc, acc);
-                ptx::mma_f8_ss(d_im, dar, dbi, idesc_negb, 1u);
-              } else {
-                ptx::mma_f16_ss(d_re, dar, dbr, idesc, acc);
-                ptx::mma_f16_ss(d_re, dai, dbi, idesc, 1u);
-                ptx::mma_f16_ss(d_im, dai, dbr, idesc, acc);
-                ptx::mma_f16_ss(d_im, dar, dbi, idesc_negb, 1u);
-              }
-            }
-            issued_any = true;
-            if constexpr (PAIR) {
-              ptx::mma_commit_pair_mc(empty_bar(stage), 0x3);
-            } else {
-              ptx::mma_commit(empty_bar(stage));
-            }
-            stage = nstage;
-            phase = nphase;
-
+          word = __shfl_sync(0xffffffffu, static_cast<uint32_t>(stage_acc[stage]), 0);
+        }
+        if (word & kAccStart) {
+          if (open) {
+            commit_acc(ab);
+            ++u;
           }
-          if (!ok) break;
-          if constexpr (PAIR) {
-            ptx::mma_commit_pair_mc(accf_bar(ab), 0x3);
+          ab = kOneSet ? 0u : (u & 1u);
+          const uint32_t ap = kOneSet ? (u & 1u) : ((u >> 1) & 1u);
+          const bool drained = ptx::wait_bounded(acce_bar(ab), ap ^ 1u, wc);
+          if (!__all_sync(0xffffffffu, drained)) {
+            ok = false;
+            break;
+          }
+          d_acc = tmem + ab * 256;
+          open = true;
+          started = 0;
+        }
+        ptx::tc_fence_after();
+        const uint32_t d_re = d_acc + kReCol, d_im = d_acc + kImCol;
+        const int mma_n = static_cast<int>(word >> kAccNShift);
+        const uint32_t idesc = ptx::idesc_f16_f32(PAIR ? 2 * kBlk : kBlk, mma_n);
+        const uint32_t idesc_negb = idesc | (1u << 14);
+        const uint64_t dar0 = desc0 + static_cast<uint64_t>(stage) * kStageDesc;
+        const bool same = !PAIR && !WIDE && (word & kAccSame);
+        const uint64_t dbr0 = same ? dar0 : dar0 + 2 * kTileDesc;
+        // Full 128 x 128 blocks: Im += Ai Br^T and Re += Ai Bi^T in one
+        // 128 x 256 MMA (the Br and Bi tiles and the two accumulators lie side
+        // by side), then Re += Ar Br^T, Im -= Ar Bi^T.  The wide MMA reads Ai
+        // from shared memory once for both: 28 instead of 32 KiB per K-step of
+        // the shared-memory bandwidth that the stage copies and the converters
+        // share.  Alone, with stages arriving, 64 samples take 1025 cycles this
+        // way and 1114 with four 128 x 128 MMAs (1024 is the tensor rate).
+        constexpr uint32_t idesc2 = ptx::idesc_f16_f32(kBlk, 2 * kBlk);
+        const bool full_blk = SHAPE == kShape128 && mma_n == kBlk;
+        // K-step kk: 16-byte chunks 2kk and 2kk + 1 (16 fp16 or 32 e4m3 samples).
+        auto kstep = [&](int kk) {
+          const uint32_t acc = kk > 0 ? 1u : started;
+          const uint64_t kd = static_cast<uint64_t>(kk * 2 * kCoreBytes) >> 4;
+          const uint64_t dar = dar0 + kd, dai = dar + kTileDesc;
+          const uint64_t dbr = dbr0 + kd;
+          const uint64_t dbi = dbr + (PAIR ? kTileDesc / 2 : (WIDE ? 2 : 1) * kTileDesc);
+          if constexpr (PAIR && FMT == kFmtF8) {
+            ptx::mma_f8_ss_pair(d_re, dar, dbr, idesc, acc);       // Re += Ar Br^T
+            ptx::mma_f8_ss_pair(d_re, dai, dbi, idesc, 1u);        // Re += Ai Bi^T
+            ptx::mma_f8_ss_pair(d_im, dai, dbr, idesc, acc);       // Im += Ai Br^T
+            ptx::mma_f8_ss_pair(d_im, dar, dbi, idesc_negb, 1u);   // Im -= Ar Bi^T
+          } else if constexpr (PAIR) {
+            ptx::mma_f16_ss_pair(d_re, dar, dbr, idesc, acc);
+            ptx::mma_f16_ss_pair(d_re, dai, dbi, idesc, 1u);
+            ptx::mma_f16_ss_pair(d_im, dai, dbr, idesc, acc);
+            ptx::mma_f16_ss_pair(d_im, dar, dbi, idesc_negb, 1u);
+          } else if (full_blk) {
+            if constexpr (FMT == kFmtF8) {
+              ptx::mma_f8_ss(d_im, dai, dbr, idesc2, acc);
+              ptx::mma_f8_ss(d_re, dar, dbr, idesc, 1u);
+              ptx::mma_f8_ss(d_im, dar, dbi, idesc_negb, 1u);
+            } else {
+              ptx::mma_f16_ss(d_im, dai, dbr, idesc2, acc);
+              ptx::mma_f16_ss(d_re, dar, dbr, idesc, 1u);
+              ptx::mma_f16_ss(d_im, dar, dbi, idesc_negb, 1u);
+            }
+          } else if constexpr (FMT == kFmtF8) {
+            ptx::mma_f8_ss(d_re, dar, dbr, idesc, acc);
+            ptx::mma_f8_ss(d_re, dai, dbi, idesc, 1u);
+            ptx::mma_f8_ss(d_im, dai, dbr, idesc, acc);
+            ptx::mma_f8_ss(d_im, dar, dbi, idesc_negb, 1u);
           } else {
-            ptx::mma_commit(accf_bar(ab));
+            ptx::mma_f16_ss(d_re, dar, dbr, idesc, acc);
+            ptx::mma_f16_ss(d_re, dai, dbi, idesc, 1u);
+            ptx::mma_f16_ss(d_im, dai, dbr, idesc, acc);
+            ptx::mma_f16_ss(d_im, dar, dbi, idesc_negb, 1u);
           }
+        };
+        constexpr int kAll = FmtT<FMT, SHAPE>::kChunks / 2;
+        if (issuer) {
+#pragma unroll
+          for (int kk = 0; kk < kAll - 1; ++kk) kstep(kk);
+        }
+        __syncwarp();
+        const int nstage = stage + 1 == kStages ? 0 : stage + 1;
+        const uint32_t nphase = stage + 1 == kStages ? phase ^ 1u : phase;
+        ahead = ptx::mbar_test_wait(full_bar(nstage), nphase) &&
+                (!PAIR || ptx::mbar_test_wait(pfull_bar(nstage), nphase));
+        ahead = __all_sync(0xffffffffu, ahead);
+        uint32_t next_word = 0;
+        if (ahead) next_word = __shfl_sync(0xffffffffu, static_cast<uint32_t>(stage_acc[nstage]), 0);
+        if (issuer) {
+          kstep(kAll - 1);
+          if constexpr (PAIR) {
+            ptx::mma_commit_pair_mc(empty_bar(stage), 0x3);
+          } else {
+            ptx::mma_commit(empty_bar(stage));
+          }
+        }
+        started = 1;
+        if (word & kAccEnd) {
+          commit_acc(ab);
           ++u;
-          }
+          open = false;
         }
-      }
-      if (!ok && issued_any) {
-        if constexpr (PAIR) {
-          ptx::mma_commit_pair_mc(drain_bar, 0x1);
-        } else {
-          ptx::mma_commit(drain_bar);
-        }
-        const uint64_t t0 = ptx::globaltimer();
-        while (!ptx::mbar_try_wait(drain_bar, 0) && ptx::globaltimer() - t0 < wc.timeout_ns) {
-        }
+        word = next_word;
+        stage = nstage;
+        phase = nphase;
       }
     }
+    if (!ok && issuer) {
+      // The MMAs issued so far complete before TMEM is freed (bounded).
+      if constexpr (PAIR) {
+        ptx::mma_commit_pair_mc(drain_bar, 0x1);
+      } else {
+        ptx::mma_commit(drain_bar);
+      }
+      const uint64_t t0 = ptx::globaltimer();
+      while (!ptx::mbar_try_wait(drain_bar, 0) && ptx::globaltimer() - t0 < wc.timeout_ns) {
+      }
+    }
+    __syncwarp();
   } else if (warp < 2 + kNumEpiWarps) {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;
     const uint32_t t_lanes = tmem + (static_cast<uint32_t>(q * 32) << 16);
     uint32_t u = 0;
     bool ok = true;
-    int sb = 0;
+    // The visibilities are written once: first in line for L2 replacement.
+    const uint64_t pol_out = ptx::l2_policy_evict_first();
     // Accumulator b has been read: local arrive, or remote on the leader's barrier.
     auto release_acc = [&](uint32_t ab) {
       ptx::tc_fence_before();
@@ -1776,11 +2091,11 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           ptx::mbar_arrive_remote(ptx::mapa_shared(acce_bar(ab), 0));
       }
     };
-    for (long long it = it0; ok && it < nitems; it += istep) {
-      sb = advance_sub<MULTI>(bt.item_base, bt.nsub, it, sb);
-      const Params& p = bt.sub[sb];
+    for (Item x = item_start<MULTI>(bt, it0, nitems); ok && x.it < nitems;
+         item_step<MULTI>(bt, x, istep, nitems)) {
+      const Params& p = bt.sub[x.sb];
       const int P = p.g.P;
-      const Blk k = item_block<SHAPE>(p, it - bt.item_base[sb], rank);
+      const Blk k = item_block<SHAPE>(p, x, rank);
       const int f = k.f;
       const int a = k.a * kBlk + q * 32 + lane;  // this thread's row input
       // The item's column blocks and, per block, the pieces piece0..last this
@@ -1794,12 +2109,11 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
         const int b = cb[j];
         if (k.idle) continue;
         if (b > k.a) {
-          for (int piece = 0; piece < kBlk / 32; ++piece)
-            if (b * kBlk + piece * 32 < p.n) last_p[j] = piece;
+          last_p[j] = min(kBlk / 32 - 1, (p.n - 1 - b * kBlk) >> 5);
         } else {
-          const int s1_hi = min(p.g.N - 1, (k.a * kBlk + q * 32 + 31) / P);
-          for (int piece = 0; piece < kBlk / 32; ++piece)
-            if ((b * kBlk + piece * 32) / P <= s1_hi) last_p[j] = piece;
+          // The last input of this warp's highest station row.
+          const int hi = min(p.n - 1, k.a * kBlk + q * 32 + 31);
+          last_p[j] = max(-1, min(kBlk / 32 - 1, (hi - b * kBlk) >> 5));
           if (p.pack > 1) {
             const int col0 = (k.a * kBlk + q * 32) / P / p.Nr * p.Nr * P;  // first column of that channel
             first_p[j] = max(0, (col0 - b * kBlk) / 32);
@@ -1809,19 +2123,38 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
       }
       // The last block with pieces to read releases the accumulator after them.
       const int jlast = (nblk == 2 && last_p[1] >= 0) ? 1 : (last_p[0] >= 0 ? 0 : -1);
-      const bool rdy = channel_ready(p, f, abort_flag);
-      if (!__all_sync(0xffffffffu, rdy)) {
-        ok = false;
-        break;
+      // 8-bit input: does one exact chunk hold the whole integration?  (Lane l
+      // looks at segments l, l + 32, ... once they are converted.)
+      bool one_chunk = true;
+      int width;
+      const int G0 = seg_first(p, f, &width);
+      if constexpr (IS_INT) {
+        bool rdy = true;
+        unsigned sum = 0;  // capped: at most 32 lanes x 2^25
+        for (int sg = lane; sg < p.nseg; sg += 32) {
+          const int G = G0 + sg * width, gen = fast_div(G, p.ring_slots, p.mag_slots);
+          rdy = rdy && wait_counter(p.ready + G - gen * p.ring_slots,
+                                    static_cast<unsigned>(gen + 1) * static_cast<unsigned>(p.seg_units), p,
+                                    abort_flag);
+          const unsigned nk = static_cast<unsigned>(min(p.seg_kb, p.nkb - sg * p.seg_kb));
+          sum = min(sum + min(nk * kblock_growth(p, G), 2 * kExactSum), 2 * kExactSum);
+        }
+        if (!__all_sync(0xffffffffu, rdy)) {
+          ok = false;
+          break;
+        }
+        one_chunk = __reduce_add_sync(0xffffffffu, sum) <= kExactSum;
       }
-      const int chunk_kb = chunk_kblocks(p, f);
-      const int nchunks = (p.nkb + chunk_kb - 1) / chunk_kb;
-      for (int ch = 0; ok && ch < nchunks; ++ch) {
-        const int kb0 = ch * chunk_kb;
-        const int kb1 = min(p.nkb, kb0 + chunk_kb);
+      int ch = -1;
+      for (int kb0 = 0, kb1; ok && kb0 < p.nkb; kb0 = kb1) {
+        ++ch;
+        if (IS_INT)
+          kb1 = one_chunk ? p.nkb : exact_chunk_end(p, G0, width, kb0);
+        else
+          kb1 = min(p.nkb, kb0 + p.f_chunk_kb);
         const int gstep = kTmemSum ? 1 : (kb1 - kb0);
         const bool add = p.accumulate || ch > 0;
-        const bool last_chunk = ch == nchunks - 1;
+        const bool last_chunk = kb1 == p.nkb;
         // FP64 block sums: chunks pair off, (0, 1), (2, 3), ...  The first
         // chunk of a pair stays in its TMEM accumulator (`hold`); the second's
         // drain adds it in fp32 (a correctly rounded sum of the two partials,
@@ -1829,7 +2162,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
         // running sum once per pair: half the passes over it, none at all for
         // an integration of two chunks.  Needs the two accumulator sets.
         const bool f64pair = !IS_INT && !kOneSet && p.acc64 != nullptr;
-        const bool hold = f64pair && (ch % 2 == 0) && ch + 1 < nchunks;
+        const bool hold = f64pair && (ch % 2 == 0) && !last_chunk;
         const bool paired = f64pair && (ch % 2 == 1);
         const bool first = f64pair ? ch < 2 : ch == 0;
         for (int g0 = kb0; g0 < kb1; g0 += gstep) {
@@ -1863,11 +2196,6 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
             break;
           }
           ptx::tc_fence_after();
-          // The item's last group is complete, so every MMA of the item (in
-          // both CTAs of a pair) has read its operands: the item is done with
-          // its ring slot.  (Released here, off the MMA thread's path.)
-          if (last_chunk && glast && q == 0 && lane == 0 && leader)
-            red_release_add(p.done + (f % p.ring_slots), 1u);
           if (hold) {  // drained with the next chunk
             ++u;
             continue;
@@ -1876,8 +2204,8 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
             // Add the held chunk into this one inside TMEM and free it at
             // once, so the next item's MMAs need not wait for the stores.
             for (int j = 0; j < nblk; ++j) {
-              const uint32_t c_re = ab * 256, c_im = ab * 256 + 128;
-              const uint32_t h_re = (ab ^ 1u) * 256, h_im = (ab ^ 1u) * 256 + 128;
+              const uint32_t c_re = ab * 256 + kReCol, c_im = ab * 256 + kImCol;
+              const uint32_t h_re = (ab ^ 1u) * 256 + kReCol, h_im = (ab ^ 1u) * 256 + kImCol;
 #pragma unroll 1
               for (int piece = first_p[j]; piece <= last_p[j]; ++piece) {
                 uint32_t vr[32], vi[32], sr[32], si[32];
@@ -1902,8 +2230,8 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           for (int j = 0; j < nblk; ++j) {
             const int b = cb[j];
             // TMEM columns of block j: D_re and D_im of its 128 columns.
-            const uint32_t c_re = WIDE ? j * kBlk : ab * 256;
-            const uint32_t c_im = WIDE ? 256 + j * kBlk : ab * 256 + 128;
+            const uint32_t c_re = WIDE ? j * kBlk : ab * 256 + kReCol;
+            const uint32_t c_im = WIDE ? 256 + j * kBlk : ab * 256 + kImCol;
 #pragma unroll 1
             for (int piece = first_p[j]; piece <= last_p[j]; ++piece) {
               uint32_t vr[32], vi[32];
@@ -1933,9 +2261,9 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
               const bool tr = b > k.a;  // a mirrored block
               if constexpr (IS_INT) {
                 if (tr)
-                  store_piece_tr<true>(vr, vi, p, f, a, b0, add);
+                  store_piece_tr<kWordInt>(vr, vi, p, f, a, b0, add, pol_out);
                 else
-                  store_piece<true>(vr, vi, p, f, a, b0, add);
+                  store_piece<kWordInt>(vr, vi, p, f, a, b0, add, pol_out);
               } else {
                 if (p.in_amax) scale_piece<FMT>(vr, vi, p, f, a, b0);
                 // A drain that is both the first and the last of the running
@@ -1945,16 +2273,16 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
                   if (tr)
                     store_piece_f64_tr(vr, vi, p, f, a, b0, first, last_chunk);
                   else
-                    store_piece_f64(vr, vi, p, f, a, b0, first, last_chunk);
+                    store_piece_f64(vr, vi, p, f, a, b0, first, last_chunk, pol_out);
                 } else {
                   // With block sums on, this drain holds the whole
                   // integration: it overwrites `out` (a paired chunk's
                   // ch > 0 must not make it add).
                   const bool add_out = add && !p.acc64;
                   if (tr)
-                    store_piece_tr<false>(vr, vi, p, f, a, b0, add_out);
+                    store_piece_tr<kWordFloat>(vr, vi, p, f, a, b0, add_out, pol_out);
                   else
-                    store_piece<false>(vr, vi, p, f, a, b0, add_out);
+                    store_piece<kWordFloat>(vr, vi, p, f, a, b0, add_out, pol_out);
                 }
               }
             }
@@ -1970,15 +2298,15 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
     const uint32_t cbuf = sbase + C::kConvOff + cw * kConvBufBytes;
     if constexpr (DT == 0) {
       if (bt.sub[0].tma_in) {  // set for every subarray or for none
-        converter_tma<FMT, MULTI>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
+        converter_tma<FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
       } else {
-        converter_direct<DT, FMT, MULTI>(bt, cw, lane, abort_flag);
+        converter_direct<DT, FMT, MULTI, SHAPE>(bt, cw, lane, abort_flag);
       }
     } else {
       if (bt.sub[0].tma_in) {
-        converter_tma_float<DT, FMT, MULTI>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
+        converter_tma_float<DT, FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
       } else {
-        converter_direct<DT, FMT, MULTI>(bt, cw, lane, abort_flag);
+        converter_direct<DT, FMT, MULTI, SHAPE>(bt, cw, lane, abort_flag);
       }
     }
   }

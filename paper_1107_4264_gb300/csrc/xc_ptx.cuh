@@ -49,6 +49,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Has the phase with this parity completed?  (No wait.)
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait for the phase of `bar` with parity `parity` to complete.
 // Gives up when another role of the CTA has already given up (*abort set) or
 // after timeout_ns of wall time; then it records kStatusTimeout in the
@@ -149,6 +162,17 @@ __device__ __forceinline__ void st_global_v4_hint(void* p, uint32_t a, uint32_t 
   asm volatile("st.global.L1::no_allocate.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p),
                "r"(a), "r"(b), "r"(c), "r"(d), "l"(pol)
                : "memory");
+}
+
+// True in one lane of a converged warp, the same one each time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 // ---------------------------------------------------------------- tcgen05
