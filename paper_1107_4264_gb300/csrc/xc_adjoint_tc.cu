@@ -8,18 +8,24 @@
 //     grad_g[a]   += sum_t conj(x[t][a]) grad_y[a][t],
 //
 // a complex GEMM with M = a (inputs), N = t (samples), K = b (inputs).  It
-// runs on tcgen05 in the planar form of the forward engine:
-//     Re = Hr Xr^T - Hi Xi^T,   Im = Hr Xi^T + Hi Xr^T
-// (four MMAs per 16-b step, the second with negate-B).  Operands are split
-// into fp16 hi + lo parts after a power-of-two scale per channel (from the
-// largest component), and each 64-b block runs three steps (hi hi, lo hi,
-// hi lo), about 22 significant bits with fp32 accumulation over K = n.
+// runs on tcgen05 in planar form:
+//     Re = Hr Xr^T - Hi Xi^T,   Im = Hr Xi^T + Hi Xr^T,
+// per 16-b step one 128 x 256 MMA, Hr [Xr Xi]^T into the adjacent accumulators
+// (D_re | D_im), and two of 128 x 128, Re -= Hi Xi^T (negate-B) and
+// Im += Hi Xr^T.  Operands are split into fp16 hi + lo parts after a
+// power-of-two scale per row (input a of H', sample t of x, from its largest
+// component), and each step runs three times (hi hi, lo hi, hi lo): about 22
+// significant bits with fp32 accumulation over K = n.
 //
-// Kernels: amax of H' and of x per channel; operand formation into 16 KiB
-// MMA-ready tiles ([8-column chunk][128 rows][8 fp16], the no-swizzle K-major
-// layout); the GEMM, a persistent kernel over 128 x 128 (a, t) tiles with a
-// bulk-copy producer warp, an MMA warp and four epilogue warps that re-read
-// x (nothing from the forward is stored).
+// Kernels: operand formation, one pass over x and one over grad_out (H' is
+// formed straight from it), into 8 KiB MMA-ready tiles ([8-row group]
+// [8-column chunk][8 rows][8 fp16], the no-swizzle K-major layout, in which two
+// tiles one after the other are one operand of 256 rows); the GEMM, a persistent
+// kernel over 128 x 128 (a, t) tiles with a bulk-copy producer warp, an MMA
+// warp and eight epilogue warps that re-read x (nothing from the forward is
+// stored).  A stage holds all eight tiles of 32 b (hi and lo, re and im, of
+// both operands), 64 KiB for 18 MMAs: the three combinations share their
+// operands' copies.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -32,25 +38,28 @@ namespace xc {
 namespace {
 
 constexpr int kBlk = 128;  // rows per tile (a or t)
-constexpr int kBK = 64;    // K (b) per tile
+constexpr int kBK = 32;    // K (b) per tile
 constexpr int kTile = kBlk * kBK * 2;
-constexpr uint32_t kChunkStride = kBlk * 16;
-constexpr uint32_t kGroupStride = 8 * 16;
+constexpr uint32_t kChunkStride = 8 * 16;  // between core matrices (8 rows x 16 B) adjacent in K
+constexpr uint32_t kGroupStride = (kBK / 8) * kChunkStride;  // and in M / N
 constexpr int kStages = 3;
-constexpr int kStageBytes = 4 * kTile;
-constexpr int kThreads = 192;  // producer, MMA, 4 epilogue warps
+constexpr int kOperand = 4 * kTile;  // (hi r, hi i, lo r, lo i)
+constexpr int kStageBytes = 2 * kOperand;
+constexpr int kEpiWarps = 8;  // two per TMEM lane quarter, half of the columns each
+constexpr int kThreads = 32 * (2 + kEpiWarps);  // producer, MMA, epilogue
 constexpr int kBarOff = kStages * kStageBytes;
 constexpr int kNumBars = 2 * kStages + 5;
 constexpr int kSmemBytes = kBarOff + kNumBars * 8 + 16 + 1024;
 constexpr uint32_t kTmemCols = 512;  // 2 sets x (D_re, D_im)
 constexpr uint32_t kIdesc = ptx::idesc_f16_f32(kBlk, kBlk);
 constexpr uint32_t kIdescNegB = kIdesc | (1u << 14);
+constexpr uint32_t kIdescWide = ptx::idesc_f16_f32(kBlk, 2 * kBlk);
 
 struct AdjGeom {
   Geometry g;
   int n;   // complex inputs N * P
   int na;  // 128-row blocks over a
-  int nk;  // 64-column blocks over b (K)
+  int nk;  // 32-column blocks over b (K)
   int nt;  // 128-row blocks over t
 };
 
@@ -67,46 +76,10 @@ __device__ __forceinline__ int adj_scale_exp(unsigned bits) {
 }
 __device__ __forceinline__ float adj_exp2i(int e) { return __int_as_float((127 + e) << 23); }
 
-// Byte offset of tile (f, plane, hl, row block rb, K block kb) in an operand
-// buffer with nrb row blocks per channel.
-__device__ __forceinline__ size_t tile_off(int f, int plane, int hl, int rb, int kb, int nrb, int nk) {
-  return (((((static_cast<size_t>(f) * 2 + plane) * 2 + hl) * nrb + rb) * nk) + kb) *
-         static_cast<size_t>(kTile);
-}
-
-// amax[f] = max |component| of H'_f = H_f diag(g).  Block: 8 rows a of one
-// channel, threads along b.
-__global__ void adj_amax_h(const float2* __restrict__ H, const float2* __restrict__ gains,
-                           unsigned* __restrict__ amax, int n) {
-  const int f = blockIdx.y;
-  float m = 0.f;
-  for (int a = blockIdx.x * 8; a < min(n, blockIdx.x * 8 + 8); ++a) {
-    const float2* row = H + (static_cast<size_t>(f) * n + a) * n;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-      float2 v = row[b];
-      if (gains) v = cmul(v, gains[b]);
-      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax + f, __float_as_uint(m));
-}
-
-// amax[F + f] = max |component| of x over channel f.  Block: 32 samples t of
-// one channel, threads along b.
-__global__ void adj_amax_x(const float2* __restrict__ x, unsigned* __restrict__ amax, Geometry g,
-                           int n) {
-  const int f = blockIdx.y;
-  float m = 0.f;
-  for (int t = blockIdx.x * 32; t < min(g.T, blockIdx.x * 32 + 32); ++t) {
-    const float2* row = x + (static_cast<size_t>(t) * g.F + f) * n;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-      const float2 v = row[b];
-      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax + g.F + f, __float_as_uint(m));
+// Byte offset of the operand tiles (hi r, hi i, lo r, lo i) of (channel f, row
+// block rb, K block kb) in an operand buffer with nrb row blocks per channel.
+__device__ __forceinline__ size_t tile_off(int f, int rb, int kb, int nrb, int nk) {
+  return ((static_cast<size_t>(f) * nrb + rb) * nk + kb) * static_cast<size_t>(kOperand);
 }
 
 // hi + lo fp16 pairs of 8 scaled values: hi[4], lo[4] (two values per word).
@@ -120,72 +93,150 @@ __device__ __forceinline__ void split8(const float (&v)[8], uint32_t (&hi)[4], u
   }
 }
 
-// Write the four 16-byte row chunks (re hi, re lo, im hi, im lo) of row r,
-// chunk c of tile (rb, kb) in channel f.
-__device__ __forceinline__ void put_chunks(uint8_t* buf, int f, int rb, int kb, int nrb, int nk,
-                                           int c, int r, const float (&re)[8], const float (&im)[8]) {
+// Write the four 16-byte row chunks (hi re, hi im, lo re, lo im) of row r,
+// 8-column chunk bc.
+__device__ __forceinline__ void put_chunks(uint8_t* buf, int f, int r, int bc, int nrb, int nk,
+                                           const float (&re)[8], const float (&im)[8]) {
   uint32_t rh[4], rl[4], ih[4], il[4];
   split8(re, rh, rl);
   split8(im, ih, il);
-  const size_t o = static_cast<size_t>(c) * kChunkStride + static_cast<size_t>(r) * 16;
-  *reinterpret_cast<uint4*>(buf + tile_off(f, 0, 0, rb, kb, nrb, nk) + o) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
-  *reinterpret_cast<uint4*>(buf + tile_off(f, 0, 1, rb, kb, nrb, nk) + o) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
-  *reinterpret_cast<uint4*>(buf + tile_off(f, 1, 0, rb, kb, nrb, nk) + o) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
-  *reinterpret_cast<uint4*>(buf + tile_off(f, 1, 1, rb, kb, nrb, nk) + o) = make_uint4(il[0], il[1], il[2], il[3]);
+  uint8_t* o = buf + tile_off(f, r / kBlk, bc / (kBK / 8), nrb, nk) + (r % kBlk / 8) * kGroupStride +
+               (bc % (kBK / 8)) * kChunkStride + (r % 8) * 16;
+  *reinterpret_cast<uint4*>(o) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+  *reinterpret_cast<uint4*>(o + kTile) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+  *reinterpret_cast<uint4*>(o + 2 * kTile) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+  *reinterpret_cast<uint4*>(o + 3 * kTile) = make_uint4(il[0], il[1], il[2], il[3]);
 }
 
-// A operand: H' tiles, rows a (padded to na * 128), K = b (padded to nk * 64).
-// One thread per (row a, 8-column chunk); consecutive threads take
-// consecutive rows, so a warp writes 512 contiguous bytes per plane.
-__global__ void adj_form_h(const float2* __restrict__ H, const float2* __restrict__ gains,
-                           const unsigned* __restrict__ amax, uint8_t* __restrict__ At, AdjGeom G) {
-  const int f = blockIdx.y;
-  const int rows = G.na * kBlk, chunks = G.nk * (kBK / 8);
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= rows * chunks) return;
-  const int a = idx % rows, bc = idx / rows;
-  const float s = adj_exp2i(-adj_scale_exp(amax[f]));
-  float re[8], im[8];
+// Operand formation of 16 rows: thread (r, c) = (tid & 15, tid >> 4) takes
+// chunks c, c + 16, ... of row r (consecutive threads take consecutive rows, so
+// a warp writes four whole core matrices per plane).  load(chunk, v) gives the
+// chunk's eight values.  Up to NC chunks per thread stay in registers between
+// the row's maximum and its conversion: one pass over the input (rows of more
+// chunks are loaded twice).  The row's exponent goes to exps[row].
+constexpr int kFormRows = 16, kFormThreads = 256, kFormCols = kFormThreads / kFormRows;
+template <int NC, typename Load>
+__device__ __forceinline__ void form_rows(Load load, int row, int f, uint8_t* buf, int* exps, int nrb, int nk) {
+  __shared__ unsigned smax[kFormRows];
+  const int r = threadIdx.x % kFormRows, c = threadIdx.x / kFormRows;
+  const int nch = nk * (kBK / 8);
+  if (threadIdx.x < kFormRows) smax[threadIdx.x] = 0;
+  __syncthreads();
+  float2 v[NC][8];
+  float m = 0.f;
+  const bool fits = nch <= NC * kFormCols;
+  if (fits) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int b = bc * 8 + j;
-    float2 v = make_float2(0.f, 0.f);
-    if (a < G.n && b < G.n) {
-      v = H[(static_cast<size_t>(f) * G.n + a) * G.n + b];
-      if (gains) v = cmul(v, gains[b]);
+    for (int i = 0; i < NC; ++i)
+      if (c + i * kFormCols < nch) load(c + i * kFormCols, v[i]);
+#pragma unroll
+    for (int i = 0; i < NC; ++i)
+      if (c + i * kFormCols < nch)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) m = fmaxf(m, fmaxf(fabsf(v[i][j].x), fabsf(v[i][j].y)));
+  } else {
+    for (int ch = c; ch < nch; ch += kFormCols) {
+      load(ch, v[0]);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) m = fmaxf(m, fmaxf(fabsf(v[0][j].x), fabsf(v[0][j].y)));
     }
-    re[j] = v.x * s;
-    im[j] = v.y * s;
   }
-  put_chunks(At, f, a / kBlk, bc / (kBK / 8), G.na, G.nk, bc % (kBK / 8), a % kBlk, re, im);
+  // (The lanes l and l + 16 of a warp have the same row.)
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  if ((threadIdx.x & 16) == 0) atomicMax(&smax[r], __float_as_uint(m));
+  __syncthreads();
+  const int e = adj_scale_exp(smax[r]);
+  if (c == 0) exps[row] = e;
+  const float s = adj_exp2i(-e);
+  auto put = [&](int ch, const float2 (&w)[8]) {
+    float re[8], im[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      re[j] = w[j].x * s;
+      im[j] = w[j].y * s;
+    }
+    put_chunks(buf, f, row, ch, nrb, nk, re, im);
+  };
+  if (fits) {
+#pragma unroll
+    for (int i = 0; i < NC; ++i)
+      if (c + i * kFormCols < nch) put(c + i * kFormCols, v[i]);
+  } else {
+    for (int ch = c; ch < nch; ch += kFormCols) {
+      load(ch, v[0]);
+      put(ch, v[0]);
+    }
+  }
 }
 
-// B operand: x tiles, rows t (padded to nt * 128), K = b.
-__global__ void adj_form_x(const float2* __restrict__ x, const unsigned* __restrict__ amax,
-                           uint8_t* __restrict__ Bt, AdjGeom G) {
-  const int f = blockIdx.y;
-  const int rows = G.nt * kBlk, chunks = G.nk * (kBK / 8);
-  const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= static_cast<int64_t>(rows) * chunks) return;
-  const int t = static_cast<int>(idx % rows), bc = static_cast<int>(idx / rows);
-  const float s = adj_exp2i(-adj_scale_exp(amax[G.g.F + f]));
-  float re[8], im[8];
+// A operand: H'_f = H_f diag(g) with H_f = G_f + G_f^H, rows a (padded to na *
+// 128), K = b (padded to nk * 32), straight from the packed grad_out (each
+// off-diagonal entry of it is read twice, through L2): 60 us at 64 channels of
+// 512 inputs (182 us by way of H in memory and a pass for its maximum).
+template <int NC>
+__global__ void __launch_bounds__(kFormThreads) adj_form_h(const float2* __restrict__ grad_out,
+                                                           const float2* __restrict__ gains,
+                                                           uint8_t* __restrict__ At, int* __restrict__ exps,
+                                                           AdjGeom G) {
+  const int f = blockIdx.y, a = blockIdx.x * kFormRows + threadIdx.x % kFormRows;
+  const int P = G.g.P, PP = P * P, sh = P - 1;  // P is 1 or 2
+  const int sa = a >> sh, pa = a & sh;
+  const float2* go = grad_out + static_cast<int64_t>(f) * G.g.NB * PP;
+  const float2* row = go + static_cast<int64_t>(sa) * (sa + 1) / 2 * PP + pa * P;
+  auto load = [&](int ch, float2 (&v)[8]) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int b = bc * 8 + j;
-    float2 v = make_float2(0.f, 0.f);
-    if (t < G.g.T && b < G.n) v = x[(static_cast<size_t>(t) * G.g.F + f) * G.n + b];
-    re[j] = v.x * s;
-    im[j] = v.y * s;
-  }
-  put_chunks(Bt, f, t / kBlk, bc / (kBK / 8), G.nt, G.nk, bc % (kBK / 8), t % kBlk, re, im);
+    for (int j = 0; j < 8; ++j) {
+      const int b = ch * 8 + j, sb = b >> sh, pb = b & sh;
+      float2 h = make_float2(0.f, 0.f);
+      if (a < G.n && b < G.n) {
+        if (sb <= sa) h = row[sb * PP + pb];  // G[a][b]
+        if (sb >= sa) {                       // conj(G[b][a])
+          const float2 w = go[(static_cast<int64_t>(sb) * (sb + 1) / 2 + sa) * PP + pb * P + pa];
+          h.x += w.x;
+          h.y -= w.y;
+        }
+        if (gains) h = cmul(h, gains[b]);
+      }
+      v[j] = h;
+    }
+  };
+  form_rows<NC>(load, a, f, At, exps + static_cast<size_t>(f) * G.na * kBlk, G.na, G.nk);
+}
+
+// B operand: x tiles, rows t (padded to nt * 128), K = b.  Bound by its one
+// read of x and the same bytes written (hi and lo halves): 2.1 GB in 308 us on
+// 256 stations x 2 pols, F=64, T=4096 (a pass for one maximum per channel and
+// one to form the tiles took 241 + 481 us).
+template <int NC>
+__global__ void __launch_bounds__(kFormThreads) adj_form_x(const float2* __restrict__ x, uint8_t* __restrict__ Bt,
+                                                           int* __restrict__ exps, AdjGeom G) {
+  const int f = blockIdx.y, t = blockIdx.x * kFormRows + threadIdx.x % kFormRows;
+  const float2* row = x + (static_cast<int64_t>(t) * G.g.F + f) * G.n;
+  const bool vec = G.n % 2 == 0;  // rows start on 16 bytes
+  auto load = [&](int ch, float2 (&v)[8]) {
+    if (t < G.g.T && vec && ch * 8 + 8 <= G.n) {
+      const float4* q = reinterpret_cast<const float4*>(row + ch * 8);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 w = __ldg(q + j);
+        v[2 * j] = make_float2(w.x, w.y);
+        v[2 * j + 1] = make_float2(w.z, w.w);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        v[j] = t < G.g.T && ch * 8 + j < G.n ? __ldg(row + ch * 8 + j) : make_float2(0.f, 0.f);
+    }
+  };
+  form_rows<NC>(load, t, f, Bt, exps + static_cast<size_t>(f) * G.nt * kBlk, G.nt, G.nk);
 }
 
 struct AdjParams {
   AdjGeom G;
   const uint8_t* At;
   const uint8_t* Bt;
-  const unsigned* amax;  // [2F]: H' then x
+  const int* exp_h;  // [F][na * 128] row exponents of H'
+  const int* exp_x;  // [F][nt * 128] of x
   const float2* x;
   const float2* gains;
   float2* grad_x;
@@ -212,7 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
   const uint32_t drain_bar = bar0 + 8u * (2 * kStages + 4);
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + kBarOff + kNumBars * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known uniform)
+  const int lane = threadIdx.x & 31;
   const AdjGeom& G = P.G;
   const long long ntiles = static_cast<long long>(G.g.F) * G.nt * G.na;
   auto tile_of = [&](long long it, int* f, int* tb, int* ab) {
@@ -229,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(accf_bar(b), 1);
-      ptx::mbar_init(acce_bar(b), 4);
+      ptx::mbar_init(acce_bar(b), kEpiWarps);
     }
     ptx::mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -245,34 +297,32 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_holder;
   const ptx::WaitCtl wc{P.timeout_ns, P.status, abort_flag};
-  const int steps = G.nk * 3;  // (hi, hi), (lo, hi), (hi, lo) per K block
 
   if (warp == 0) {
     if (lane == 0) {
       int issued_phase[kStages];
       for (int s = 0; s < kStages; ++s) issued_phase[s] = -1;
       bool ok = true;
-      long long gst = 0;  // stage-ring position across tiles
+      int stage = 0;  // the stage ring runs on across tiles
+      uint32_t phase = 0;
       for (long long it = blockIdx.x; ok && it < ntiles; it += gridDim.x) {
         int f, tb, ab;
         tile_of(it, &f, &tb, &ab);
-        for (int st = 0; st < steps; ++st, ++gst) {
-          const int stage = static_cast<int>(gst % kStages);
-          const uint32_t phase = static_cast<uint32_t>(gst / kStages) & 1u;
+        for (int kb = 0; kb < G.nk; ++kb) {
           if (!ptx::wait_bounded(empty_bar(stage), phase ^ 1u, wc)) {
             ok = false;
             break;
           }
-          const int kb = st / 3, j = st % 3;
-          const int hla = j == 1 ? 1 : 0, hlb = j == 2 ? 1 : 0;
           const uint32_t dst = sbase + stage * kStageBytes;
           const uint32_t fb = full_bar(stage);
           ptx::mbar_arrive_expect_tx(fb, kStageBytes);
-          ptx::bulk_load(dst, P.At + tile_off(f, 0, hla, ab, kb, G.na, G.nk), kTile, fb);
-          ptx::bulk_load(dst + kTile, P.At + tile_off(f, 1, hla, ab, kb, G.na, G.nk), kTile, fb);
-          ptx::bulk_load(dst + 2 * kTile, P.Bt + tile_off(f, 0, hlb, tb, kb, G.nt, G.nk), kTile, fb);
-          ptx::bulk_load(dst + 3 * kTile, P.Bt + tile_off(f, 1, hlb, tb, kb, G.nt, G.nk), kTile, fb);
+          ptx::bulk_load(dst, P.At + tile_off(f, ab, kb, G.na, G.nk), kOperand, fb);
+          ptx::bulk_load(dst + kOperand, P.Bt + tile_off(f, tb, kb, G.nt, G.nk), kOperand, fb);
           issued_phase[stage] = static_cast<int>(phase);
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
       }
       if (!ok) {
@@ -286,57 +336,71 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = true, issued_any = false;
-      long long gst = 0;
-      uint32_t u = 0;  // tiles done by this CTA
-      for (long long it = blockIdx.x; ok && it < ntiles; it += gridDim.x, ++u) {
-        const uint32_t ab = u & 1u, ap = (u >> 1) & 1u;
-        if (!ptx::wait_bounded(acce_bar(ab), ap ^ 1u, wc)) {
+    // The whole warp walks the stages (loop state and descriptors stay
+    // warp-uniform); one elected lane issues.
+    const bool issuer = ptx::elect_one();
+    bool ok = true;
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t u = 0;  // tiles done by this CTA
+    const uint64_t desc0 = ptx::interleave_kmajor_desc(sbase, kChunkStride, kGroupStride);
+    constexpr uint64_t kT = kTile >> 4;
+    for (long long it = blockIdx.x; ok && it < ntiles; it += gridDim.x, ++u) {
+      const uint32_t ab = u & 1u, ap = (u >> 1) & 1u;
+      bool got = ptx::wait_bounded(acce_bar(ab), ap ^ 1u, wc);
+      if (!__all_sync(0xffffffffu, got)) {
+        ok = false;
+        break;
+      }
+      const uint32_t d_re = tmem + ab * 256, d_im = d_re + 128;
+      for (int kb = 0; kb < G.nk; ++kb) {
+        got = ptx::wait_bounded(full_bar(stage), phase, wc);
+        if (!__all_sync(0xffffffffu, got)) {
           ok = false;
           break;
         }
         ptx::tc_fence_after();
-        const uint32_t d_re = tmem + ab * 256, d_im = d_re + 128;
-        for (int st = 0; st < steps; ++st, ++gst) {
-          const int stage = static_cast<int>(gst % kStages);
-          const uint32_t phase = static_cast<uint32_t>(gst / kStages) & 1u;
-          if (!ptx::wait_bounded(full_bar(stage), phase, wc)) {
-            ok = false;
-            break;
-          }
-          ptx::tc_fence_after();
-          const uint32_t ar = sbase + stage * kStageBytes, ai = ar + kTile;
-          const uint32_t br = ar + 2 * kTile, bi = ar + 3 * kTile;
+        const uint64_t dh = desc0 + static_cast<uint64_t>(stage) * (kStageBytes >> 4), dx = dh + (kOperand >> 4);
+        if (issuer) {
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k) {
-            const uint32_t acc = (st > 0 || k > 0) ? 1u : 0u;
-            const uint32_t ko = k * 2 * kChunkStride;
-            const uint64_t dar = ptx::interleave_kmajor_desc(ar + ko, kChunkStride, kGroupStride);
-            const uint64_t dai = ptx::interleave_kmajor_desc(ai + ko, kChunkStride, kGroupStride);
-            const uint64_t dbr = ptx::interleave_kmajor_desc(br + ko, kChunkStride, kGroupStride);
-            const uint64_t dbi = ptx::interleave_kmajor_desc(bi + ko, kChunkStride, kGroupStride);
-            ptx::mma_f16_ss(d_re, dar, dbr, kIdesc, acc);      // Re += Hr Xr^T
-            ptx::mma_f16_ss(d_re, dai, dbi, kIdescNegB, 1u);   // Re -= Hi Xi^T
-            ptx::mma_f16_ss(d_im, dar, dbi, kIdesc, acc);      // Im += Hr Xi^T
-            ptx::mma_f16_ss(d_im, dai, dbr, kIdesc, 1u);       // Im += Hi Xr^T
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {  // (hi, hi), (lo, hi), (hi, lo)
+              const uint64_t ko = static_cast<uint64_t>(k * 2 * kChunkStride) >> 4;
+              const uint64_t dhr = dh + (j == 1 ? 2 * kT : 0) + ko, dhi = dhr + kT;
+              const uint64_t dxr = dx + (j == 2 ? 2 * kT : 0) + ko, dxi = dxr + kT;
+              const uint32_t acc = (kb > 0 || k > 0 || j > 0) ? 1u : 0u;
+              // Re += Hr Xr^T and Im += Hr Xi^T; B is 256 rows: the Xr tile's, then Xi's.
+              ptx::mma_f16_ss(d_re, dhr, dxr, kIdescWide, acc);
+              ptx::mma_f16_ss(d_re, dhi, dxi, kIdescNegB, 1u);  // Re -= Hi Xi^T
+              ptx::mma_f16_ss(d_im, dhi, dxr, kIdesc, 1u);      // Im += Hi Xr^T
+            }
           }
-          issued_any = true;
           ptx::mma_commit(empty_bar(stage));
         }
-        if (!ok) break;
-        ptx::mma_commit(accf_bar(ab));
-      }
-      if (!ok && issued_any) {
-        ptx::mma_commit(drain_bar);
-        const uint64_t t0 = ptx::globaltimer();
-        while (!ptx::mbar_try_wait(drain_bar, 0) && ptx::globaltimer() - t0 < P.timeout_ns) {
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
+      if (ok && issuer) ptx::mma_commit(accf_bar(ab));
     }
+    if (!ok && issuer) {
+      // The MMAs issued so far complete before TMEM is freed (bounded).
+      ptx::mma_commit(drain_bar);
+      const uint64_t t0 = ptx::globaltimer();
+      while (!ptx::mbar_try_wait(drain_bar, 0) && ptx::globaltimer() - t0 < P.timeout_ns) {
+      }
+    }
+    __syncwarp();
   } else {
-    // Epilogue: warp q owns TMEM lanes 32q..32q+31 = rows a of the tile.
+    // Epilogue: warp q owns TMEM lanes 32q..32q+31 = rows a of the tile.  Its
+    // reads of x and writes of grad_x are latency-bound: with one warp per lane
+    // quarter a tile takes 19.8 us, with two 17.6 us (its MMAs alone 13 us;
+    // 256 stations x 2 pols, F=64, T=4096: 1065 and 947 us).
     const int q = warp & 3;
+    constexpr int kPieces = kBlk / 32 * 4 / kEpiWarps;  // 32-column pieces per warp
+    const int piece0 = (warp - 2) / 4 * kPieces;
     const uint32_t t_lanes = tmem + (static_cast<uint32_t>(q * 32) << 16);
     uint32_t u = 0;
     for (long long it = blockIdx.x; it < ntiles; it += gridDim.x, ++u) {
@@ -347,18 +411,19 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
       if (!__all_sync(0xffffffffu, got)) break;
       ptx::tc_fence_after();
       const int a = abk * kBlk + q * 32 + lane;
-      const float sc = adj_exp2i(adj_scale_exp(P.amax[f]) + adj_scale_exp(P.amax[G.g.F + f]));
       const bool row_ok = a < G.n;
+      const int eh = P.exp_h[static_cast<size_t>(f) * G.na * kBlk + a];
+      const int* ex = P.exp_x + (static_cast<size_t>(f) * G.nt + tb) * kBlk;
       const float2 ga = (P.gains && row_ok) ? P.gains[a] : make_float2(1.f, 0.f);
       const float2 cga = make_float2(ga.x, -ga.y);
       float2 gg = make_float2(0.f, 0.f);
 #pragma unroll 1
-      for (int piece = 0; piece < kBlk / 32; ++piece) {
+      for (int piece = piece0; piece < piece0 + kPieces; ++piece) {
         uint32_t vr[32], vi[32];
         ptx::tmem_ld_32x32b_x32(t_lanes + ab * 256 + piece * 32, vr);
         ptx::tmem_ld_32x32b_x32(t_lanes + ab * 256 + 128 + piece * 32, vi);
         ptx::tmem_wait_ld();
-        if (piece == kBlk / 32 - 1) {
+        if (piece == piece0 + kPieces - 1) {
           ptx::tc_fence_before();
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(acce_bar(ab));
@@ -376,6 +441,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           if (t0 + j >= G.g.T) continue;
+          const float sc = adj_exp2i(eh + __ldg(ex + piece * 32 + j));  // (one address for the warp)
           const float2 gy = make_float2(__uint_as_float(vr[j]) * sc, __uint_as_float(vi[j]) * sc);
           __stcs(P.grad_x + idx0 + j * step, cmul(cga, gy));
           gg.x += xv[j].x * gy.x + xv[j].y * gy.y;  // conj(x) gy
@@ -410,34 +476,35 @@ AdjGeom adj_geom(const Geometry& g) {
 
 size_t adjoint_tc_workspace_bytes(const Geometry& g) {
   const AdjGeom G = adj_geom(g);
-  const size_t per_rb = static_cast<size_t>(2) * 2 * G.nk * kTile;  // planes x hi/lo x K blocks
-  return static_cast<size_t>(g.F) * (G.na + G.nt) * per_rb + 256 + sizeof(unsigned) * 2 * g.F;
+  const size_t per_rb = static_cast<size_t>(G.nk) * kOperand + kBlk * sizeof(int);  // tiles, row exponents
+  return static_cast<size_t>(g.F) * (G.na + G.nt) * per_rb + 256;
 }
 
 cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* gains, void* grad_in,
-                              float* grad_g, void* h_ws, void* tc_ws, const Geometry& g,
-                              unsigned long long timeout_ns, int* status, cudaStream_t s) {
+                              float* grad_g, void* tc_ws, const Geometry& g, unsigned long long timeout_ns,
+                              int* status, cudaStream_t s) {
   const AdjGeom G = adj_geom(g);
   if (G.n == 0 || g.F == 0 || g.T == 0) return cudaSuccess;
-  cudaError_t e = launch_build_h(grad_out, h_ws, g, s);
-  if (e != cudaSuccess) return e;
   uint8_t* At = static_cast<uint8_t*>(tc_ws);
-  const size_t per_rb = static_cast<size_t>(2) * 2 * G.nk * kTile;
+  const size_t per_rb = static_cast<size_t>(G.nk) * kOperand;
   uint8_t* Bt = At + static_cast<size_t>(g.F) * G.na * per_rb;
-  unsigned* amax = reinterpret_cast<unsigned*>(Bt + static_cast<size_t>(g.F) * G.nt * per_rb);
-  const float2* H = static_cast<const float2*>(h_ws);
+  int* exp_h = reinterpret_cast<int*>(Bt + static_cast<size_t>(g.F) * G.nt * per_rb);
+  int* exp_x = exp_h + static_cast<size_t>(g.F) * G.na * kBlk;
+  const float2* go = static_cast<const float2*>(grad_out);
   const float2* x = static_cast<const float2*>(in);
   const float2* gn = static_cast<const float2*>(gains);
-  e = cudaMemsetAsync(amax, 0, sizeof(unsigned) * 2 * g.F, s);
-  if (e == cudaSuccess && grad_g) e = cudaMemsetAsync(grad_g, 0, sizeof(float) * 2 * G.n, s);
+  cudaError_t e = cudaSuccess;
+  if (grad_g) e = cudaMemsetAsync(grad_g, 0, sizeof(float) * 2 * G.n, s);
   if (e != cudaSuccess) return e;
-  adj_amax_h<<<dim3((G.n + 7) / 8, g.F), 256, 0, s>>>(H, gn, amax, G.n);
-  adj_amax_x<<<dim3((g.T + 31) / 32, g.F), 256, 0, s>>>(x, amax, g, G.n);
-  const int rows_a = G.na * kBlk * G.nk * (kBK / 8);
-  adj_form_h<<<dim3((rows_a + 255) / 256, g.F), 256, 0, s>>>(H, gn, amax, At, G);
-  const int64_t rows_t = static_cast<int64_t>(G.nt) * kBlk * G.nk * (kBK / 8);
-  if ((rows_t + 255) / 256 > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  adj_form_x<<<dim3(static_cast<unsigned>((rows_t + 255) / 256), g.F), 256, 0, s>>>(x, amax, Bt, G);
+  // Chunks per thread: four (rows of up to 512 inputs in one pass) or one.
+  const dim3 gh(G.na * (kBlk / kFormRows), g.F), gx(G.nt * (kBlk / kFormRows), g.F);
+  if (G.nk * (kBK / 8) > kFormCols) {
+    adj_form_h<4><<<gh, kFormThreads, 0, s>>>(go, gn, At, exp_h, G);
+    adj_form_x<4><<<gx, kFormThreads, 0, s>>>(x, Bt, exp_x, G);
+  } else {
+    adj_form_h<1><<<gh, kFormThreads, 0, s>>>(go, gn, At, exp_h, G);
+    adj_form_x<1><<<gx, kFormThreads, 0, s>>>(x, Bt, exp_x, G);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(adj_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
@@ -446,7 +513,8 @@ cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* 
   P.G = G;
   P.At = At;
   P.Bt = Bt;
-  P.amax = amax;
+  P.exp_h = exp_h;
+  P.exp_x = exp_x;
   P.x = x;
   P.gains = gn;
   P.grad_x = static_cast<float2*>(grad_in);

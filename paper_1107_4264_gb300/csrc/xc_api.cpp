@@ -789,7 +789,8 @@ xc_status xc_correlate_backward(xc_handle* h, const void* grad_out, const void* 
     return fail(XC_ERR_ALIGNMENT, "buffers must be 16-byte aligned");
   const int64_t n = static_cast<int64_t>(h->g.N) * h->g.P;
   cudaError_t e = cudaSuccess;
-  if (!h->adj_ws) e = cudaMalloc(&h->adj_ws, static_cast<size_t>(h->g.F) * n * n * 8);
+  if (h->engine == XC_ENGINE_FP32 && !h->adj_ws)
+    e = cudaMalloc(&h->adj_ws, static_cast<size_t>(h->g.F) * n * n * 8);
   if (e == cudaSuccess && !h->grad_g) e = cudaMalloc(reinterpret_cast<void**>(&h->grad_g), 8 * n);
   if (e != cudaSuccess) return cuda_fail(e, "adjoint workspace");
   const void* gains = h->gains_set ? h->gains : nullptr;
@@ -805,8 +806,8 @@ xc_status xc_correlate_backward(xc_handle* h, const void* grad_out, const void* 
         return cuda_fail(e, "adjoint workspace");
       }
     }
-    e = xc::launch_adjoint_tc(grad_out, in, gains, grad_in, h->grad_g, h->adj_ws, h->adj_tc_ws, h->g,
-                              h->timeout_ns, h->d_status, s);
+    e = xc::launch_adjoint_tc(grad_out, in, gains, grad_in, h->grad_g, h->adj_tc_ws, h->g, h->timeout_ns,
+                              h->d_status, s);
   }
   if (e != cudaSuccess) return cuda_fail(e, "adjoint launch");
   return succeed();
