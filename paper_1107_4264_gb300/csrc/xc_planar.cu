@@ -40,33 +40,73 @@ const void* select_kernel(int in_dtype, int fmt, bool multi) {
 
 // Scale pre-pass for float input: amax[f][a] = max over t of the largest
 // component of g_a x_a(t) (fp32 bits; non-negative floats order as
-// unsigned integers).  A thread per (input, channel, 128-sample range);
-// a warp reads 32 consecutive inputs of one sample row.
-template <int DT>
-__global__ void __launch_bounds__(128) input_amax_kernel(const void* __restrict__ in,
-                                                         const float2* __restrict__ gains,
-                                                         unsigned* __restrict__ amax, Geometry g,
-                                                         int n, int gain_n) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
+// unsigned integers).  Bound by the one read of the input: a thread keeps
+// eight 16-byte loads in flight (VEC = 2 complex fp32 or 4 complex fp16
+// inputs; VEC = 1 when a row is not a multiple of 16 bytes).  A block takes
+// kAmaxIter x `rows` samples of one channel, `rows` of them side by side when
+// a row has fewer than 128 vectors.  On 512 stations x 2 pols, F=60, T=2048,
+// fp32 (1.0 GB): 138 us (291 us with one 8-byte load per input and sample).
+constexpr int kAmaxThreads = 128, kAmaxIter = 64;
+template <int DT, int VEC>
+__global__ void __launch_bounds__(kAmaxThreads) input_amax_kernel(const void* __restrict__ in,
+                                                                  const float2* __restrict__ gains,
+                                                                  unsigned* __restrict__ amax, Geometry g,
+                                                                  int n, int gain_n, int rows) {
+  const int nv = n / VEC;  // vectors of a row
+  const int r = rows > 1 ? threadIdx.x / nv : 0;
+  const int v = rows > 1 ? threadIdx.x - r * nv : blockIdx.x * kAmaxThreads + threadIdx.x;
   const int f = blockIdx.y;
-  if (a >= n) return;
-  const int t0 = blockIdx.z * 128;
-  const int t1 = min(g.T, t0 + 128);
-  const float2 ga = gains ? gains[a % gain_n] : make_float2(1.f, 0.f);
-  float m = 0.f;
-#pragma unroll 8
-  for (int t = t0; t < t1; ++t) {
-    const int64_t idx = (static_cast<int64_t>(t) * g.F + f) * n + a;
-    float2 v;
-    if constexpr (DT == 1) {
-      v = __half22float2(static_cast<const __half2*>(in)[idx]);
-    } else {
-      v = static_cast<const float2*>(in)[idx];
-    }
-    if (gains) v = make_float2(ga.x * v.x - ga.y * v.y, ga.x * v.y + ga.y * v.x);
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+  if (v >= nv || r >= rows) return;
+  const int a = v * VEC;
+  const int t0 = blockIdx.z * kAmaxIter * rows + r;
+  const int t1 = min(g.T, static_cast<int>(blockIdx.z + 1) * kAmaxIter * rows);
+  float2 ga[VEC];
+  float m[VEC];
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) {
+    ga[i] = gains ? gains[(a + i) % gain_n] : make_float2(1.f, 0.f);
+    m[i] = 0.f;
   }
-  atomicMax(amax + static_cast<int64_t>(f) * n + a, __float_as_uint(m));
+  constexpr int kBytes = (DT == 1 ? 4 : 8) * VEC;
+  using Raw = typename std::conditional<kBytes == 16, uint4, typename std::conditional<kBytes == 8, uint2, unsigned>::type>::type;
+  const Raw* p = reinterpret_cast<const Raw*>(in) + (static_cast<int64_t>(t0) * g.F + f) * nv + v;
+  const int64_t step = static_cast<int64_t>(rows) * g.F * nv;
+  auto use = [&](const Raw& raw) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+      float2 x;
+      if constexpr (DT == 1) {
+        x = __half22float2(reinterpret_cast<const __half2*>(&raw)[i]);
+      } else {
+        x = reinterpret_cast<const float2*>(&raw)[i];
+      }
+      if (gains) x = make_float2(ga[i].x * x.x - ga[i].y * x.y, ga[i].x * x.y + ga[i].y * x.x);
+      m[i] = fmaxf(m[i], fmaxf(fabsf(x.x), fabsf(x.y)));
+    }
+  };
+  int t = t0;
+  for (; t + 7 * rows < t1; t += 8 * rows, p += 8 * step) {
+    Raw w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = __ldg(p + i * step);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) use(w[i]);
+  }
+  for (; t < t1; t += rows, p += step) use(__ldg(p));
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) atomicMax(amax + static_cast<int64_t>(f) * n + a + i, __float_as_uint(m[i]));
+}
+
+template <int DT, int VEC>
+cudaError_t launch_amax(const XeLaunch& L, int n, cudaStream_t s) {
+  const int nv = n / VEC;
+  const int rows = std::max(1, kAmaxThreads / nv);
+  const dim3 grid(rows > 1 ? 1 : (nv + kAmaxThreads - 1) / kAmaxThreads, L.g.F,
+                  (L.g.T + kAmaxIter * rows - 1) / (kAmaxIter * rows));
+  if (grid.z > 65535u) return cudaErrorInvalidConfiguration;
+  input_amax_kernel<DT, VEC><<<grid, kAmaxThreads, 0, s>>>(L.in, static_cast<const float2*>(L.gains), L.in_amax,
+                                                          L.g, n, n / std::max(1, L.pack), rows);
+  return cudaGetLastError();
 }
 
 int fmt_kt(int fmt) { return fmt == kFmtHiLo ? 2 : 1; }
@@ -306,15 +346,12 @@ cudaError_t planar_setup(const XeLaunch* subs, int nsub, cudaStream_t s) {
     if (L.in_dtype != 0 && L.in_amax) {
       e = cudaMemsetAsync(L.in_amax, 0, sizeof(unsigned) * L.g.F * static_cast<size_t>(n), s);
       if (e != cudaSuccess) return e;
-      const dim3 ag((n + 127) / 128, L.g.F, (L.g.T + 127) / 128);
-      if (ag.z > 65535u) return cudaErrorInvalidConfiguration;
-      const float2* gains = static_cast<const float2*>(L.gains);
-      const int gain_n = n / std::max(1, L.pack);
+      // (The input is 16-byte aligned, so its rows are when they are a
+      // multiple of 16 bytes.)
       if (L.in_dtype == 1)
-        input_amax_kernel<1><<<ag, 128, 0, s>>>(L.in, gains, L.in_amax, L.g, n, gain_n);
+        e = n % 4 == 0 ? launch_amax<1, 4>(L, n, s) : launch_amax<1, 1>(L, n, s);
       else
-        input_amax_kernel<2><<<ag, 128, 0, s>>>(L.in, gains, L.in_amax, L.g, n, gain_n);
-      e = cudaGetLastError();
+        e = n % 2 == 0 ? launch_amax<2, 2>(L, n, s) : launch_amax<2, 1>(L, n, s);
       if (e != cudaSuccess) return e;
     }
   }
