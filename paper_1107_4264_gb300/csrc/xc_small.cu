@@ -251,7 +251,8 @@ __global__ void __launch_bounds__(Cfg<W, F8>::kThreads, 1)
   const uint32_t bars = sbase + C::kBarOff;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sgen + C::kMiscOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + C::kMiscOff + 4);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known uniform)
+  const int lane = threadIdx.x & 31;
   const int items = p.ngroups * p.nseg;
 
   if (threadIdx.x == 0) {
@@ -319,59 +320,59 @@ __global__ void __launch_bounds__(Cfg<W, F8>::kThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_f16_f32(kRows, kRows);
-      int so = 0, ab = 0;
-      uint32_t oph = 0;
-      uint32_t usep = 0;  // bit ab: parity of buffer ab's use count
-      bool ok = true;
-      for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
-        const Item x = item_of(p, it);
-        for (int c0 = x.t0; ok && c0 < x.t1; c0 += kChunk) {
-          const int c1 = min(x.t1, c0 + kChunk);
-          // The epilogue has read this buffer's previous chunk.  (W = 256:
-          // each block's drain is awaited just before the chunk's first
-          // MMAs into that block, below.)
-          const uint32_t drained = ((usep >> ab) & 1u) ^ 1u;
-          if (C::kTiles == 1 && !ptx::wait_bounded(C::acce(bars, ab), drained, wc)) {
+    // The whole warp walks the stages, so that loop state and descriptors stay
+    // warp-uniform; one elected lane issues.  A stage is 4 MMAs of 64 cycles,
+    // and what one divergent thread spent between stages set the kernel's pace
+    // (T = 1000: N = 32, F = 8192 297 -> 258 us; N = 64, F = 2048 197 -> 165).
+    // Now shared memory does: of 584 cycles per stage at N = 32 its copies,
+    // conversion and operand reads fill about 512.
+    const bool issuer = ptx::elect_one();
+    constexpr uint32_t idesc = ptx::idesc_f16_f32(kRows, kRows);
+    const uint64_t desc0 = ptx::interleave_kmajor_desc(sbase + C::kOpOff, kCore, kSbo);
+    int so = 0, ab = 0;
+    uint32_t oph = 0;
+    uint32_t usep = 0;  // bit ab: parity of buffer ab's use count
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
+      const Item x = item_of(p, it);
+      for (int c0 = x.t0; ok && c0 < x.t1; c0 += kChunk) {
+        const int c1 = min(x.t1, c0 + kChunk);
+        // The epilogue has read this buffer's previous chunk.  (W = 256:
+        // each block's drain is awaited just before the chunk's first
+        // MMAs into that block, below.)
+        const uint32_t drained = ((usep >> ab) & 1u) ^ 1u;
+        if (C::kTiles == 1 && !warp_wait(C::acce(bars, ab), drained, wc)) {
+          ok = false;
+          break;
+        }
+        for (int t = c0; t < c1; t += kBK) {
+          if (!warp_wait(C::op_full(bars, so), oph, wc)) {
             ok = false;
             break;
           }
           ptx::tc_fence_after();
-          for (int t = c0; t < c1; t += kBK) {
-            if (!ptx::wait_bounded(C::op_full(bars, so), oph, wc)) {
-              ok = false;
-              break;
-            }
-            ptx::tc_fence_after();
-            const uint32_t stage = sbase + C::kOpOff + so * C::kOpBytes;
-            // Row ta of the lower tile triangle: A = tile ta, B = tiles
-            // 0 .. ta (contiguous, so one descriptor covers them: N = 128 (ta
-            // + 1)), D = blocks (ta, 0) .. (ta, ta), which sit side by side in
-            // TMEM; the row's K steps (chunks 2kk, 2kk + 1) in a row.
-            // With one tile, A = B = the tile: D holds every channel's block
-            // on its diagonal and the epilogue reads only those.
+          const uint64_t stage = desc0 + static_cast<uint64_t>(so) * (C::kOpBytes >> 4);
+          // Row ta of the lower tile triangle: A = tile ta, B = tiles
+          // 0 .. ta (contiguous, so one descriptor covers them: N = 128 (ta
+          // + 1)), D = blocks (ta, 0) .. (ta, ta), which sit side by side in
+          // TMEM; the row's K steps (chunks 2kk, 2kk + 1) in a row.
+          // With one tile, A = B = the tile: D holds every channel's block
+          // on its diagonal and the epilogue reads only those.
 #pragma unroll
-            for (int ta = 0; ta < C::kTiles; ++ta) {
-              const int blk0 = ta * (ta + 1) / 2;
-              if (C::kTiles > 1 && t == c0) {
-                for (int b = blk0; b <= blk0 + ta; ++b) {
-                  if (!ptx::wait_bounded(C::acce(bars, b), drained, wc)) {
-                    ok = false;
-                    break;
-                  }
-                }
-                if (!ok) break;
-                ptx::tc_fence_after();
-              }
-              const uint32_t idesc_row = ta == 0 ? idesc : ptx::idesc_f16_f32(kRows, kRows * (ta + 1));
+          for (int ta = 0; ta < C::kTiles; ++ta) {
+            const int blk0 = ta * (ta + 1) / 2;
+            if (C::kTiles > 1 && t == c0) {
+              for (int b = blk0; ok && b <= blk0 + ta; ++b) ok = warp_wait(C::acce(bars, b), drained, wc);
+              if (!ok) break;
+              ptx::tc_fence_after();
+            }
+            const uint32_t idesc_row = ta == 0 ? idesc : ptx::idesc_f16_f32(kRows, kRows * (ta + 1));
+            const uint32_t dcol = tmem + static_cast<uint32_t>(ab * C::kAccCols + blk0 * kRows);
+            if (issuer) {
 #pragma unroll
               for (int kk = 0; kk < kBK / C::kKStep; ++kk) {
                 // K step kk: two 16-byte chunks of every row.
-                const uint64_t da =
-                    ptx::interleave_kmajor_desc(stage + ta * kTileBytes + kk * 2 * kCore, kCore, kSbo);
-                const uint64_t db = ptx::interleave_kmajor_desc(stage + kk * 2 * kCore, kCore, kSbo);
-                const uint32_t dcol = tmem + static_cast<uint32_t>(ab * C::kAccCols + blk0 * kRows);
+                const uint64_t db = stage + ((kk * 2 * kCore) >> 4), da = db + ((ta * kTileBytes) >> 4);
                 // (kind::f8f6f4 with e4m3 A and B takes the same descriptor type fields as f16.)
                 if constexpr (F8)
                   ptx::mma_f8_ss(dcol, da, db, idesc_row, (t > c0 || kk > 0) ? 1u : 0u);
@@ -379,25 +380,28 @@ __global__ void __launch_bounds__(Cfg<W, F8>::kThreads, 1)
                   ptx::mma_f16_ss(dcol, da, db, idesc_row, (t > c0 || kk > 0) ? 1u : 0u);
               }
             }
-            if (!ok) break;
-            ptx::mma_commit(C::op_empty(bars, so));  // the tile may be refilled once read
-            if (++so == C::kOpStages) {
-              so = 0;
-              oph ^= 1u;
-            }
           }
           if (!ok) break;
-          ptx::mma_commit(C::accf(bars, ab));
-          usep ^= 1u << ab;
-          ab = (ab + 1) % C::kBufs;
+          if (issuer) ptx::mma_commit(C::op_empty(bars, so));  // the tile may be refilled once read
+          if (++so == C::kOpStages) {
+            so = 0;
+            oph ^= 1u;
+          }
         }
+        if (!ok) break;
+        if (issuer) ptx::mma_commit(C::accf(bars, ab));
+        usep ^= 1u << ab;
+        ab = (ab + 1) % C::kBufs;
       }
-      // Every MMA issued completes before TMEM is freed and the CTA exits.
+    }
+    // Every MMA issued completes before TMEM is freed and the CTA exits.
+    if (issuer) {
       ptx::mma_commit(C::drain(bars));
       const uint64_t t0 = ptx::globaltimer();
       while (!ptx::mbar_try_wait(C::drain(bars), 0u) && ptx::globaltimer() - t0 < p.timeout_ns) {
       }
     }
+    __syncwarp();
   } else if (warp < kConvWarp0 || warp >= kConvWarp0 + C::kConvWarps) {
     // --------------------------------------------------------- epilogue
     // Warps 2 .. 5 (group 0) and, at W = 256, the warps after the
