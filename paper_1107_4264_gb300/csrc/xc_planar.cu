@@ -305,11 +305,15 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     const long long resident = static_cast<long long>(per_sm) * subs[0].grid;
     k->grid = static_cast<int>(std::min<long long>({items, static_cast<long long>(subs[0].grid), resident}));
   }
-  // A converter warp's step from one run to its next, for its incremental
-  // unit numbers.
-  const long long step = static_cast<long long>(k->grid) * conv * kUnitRun;
+  // Runs of two units once every converter warp has eight or more to do, of one
+  // below (2 stations x 1 pol, F=11, T=102: one CTA, 24 -> 17 us).  Then a
+  // warp's step from one run to its next, for its incremental unit numbers.
+  const long long workers = static_cast<long long>(k->grid) * conv;
+  const int run = b->unit_base[nsub] >= 8 * workers ? kUnitRun : 1;
+  const long long step = workers * run;
   for (int i = 0; i < nsub; ++i) {
     Params& p = b->sub[i];
+    p.run = run;
     p.step_seg = static_cast<int>(step / p.seg_units);
     p.step_rem = static_cast<int>(step % p.seg_units);
     p.step_gen = p.step_seg / p.ring_slots;

@@ -240,13 +240,14 @@ struct Params {
   // wave_last, from segment number last_base on): see seg_first.
   int wave, wave_segs, wave_full, wave_last, last_base;
   unsigned mag_kb, mag_wave, mag_wsegs, mag_last, mag_slots;  // fast_div magics
-  // From one of a converter warp's runs to its next (kUnitRun * converter
-  // warps units on): step_seg segments and step_rem units, and step_seg as
+  int run;  // units per run (the same in all subarrays)
+  // From one of a converter warp's runs to its next (run * converter warps
+  // units on): step_seg segments and step_rem units, and step_seg as
   // ring generations and slots.
   int step_seg, step_rem, step_gen, step_slot;
   // From one of a CTA's (cluster's) items to its next: channels and items.
   int it_step_f, it_step_i;
-  int tma_in;          // 8-bit input staged by TMA (else direct loads)
+  int tma_in;          // input staged by TMA (rows are a multiple of 16 bytes)
   unsigned long long timeout_ns;
   int* status;
   int test_no_publish;  // test hook: converted units are never published
@@ -528,11 +529,11 @@ struct Unit {
   int w, hb, k;     // unit in the segment
 };
 
-// Converter warps take their units in runs of kUnitRun consecutive units
+// Converter warps take their units in runs of p.run (1 or 2) consecutive units
 // (always of one segment, whose unit count is even): one slot claim and one
 // publish (fence + release of the whole count) per run instead of per unit.
 // Warp gw of nw takes runs gw, gw + nw, gw + 2 nw, ... of the global unit
-// list.
+// list.  Runs of one unit where there are too few units to go round.
 constexpr int kUnitRun = 2;
 
 // Unit u by division (a warp's first one, and the first in another subarray).
@@ -552,19 +553,20 @@ __device__ __forceinline__ void unit_locate(const Batch& bt, Unit& x) {
 // they were about a quarter of a converter warp's time per unit.
 template <bool MULTI>
 __device__ __forceinline__ bool unit_step(const Batch& bt, Unit& x, long long nw, long long total) {
-  if ((x.u & (kUnitRun - 1)) != kUnitRun - 1) {
+  const int run = bt.sub[0].run;
+  if ((x.u & (run - 1)) != run - 1) {
     ++x.u;
     ++x.w;
     return true;
   }
-  x.u += 1 + (nw - 1) * kUnitRun;
+  x.u += 1 + (nw - 1) * run;
   if (x.u >= total) return false;
   if (MULTI && x.u >= bt.unit_base[x.sb + 1]) {
     unit_locate<MULTI>(bt, x);
     return true;
   }
   const Params& p = bt.sub[x.sb];
-  x.w += p.step_rem - (kUnitRun - 1);
+  x.w += p.step_rem - (run - 1);
   const int carry = x.w >= p.seg_units ? 1 : 0;
   x.w -= carry ? p.seg_units : 0;
   x.G += p.step_seg + carry;
@@ -593,7 +595,7 @@ __device__ __forceinline__ bool unit_decode(const Params& p, Unit& x) {
 template <bool MULTI>
 __device__ __forceinline__ bool unit_first(const Batch& bt, Unit& x, long long gw, long long nw,
                                            long long total) {
-  x.u = gw * kUnitRun;
+  x.u = gw * bt.sub[0].run;
   x.sb = 0;
   if (x.u >= total) return false;
   unit_locate<MULTI>(bt, x);
@@ -654,10 +656,7 @@ __device__ __forceinline__ void publish_unit(const Params& p, int slot, int lane
 template <int DT>
 __device__ __forceinline__ float2 load_cx(const Params& p, int c, int a, int t) {
   const int64_t idx = (static_cast<int64_t>(t) * p.g.F + c) * p.n + a;
-  if constexpr (DT == 0) {
-    const char2 v = static_cast<const char2*>(p.in)[idx];
-    return make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
-  } else if constexpr (DT == 1) {
+  if constexpr (DT == 1) {
     return __half22float2(static_cast<const __half2*>(p.in)[idx]);
   } else {
     return static_cast<const float2*>(p.in)[idx];
@@ -682,7 +681,7 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
   return (lo & 0xffffu) | (hi << 16);
 }
 
-// Direct-load converter (any input type and row count), independent warps:
+// Direct-load converter (float input of any row count), independent warps:
 // lane l loads the complex samples of inputs l and l + 32 of the half block,
 // 16 samples (32 loads) in flight at a time, applies the gains and the
 // input's power-of-two scale (float input) and writes 16-byte chunks: per
@@ -690,6 +689,7 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
 // L tile) or one e4m3 chunk (16 samples).
 template <int DT, int FMT, bool MULTI, int SHAPE>
 __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int* abort_flag) {
+  static_assert(DT != 0, "8-bit input has its own converters");
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, DT>();
   int claimed = -1, claimed_sb = -1;
@@ -708,23 +708,20 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
     uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
     const int a0 = x.hb * 64 + lane, a1 = a0 + 32;
     const int row0 = (x.hb & 1) * 64 + lane;
-    // y = g x 2^-e (float input; gains are not defined for 8-bit input).
+    // y = g x 2^-e.
     float2 g0 = make_float2(1.f, 0.f), g1 = make_float2(1.f, 0.f);
-    if (DT != 0) {
-      if (p.gains) {
-        g0 = a0 < p.n ? p.gains[a0 % p.gain_n] : make_float2(0.f, 0.f);
-        g1 = a1 < p.n ? p.gains[a1 % p.gain_n] : make_float2(0.f, 0.f);
-      }
-      if (p.in_amax) {
-        const unsigned* am = p.in_amax + static_cast<int64_t>(x.c) * p.n;
-        const float s0 = a0 < p.n ? exp2i(-scale_exp<FMT>(am[a0])) : 0.f;
-        const float s1 = a1 < p.n ? exp2i(-scale_exp<FMT>(am[a1])) : 0.f;
-        g0 = make_float2(g0.x * s0, g0.y * s0);  // exact: s is a power of two
-        g1 = make_float2(g1.x * s1, g1.y * s1);
-      }
+    if (p.gains) {
+      g0 = a0 < p.n ? p.gains[a0 % p.gain_n] : make_float2(0.f, 0.f);
+      g1 = a1 < p.n ? p.gains[a1 % p.gain_n] : make_float2(0.f, 0.f);
     }
-    const bool apply = DT != 0 && (p.gains || p.in_amax);
-    bool unit_over_16 = false;
+    if (p.in_amax) {
+      const unsigned* am = p.in_amax + static_cast<int64_t>(x.c) * p.n;
+      const float s0 = a0 < p.n ? exp2i(-scale_exp<FMT>(am[a0])) : 0.f;
+      const float s1 = a1 < p.n ? exp2i(-scale_exp<FMT>(am[a1])) : 0.f;
+      g0 = make_float2(g0.x * s0, g0.y * s0);  // exact: s is a power of two
+      g1 = make_float2(g1.x * s1, g1.y * s1);
+    }
+    const bool apply = p.gains || p.in_amax;
 #pragma unroll 1
     for (int g = 0; g < kUnitT / 16; ++g) {
       float2 v0[16], v1[16];
@@ -733,12 +730,6 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
         const int t = t0 + g * 16 + i;
         v0[i] = (a0 < p.n && t < p.g.T) ? load_cx<DT>(p, x.c, a0, t) : make_float2(0.f, 0.f);
         v1[i] = (a1 < p.n && t < p.g.T) ? load_cx<DT>(p, x.c, a1, t) : make_float2(0.f, 0.f);
-      }
-      if constexpr (DT == 0 && FMT == kFmtF8) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          unit_over_16 |= fmaxf(fmaxf(fabsf(v0[i].x), fabsf(v0[i].y)),
-                                fmaxf(fabsf(v1[i].x), fabsf(v1[i].y))) > 16.f;
       }
       if (apply) {
 #pragma unroll
@@ -804,9 +795,6 @@ __device__ void converter_direct(const Batch& bt, int cw, int lane, volatile int
         }
       }
     }
-    if (DT == 0 && lane == 0) atomicMax(p.amax + x.G, 128u);  // no scan: worst case
-    if (DT == 0 && FMT == kFmtF8 && __any_sync(0xffffffffu, unit_over_16) && lane == 0)
-      atomicOr(p.status, kStatusRange);  // e4m3 is exact only for |x| <= 16
     publish_unit(p, x.slot, lane, unit_weight(p, x));
     if (*abort_flag) return;
   }
@@ -900,7 +888,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
     if (more) issue(nx);
     // A finished run is published now: its stores have drained during this
     // unit's shared-memory reads.
-    if (pend && pend_run != x.u / kUnitRun) {
+    if (pend && pend_run != x.u / p.run) {
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
@@ -984,7 +972,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
-      pend_run = x.u / kUnitRun;
+      pend_run = x.u / p.run;
       pend_n = 0;
     }
     pend_n += unit_weight(p, x);
@@ -993,6 +981,207 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       drain_tma(bar, phase, tma_pending, wc.timeout_ns);
       return;
     }
+  }
+  if (pend) publish_unit(*pend, pend_slot, lane, pend_n);
+}
+
+// 8-bit converter for rows that TMA cannot stride (not a multiple of 16 bytes).
+// As converter_tma, but the words are loaded straight into registers: an even
+// number of inputs (EVEN) has its rows on 4 bytes, an odd one is read in
+// 16-bit halves that are joined when they are used.  As soon as 8 samples are
+// converted their registers take the loads kRing chunks on (64 samples, or
+// 32), which so have that long to arrive.  (On rows that TMA can stride this is
+// the slower one: 256 stations x 2 pols, F=1024, T=1000 1.16 against 1.03 ms.)
+// Measured against converting single components by way of floats, for any row:
+// 37 stations x 2 pols, F=2048, T=1000 1742 -> 451 us; 131 stations x 1 pol,
+// F=300, T=500 270 -> 175 us.
+// A warp publishes each run at the start of the run after it; a warp that would
+// have to wait for a slot publishes first (a consumer of the slot's previous
+// segment may need that run).
+template <int FMT, bool MULTI, int SHAPE, bool EVEN>
+__device__ void converter_words(const Batch& bt, int cw, int lane, volatile int* abort_flag) {
+  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
+  const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
+  const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
+  // The input streams through once: first in line for L2 replacement, so the
+  // operand ring it is converted into stays resident.  Ring tiles are read
+  // back by every block of the channel: keep them in L2.
+  const uint64_t pol_first = ptx::l2_policy_evict_first(), pol_last = ptx::l2_policy_evict_last();
+  // Where a unit's words come from: this lane's word of sample 0, the bytes
+  // from sample to sample, and the samples to load (0: no such input).
+  struct Src {
+    const uint8_t* ptr;
+    int64_t step;
+    int count, count_hi;  // of the word's first and second input
+  };
+  const uint32_t lane4 = static_cast<uint32_t>(lane) * 4u;
+  auto source = [&](const Unit& x) {
+    const Params& p = bt.sub[x.sb];
+    const int t0 = (x.seg * p.seg_kb + x.k) * kBK;
+    Src s;
+    s.step = static_cast<int64_t>(p.g.F) * p.g.R;
+    s.ptr = static_cast<const uint8_t*>(p.in) + t0 * s.step + static_cast<int64_t>(x.c) * p.g.R +
+            x.hb * kUnitRows;
+    const int ns = min(kBK, p.g.T - t0), row = x.hb * kUnitRows + static_cast<int>(lane4);
+    s.count = row < p.g.R ? ns : 0;
+    s.count_hi = row + 2 < p.g.R ? ns : 0;
+    return s;
+  };
+  // The registers: a ring of 8-sample chunks, one word per sample or two halves.
+  constexpr int kRing = EVEN ? 8 : 4, kPer = EVEN ? 8 : 16;
+  uint32_t w[kRing * kPer];
+  // Chunk cc of a unit into its registers (zero past the end).
+  auto load8 = [&](const Src& s, int cc) {
+    uint32_t* r = w + cc % kRing * kPer;
+    const uint8_t* q = s.ptr + 8 * cc * s.step + lane4;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if constexpr (EVEN) {
+        r[t] = ptx::ld_global_b32_if(q + t * s.step, pol_first, 8 * cc + t < s.count);
+      } else {
+        r[t] = ptx::ld_global_u16_if(q + t * s.step, pol_first, 8 * cc + t < s.count);
+        r[8 + t] = ptx::ld_global_u16_if(q + t * s.step + 2, pol_first, 8 * cc + t < s.count_hi);
+      }
+    }
+  };
+  // Chunk cc's words.
+  auto words8 = [&](int cc, uint32_t* W) {
+    const uint32_t* r = w + cc % kRing * kPer;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) W[t] = EVEN ? r[t] : (r[t] | r[8 + t] << 16);
+  };
+  int claimed = -1, claimed_sb = -1;
+  // Converted units of a run not yet published: their subarray, slot, run, count.
+  const Params* pend = nullptr;
+  int pend_slot = 0;
+  long long pend_run = -1;
+  unsigned pend_n = 0;
+  Unit x;
+  bool more = unit_first<MULTI>(bt, x, static_cast<long long>(blockIdx.x) * conv_warps<FMT, 0>() + cw, nw, total);
+  Src cs = {nullptr, 0, 0, 0};
+  if (more) {
+    cs = source(x);
+#pragma unroll
+    for (int cc = 0; cc < kRing; ++cc) load8(cs, cc);
+  }
+  while (more) {
+    const Params& p = bt.sub[x.sb];
+    if (x.G != claimed || x.sb != claimed_sb) {
+      if (pend && slot_busy(p, x, lane)) {
+        publish_unit(*pend, pend_slot, lane, pend_n);
+        pend = nullptr;
+      }
+      if (!claim_slot_warp(p, x, lane, abort_flag)) return;
+      claimed = x.G;
+      claimed_sb = x.sb;
+    }
+    Unit nx = x;
+    more = unit_next<MULTI>(bt, nx, nw, total);
+    Src ns = {nullptr, 0, 0, 0};
+    if (more) ns = source(nx);
+    // The chunk that takes chunk cc's registers: of this unit or the next.
+    auto reload = [&](int cc) {
+      if (cc + kRing < kBK / 8)
+        load8(cs, cc + kRing);
+      else
+        load8(ns, cc + kRing - kBK / 8);
+    };
+    const int ib = x.hb >> 1;
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
+    const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
+    // A finished run is published now: its last stores have had some time.
+    if (pend && pend_run != x.u / p.run) {
+      publish_unit(*pend, pend_slot, lane, pend_n);
+      pend = nullptr;
+    }
+    unsigned m = 0;  // max |x| over the unit (rows and samples past the end contribute 0)
+    if constexpr (FMT == kFmtF16) {
+      // max |x| from the converted (exact) fp16 values.
+      __half2 mx[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) mx[q] = __float2half2_rn(0.f);
+      // Rows 2l and 2l + 1 of one plane: bytes j and j + 2 of the words.
+      auto store8 = [&](uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq) {
+        uint32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
+          v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k += 2)
+          mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
+                                   __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
+        ptx::st_global_v8_hint(dst, v, pol_last);
+      };
+#pragma unroll
+      for (int cc = 0; cc < kBK / 8; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        uint32_t W[8];
+        words8(cc, W);
+        store8(tre + off, W, 0u, mx[0]);
+        store8(tim + off, W, 1u, mx[1]);
+        reload(cc);
+      }
+      const __half2 mm = __hmax2(mx[0], mx[1]);
+      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
+    } else {
+      // e4m3 operands: exact for |x| <= 16 (a larger value sets the range
+      // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
+      uint32_t mb = 0;  // per-byte |x| maximum
+      // Component j of four consecutive samples as four e4m3 bytes: the
+      // exact fp16 pair conversion of the fp16 path, then one fp16x2 ->
+      // e4m3x2 conversion per pair (exact for |x| <= 16).
+      auto cvt4 = [](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t j) {
+        const uint32_t h01 = pair_i8(w0, w1, j), h23 = pair_i8(w2, w3, j);
+        __half2_raw r01, r23;
+        r01.x = static_cast<unsigned short>(h01 & 0xffffu);
+        r01.y = static_cast<unsigned short>(h01 >> 16);
+        r23.x = static_cast<unsigned short>(h23 & 0xffffu);
+        r23.y = static_cast<unsigned short>(h23 >> 16);
+        const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
+        const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
+        return (e01 & 0xffffu) | (e23 << 16);
+      };
+#pragma unroll
+      for (int cc = 0; cc < kBK / 16; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        uint32_t W[16];
+        words8(2 * cc, W);
+        words8(2 * cc + 1, W + 8);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
+        uint32_t vr[8], vi[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          vr[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 0);
+          vi[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 1);
+          vr[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 2);
+          vi[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 3);
+        }
+        ptx::st_global_v8_hint(tre + off, vr, pol_last);
+        ptx::st_global_v8_hint(tim + off, vi, pol_last);
+        reload(2 * cc);
+        reload(2 * cc + 1);
+      }
+      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) {
+      atomicMax(p.amax + x.G, m);
+      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
+    }
+    if (!pend) {
+      pend = &p;
+      pend_slot = x.slot;
+      pend_run = x.u / p.run;
+      pend_n = 0;
+    }
+    pend_n += unit_weight(p, x);
+    x = nx;
+    cs = ns;
+    if (*abort_flag) return;
   }
   if (pend) publish_unit(*pend, pend_slot, lane, pend_n);
 }
@@ -1164,7 +1353,7 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
       } else if (more) {
         issue(nx, 0);
       }
-      if (j == 0 && pend && pend_run != x.u / kUnitRun) {
+      if (j == 0 && pend && pend_run != x.u / p.run) {
         publish_unit(*pend, pend_slot, lane, pend_n);
         pend = nullptr;
       }
@@ -1190,7 +1379,7 @@ __device__ void converter_tma_float(const Batch& bt, uint32_t buf, uint32_t bar,
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
-      pend_run = x.u / kUnitRun;
+      pend_run = x.u / p.run;
       pend_n = 0;
     }
     pend_n += unit_weight(p, x);
@@ -2300,7 +2489,12 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
       if (bt.sub[0].tma_in) {  // set for every subarray or for none
         converter_tma<FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
       } else {
-        converter_direct<DT, FMT, MULTI, SHAPE>(bt, cw, lane, abort_flag);
+        bool even = true;
+        for (int i = 0; i < bt.nsub; ++i) even = even && bt.sub[i].n % 2 == 0;
+        if (even)
+          converter_words<FMT, MULTI, SHAPE, true>(bt, cw, lane, abort_flag);
+        else
+          converter_words<FMT, MULTI, SHAPE, false>(bt, cw, lane, abort_flag);
       }
     } else {
       if (bt.sub[0].tma_in) {

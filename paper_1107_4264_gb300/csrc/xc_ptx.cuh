@@ -140,6 +140,31 @@ __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const void* tmap,
       : "memory");
 }
 
+// 4- and 2-byte global loads that do not allocate in L1, with an L2 policy: 0
+// (and no access) where `pred` is false.
+__device__ __forceinline__ uint32_t ld_global_b32_if(const void* p, uint64_t pol, bool pred) {
+  uint32_t v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "mov.b32 %0, 0;\n\t"
+      "@p ld.global.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;\n\t}"
+      : "=r"(v)
+      : "l"(p), "l"(pol), "r"(static_cast<uint32_t>(pred)));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_global_u16_if(const void* p, uint64_t pol, bool pred) {
+  uint32_t v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "mov.b32 %0, 0;\n\t"
+      "@p ld.global.L1::no_allocate.L2::cache_hint.u16 %0, [%1], %2;\n\t}"
+      : "=r"(v)
+      : "l"(p), "l"(pol), "r"(static_cast<uint32_t>(pred)));
+  return v;
+}
+
 // 32-byte global store (p 32-byte aligned) that does not allocate in L1,
 // with an L2 policy.
 __device__ __forceinline__ void st_global_v8_hint(void* p, const uint32_t (&v)[8], uint64_t pol) {
