@@ -240,7 +240,7 @@ struct AdjParams {
   const float2* x;
   const float2* gains;
   float2* grad_x;
-  float* grad_g;
+  double* grad_g;  // running sums, rounded to the caller's fp32 at the end
   unsigned long long timeout_ns;
   int* status;
 };
@@ -449,8 +449,8 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
         }
       }
       if (row_ok && P.grad_g) {
-        atomicAdd(P.grad_g + 2 * a, gg.x);
-        atomicAdd(P.grad_g + 2 * a + 1, gg.y);
+        atomicAdd(P.grad_g + 2 * a, static_cast<double>(gg.x));
+        atomicAdd(P.grad_g + 2 * a + 1, static_cast<double>(gg.y));
       }
     }
   }
@@ -460,6 +460,13 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, kTmemCols);
   }
+}
+
+// The gain gradient's sums over all tiles, added in float64 (fp32 partial sums
+// of 64 samples each).
+__global__ void adj_round_gains(const double* __restrict__ sums, float* __restrict__ grad_g, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) grad_g[i] = static_cast<float>(sums[i]);
 }
 
 AdjGeom adj_geom(const Geometry& g) {
@@ -477,7 +484,7 @@ AdjGeom adj_geom(const Geometry& g) {
 size_t adjoint_tc_workspace_bytes(const Geometry& g) {
   const AdjGeom G = adj_geom(g);
   const size_t per_rb = static_cast<size_t>(G.nk) * kOperand + kBlk * sizeof(int);  // tiles, row exponents
-  return static_cast<size_t>(g.F) * (G.na + G.nt) * per_rb + 256;
+  return static_cast<size_t>(g.F) * (G.na + G.nt) * per_rb + 2 * sizeof(double) * G.n;
 }
 
 cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* gains, void* grad_in,
@@ -494,7 +501,8 @@ cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* 
   const float2* x = static_cast<const float2*>(in);
   const float2* gn = static_cast<const float2*>(gains);
   cudaError_t e = cudaSuccess;
-  if (grad_g) e = cudaMemsetAsync(grad_g, 0, sizeof(float) * 2 * G.n, s);
+  double* sums = reinterpret_cast<double*>(exp_x + static_cast<size_t>(g.F) * G.nt * kBlk);
+  if (grad_g) e = cudaMemsetAsync(sums, 0, sizeof(double) * 2 * G.n, s);
   if (e != cudaSuccess) return e;
   // Chunks per thread: four (rows of up to 512 inputs in one pass) or one.
   const dim3 gh(G.na * (kBlk / kFormRows), g.F), gx(G.nt * (kBlk / kFormRows), g.F);
@@ -518,7 +526,7 @@ cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* 
   P.x = x;
   P.gains = gn;
   P.grad_x = static_cast<float2*>(grad_in);
-  P.grad_g = grad_g;
+  P.grad_g = grad_g ? sums : nullptr;
   P.timeout_ns = timeout_ns;
   P.status = status;
   int dev = 0, sms = 0;
@@ -527,6 +535,7 @@ cudaError_t launch_adjoint_tc(const void* grad_out, const void* in, const void* 
   if (e != cudaSuccess) return e;
   const long long ntiles = static_cast<long long>(g.F) * G.nt * G.na;
   adj_gemm_tc<<<static_cast<unsigned>(std::min<long long>(ntiles, sms)), kThreads, kSmemBytes, s>>>(P);
+  if (grad_g) adj_round_gains<<<(2 * G.n + 255) / 256, 256, 0, s>>>(sums, grad_g, 2 * G.n);
   return cudaGetLastError();
 }
 
