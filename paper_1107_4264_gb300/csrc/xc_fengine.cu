@@ -347,12 +347,18 @@ cudaError_t launch_fp(const void* in, int in_dt, void* out, int out_dt, int n, i
   return cudaGetLastError();
 }
 
-// CTA size by output type: 8-bit codes (2 bytes per complex value) take the
-// larger CTA, whose corner-turn runs cover whole 32-byte sectors.
+// CTA size by output type and length: 8-bit codes (2 bytes per complex value)
+// of more than 512 channels take the larger CTA, whose corner-turn runs cover
+// whole 32-byte sectors (1024 channels: 1.69 ms against 2.48).  Up to 512
+// channels the smaller CTA's runs do too, and two of them per SM work across
+// each other's barriers (100 stations x 2 pols, 512 channels, 4 taps, 1003
+// blocks: 504 -> 400 us).
 template <int LOGF>
 cudaError_t launch_f(const void* in, int in_dt, void* out, int out_dt, int n, int T, float scale,
                      const float* taps, int ntaps, cudaStream_t s) {
-  if (out_dt == 0) return launch_fp<LOGF, 14>(in, in_dt, out, out_dt, n, T, scale, taps, ntaps, s);
+  const bool wide_grid = n > 65535 * ((1 << 13) >> LOGF);  // too many inputs for the smaller CTA's grid
+  if (out_dt == 0 && (LOGF > 9 || wide_grid))
+    return launch_fp<LOGF, 14>(in, in_dt, out, out_dt, n, T, scale, taps, ntaps, s);
   return launch_fp<LOGF, 13>(in, in_dt, out, out_dt, n, T, scale, taps, ntaps, s);
 }
 
