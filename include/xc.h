@@ -121,11 +121,11 @@ xc_status xc_correlate(xc_handle* h, const void* in, void* out, void* stream);
  *   (re-read, nothing of the forward is stored); grad_in: device fp32,
  *   layout of `in`.  The gain gradient is kept for xc_get_grad_gains.
  *   Arithmetic: with the default XC_ENGINE_TENSOR, a tcgen05 complex GEMM on
- *   split hi/lo fp16 operands (per-channel power-of-two scales, three MMAs
- *   per step: about 22 significant bits) with fp32 accumulation; with
- *   XC_ENGINE_FP32, FP32 on the CUDA cores.  Allocates an F*n*n complex
- *   workspace (and, on the tensor cores, the hi/lo operand tiles) on first
- *   use.  Needs XC_CF32 input (XC_ERR_UNSUPPORTED otherwise).
+ *   split hi/lo fp16 operands (a power-of-two scale per input of H and per
+ *   sample of x, three MMAs per step: about 22 significant bits) with fp32
+ *   accumulation; with XC_ENGINE_FP32, FP32 on the CUDA cores.  Allocates its
+ *   workspace on first use: the hi/lo operand tiles, or with XC_ENGINE_FP32 an
+ *   F*n*n complex matrix.  Needs XC_CF32 input (XC_ERR_UNSUPPORTED otherwise).
  */
 xc_status xc_correlate_backward(xc_handle* h, const void* grad_out, const void* in, void* grad_in,
                                 void* stream);

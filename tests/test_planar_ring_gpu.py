@@ -68,3 +68,35 @@ def test_segments_bit_exact(N, P, F, T, loud, dev):
         finally:
             eng.close()
         assert np.array_equal(got[chans].cpu().numpy().astype(np.int64), want), name
+
+
+# Rows that TMA cannot stride: odd and even numbers of inputs, a half block
+# filled by one input or all but one, the last K-block by one sample; fp16 and
+# e4m3 operands; few units (dealt one by one) and many (in runs of two).
+@pytest.mark.parametrize("precision", [xc.XC_PREC_FP16, xc.XC_PREC_FP8], ids=["fp16", "fp8"])
+@pytest.mark.parametrize("N,P,F,T", [(1, 1, 1, 1), (65, 1, 3, 65), (63, 1, 40, 127), (33, 2, 7, 129),
+                                     (129, 1, 60, 513), (37, 2, 300, 320)])
+def test_unaligned_rows_bit_exact(N, P, F, T, precision, dev):
+    x = samples(N, P, F, T, "flat", 3300 + N + T)
+    chans = sorted(set([0, F // 2, F - 1]))
+    want = oracle.correlate_i8(x[:, chans].contiguous().numpy())
+    eng = xc.Correlator(N, P, F, T, "int8", precision=precision, tile=xc.XC_TILE_128)
+    try:
+        got = eng.correlate(x.to(dev), sync=True)
+    finally:
+        eng.close()
+    assert np.array_equal(got[chans].cpu().numpy().astype(np.int64), want)
+
+
+@pytest.mark.parametrize("N,P,F,T", [(449, 2, 3, 4033), (448, 2, 2, 4096), (897, 1, 2, 4032)])
+def test_default_shape_agrees_with_128(N, P, F, T, dev):
+    """Both sides of the rule that picks 128 x 256 items (N P > 896, T > 4032)."""
+    x = synth.uniform_int8((T, F, N, P, 2), -9, 9, 3400 + N, device=dev)
+    out = []
+    for tile in (xc.XC_TILE_AUTO, xc.XC_TILE_128):
+        eng = xc.Correlator(N, P, F, T, "int8", tile=tile)
+        try:
+            out.append(eng.correlate(x, sync=True))
+        finally:
+            eng.close()
+    assert torch.equal(out[0], out[1])
