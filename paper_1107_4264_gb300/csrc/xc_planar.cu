@@ -145,7 +145,7 @@ Params sub_params(const XeLaunch& L, int shape) {
   p.ring_slots = L.ring_slots;
   p.ready = L.counters;
   p.done = L.counters + L.ring_slots;
-  p.seg_units = 2 * p.nib * p.seg_kb;
+  p.seg_units = (p.n + 63) / 64 * p.seg_kb;  // (half blocks with no input are left as they are)
   p.mag_kb = div_magic(p.seg_kb);
   p.mag_slots = div_magic(p.ring_slots);
   p.tma_in = 0;
@@ -305,11 +305,13 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     const long long resident = static_cast<long long>(per_sm) * subs[0].grid;
     k->grid = static_cast<int>(std::min<long long>({items, static_cast<long long>(subs[0].grid), resident}));
   }
-  // Runs of two units once every converter warp has eight or more to do, of one
-  // below (2 stations x 1 pol, F=11, T=102: one CTA, 24 -> 17 us).  Then a
+  // Runs of two units once every converter warp has eight or more to do (and a
+  // segment is an even number of units), of one below (2 stations x 1 pol, F=11, T=102: one CTA, 24 -> 17 us).  Then a
   // warp's step from one run to its next, for its incremental unit numbers.
   const long long workers = static_cast<long long>(k->grid) * conv;
-  const int run = b->unit_base[nsub] >= 8 * workers ? kUnitRun : 1;
+  int run = b->unit_base[nsub] >= 8 * workers ? kUnitRun : 1;
+  for (int i = 0; i < nsub; ++i)
+    if (b->sub[i].seg_units % kUnitRun != 0) run = 1;
   const long long step = workers * run;
   for (int i = 0; i < nsub; ++i) {
     Params& p = b->sub[i];

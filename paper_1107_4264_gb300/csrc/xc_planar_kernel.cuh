@@ -235,7 +235,12 @@ struct Params {
   int ring_slots;      // segment slots, at least nseg
   unsigned* ready;     // [ring_slots]
   unsigned* done;      // [ring_slots]
-  int seg_units;       // converter units per segment = 2 * nib * seg_kb
+  // Converter units per segment: seg_kb for each 64-input half block that holds
+  // an input.  The last block's upper half is never written when it holds none:
+  // whatever the ring holds there only reaches rows and columns of the
+  // accumulators past n, which no one reads.  (A 48-input array converts half
+  // as many units, 400 inputs seven eighths.)
+  int seg_units;
   // Channels go through the ring in waves of `wave` (the last one of
   // wave_last, from segment number last_base on): see seg_first.
   int wave, wave_segs, wave_full, wave_last, last_base;
@@ -530,7 +535,7 @@ struct Unit {
 };
 
 // Converter warps take their units in runs of p.run (1 or 2) consecutive units
-// (always of one segment, whose unit count is even): one slot claim and one
+// (of one segment: runs are of two only where its unit count is even): one slot claim and one
 // publish (fence + release of the whole count) per run instead of per unit.
 // Warp gw of nw takes runs gw, gw + nw, gw + 2 nw, ... of the global unit
 // list.  Runs of one unit where there are too few units to go round.
