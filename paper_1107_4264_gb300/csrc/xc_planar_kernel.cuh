@@ -58,8 +58,8 @@
 // per operand, inputs 0..63 and 64..127 of a tile are its two contiguous
 // halves, and the 8 x 16 B core matrix that four converter lanes write is one
 // whole line.  8-bit input arrives by TMA in 128-row x 64-sample boxes (other
-// types likewise, other row counts by direct loads); each converter warp works
-// through its own stream of units.  Ring protocol:
+// types likewise; rows that TMA cannot stride by plain loads, 8-bit ones as
+// 32-bit words); each converter warp works through its own stream of units.  Ring protocol:
 //   ready[slot] counts converted units (64 inputs x 64 samples); segment G
 //     (generation G / slots of slot G % slots) is complete at
 //     ready >= (gen + 1) * units_per_segment;
