@@ -10,21 +10,21 @@
 // a complex GEMM with M = a (inputs), N = t (samples), K = b (inputs).  It
 // runs on tcgen05 in planar form:
 //     Re = Hr Xr^T - Hi Xi^T,   Im = Hr Xi^T + Hi Xr^T,
-// per 16-b step one 128 x 256 MMA, Hr [Xr Xi]^T into the adjacent accumulators
-// (D_re | D_im), and two of 128 x 128, Re -= Hi Xi^T (negate-B) and
-// Im += Hi Xr^T.  Operands are split into fp16 hi + lo parts after a
+// four 128 x 128 MMAs per 16-b step, the one of Hi Xi^T with negate-B.  (PTX
+// orders back-to-back MMAs on an accumulator only when they have the same
+// shape, so no 128 x 256 MMA, Hr [Xr Xi]^T, takes the place of two of them; it
+// gave no time either.)  Operands are split into fp16 hi + lo parts after a
 // power-of-two scale per row (input a of H', sample t of x, from its largest
 // component), and each step runs three times (hi hi, lo hi, hi lo): about 22
 // significant bits with fp32 accumulation over K = n.
 //
 // Kernels: operand formation, one pass over x and one over grad_out (H' is
 // formed straight from it), into 8 KiB MMA-ready tiles ([8-row group]
-// [8-column chunk][8 rows][8 fp16], the no-swizzle K-major layout, in which two
-// tiles one after the other are one operand of 256 rows); the GEMM, a persistent
-// kernel over 128 x 128 (a, t) tiles with a bulk-copy producer warp, an MMA
-// warp and eight epilogue warps that re-read x (nothing from the forward is
-// stored).  A stage holds all eight tiles of 32 b (hi and lo, re and im, of
-// both operands), 64 KiB for 18 MMAs: the three combinations share their
+// [8-column chunk][8 rows][8 fp16], the no-swizzle K-major layout); the GEMM,
+// a persistent kernel over 128 x 128 (a, t) tiles with a bulk-copy producer
+// warp, an MMA warp and eight epilogue warps that re-read x (nothing from the
+// forward is stored).  A stage holds all eight tiles of 32 b (hi and lo, re and im, of
+// both operands), 64 KiB for 24 MMAs: the three combinations share their
 // operands' copies.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -53,7 +53,6 @@ constexpr int kSmemBytes = kBarOff + kNumBars * 8 + 16 + 1024;
 constexpr uint32_t kTmemCols = 512;  // 2 sets x (D_re, D_im)
 constexpr uint32_t kIdesc = ptx::idesc_f16_f32(kBlk, kBlk);
 constexpr uint32_t kIdescNegB = kIdesc | (1u << 14);
-constexpr uint32_t kIdescWide = ptx::idesc_f16_f32(kBlk, 2 * kBlk);
 
 struct AdjGeom {
   Geometry g;
@@ -370,9 +369,9 @@ __global__ void __launch_bounds__(kThreads, 1) adj_gemm_tc(const AdjParams P) {
               const uint64_t dhr = dh + (j == 1 ? 2 * kT : 0) + ko, dhi = dhr + kT;
               const uint64_t dxr = dx + (j == 2 ? 2 * kT : 0) + ko, dxi = dxr + kT;
               const uint32_t acc = (kb > 0 || k > 0 || j > 0) ? 1u : 0u;
-              // Re += Hr Xr^T and Im += Hr Xi^T; B is 256 rows: the Xr tile's, then Xi's.
-              ptx::mma_f16_ss(d_re, dhr, dxr, kIdescWide, acc);
+              ptx::mma_f16_ss(d_re, dhr, dxr, kIdesc, acc);     // Re += Hr Xr^T
               ptx::mma_f16_ss(d_re, dhi, dxi, kIdescNegB, 1u);  // Re -= Hi Xi^T
+              ptx::mma_f16_ss(d_im, dhr, dxi, kIdesc, acc);     // Im += Hr Xi^T
               ptx::mma_f16_ss(d_im, dhi, dxr, kIdesc, 1u);      // Im += Hi Xr^T
             }
           }

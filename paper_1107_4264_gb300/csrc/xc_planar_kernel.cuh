@@ -75,7 +75,7 @@
 // CTA roles (persistent, one CTA per SM, channel-major items):
 //   warp 0      producer: 3 stages x (Ar, Ai, Br, Bi) of 64 samples (bulk copies);
 //               releases segments
-//   warp 1      MMA issuer; owns TMEM (2 sets x {D_im, D_re} x 128 columns)
+//   warp 1      MMA issuer; owns TMEM (2 sets x {D_re, D_im} x 128 columns)
 //   warps 2..5  epilogue
 //   warps 6..9  converters
 // What bounds it: the converters' and the epilogue's stores share the SM's
@@ -1868,10 +1868,8 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   static_assert(!(kTmemSum && WIDE), "hi/lo operands need TMEM columns 256..511 for their sums");
   // One accumulator set in TMEM (no double buffer) for 128 x 256 items:
   // D_re in columns 0..255, D_im in 256..511.  Other shapes alternate two
-  // sets of 128 + 128 columns, {D_im, D_re} for 128 x 128 blocks (one N = 256
-  // MMA, Ai [Br Bi]^T, adds to both) and {D_re, D_im} for pairs.
-  constexpr uint32_t kReCol = SHAPE == kShape128 ? 128 : 0;
-  constexpr uint32_t kImCol = WIDE ? 256 : (SHAPE == kShape128 ? 0 : 128);
+  // sets {D_re, D_im} of 128 + 128 columns.
+  constexpr uint32_t kImCol = WIDE ? 256 : 128;  // of D_im (D_re is at column 0 of its set)
   constexpr bool kOneSet = kTmemSum || WIDE;
   constexpr int TB = FmtT<FMT, SHAPE>::kTile;
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
@@ -2167,22 +2165,20 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           started = 0;
         }
         ptx::tc_fence_after();
-        const uint32_t d_re = d_acc + kReCol, d_im = d_acc + kImCol;
+        const uint32_t d_re = d_acc, d_im = d_acc + kImCol;
         const int mma_n = static_cast<int>(word >> kAccNShift);
         const uint32_t idesc = ptx::idesc_f16_f32(PAIR ? 2 * kBlk : kBlk, mma_n);
         const uint32_t idesc_negb = idesc | (1u << 14);
         const uint64_t dar0 = desc0 + static_cast<uint64_t>(stage) * kStageDesc;
         const bool same = !PAIR && !WIDE && (word & kAccSame);
         const uint64_t dbr0 = same ? dar0 : dar0 + 2 * kTileDesc;
-        // Full 128 x 128 blocks: Im += Ai Br^T and Re += Ai Bi^T in one
-        // 128 x 256 MMA (the Br and Bi tiles and the two accumulators lie side
-        // by side), then Re += Ar Br^T, Im -= Ar Bi^T.  The wide MMA reads Ai
-        // from shared memory once for both: 28 instead of 32 KiB per K-step of
-        // the shared-memory bandwidth that the stage copies and the converters
-        // share.  Alone, with stages arriving, 64 samples take 1025 cycles this
-        // way and 1114 with four 128 x 128 MMAs (1024 is the tensor rate).
-        constexpr uint32_t idesc2 = ptx::idesc_f16_f32(kBlk, 2 * kBlk);
-        const bool full_blk = SHAPE == kShape128 && mma_n == kBlk;
+        // Four MMAs per K-step, and every MMA into an accumulator has the same
+        // shape, as every step of an item has: only then does PTX order
+        // back-to-back MMAs on it.  (One 128 x 256 MMA for Im += Ai Br^T and
+        // Re += Ai Bi^T beside two of 128 x 128 would read 28 instead of 32 KiB
+        // of shared memory per K-step, 1025 cycles per 64 samples against 1114
+        // alone, but mixes shapes on both accumulators.  In the whole kernel it
+        // gave nothing: 256 stations, F=1024, T=1000 1.00 ms either way.)
         // K-step kk: 16-byte chunks 2kk and 2kk + 1 (16 fp16 or 32 e4m3 samples).
         auto kstep = [&](int kk) {
           const uint32_t acc = kk > 0 ? 1u : started;
@@ -2200,16 +2196,6 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
             ptx::mma_f16_ss_pair(d_re, dai, dbi, idesc, 1u);
             ptx::mma_f16_ss_pair(d_im, dai, dbr, idesc, acc);
             ptx::mma_f16_ss_pair(d_im, dar, dbi, idesc_negb, 1u);
-          } else if (full_blk) {
-            if constexpr (FMT == kFmtF8) {
-              ptx::mma_f8_ss(d_im, dai, dbr, idesc2, acc);
-              ptx::mma_f8_ss(d_re, dar, dbr, idesc, 1u);
-              ptx::mma_f8_ss(d_im, dar, dbi, idesc_negb, 1u);
-            } else {
-              ptx::mma_f16_ss(d_im, dai, dbr, idesc2, acc);
-              ptx::mma_f16_ss(d_re, dar, dbr, idesc, 1u);
-              ptx::mma_f16_ss(d_im, dar, dbi, idesc_negb, 1u);
-            }
           } else if constexpr (FMT == kFmtF8) {
             ptx::mma_f8_ss(d_re, dar, dbr, idesc, acc);
             ptx::mma_f8_ss(d_re, dai, dbi, idesc, 1u);
@@ -2398,8 +2384,8 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
             // Add the held chunk into this one inside TMEM and free it at
             // once, so the next item's MMAs need not wait for the stores.
             for (int j = 0; j < nblk; ++j) {
-              const uint32_t c_re = ab * 256 + kReCol, c_im = ab * 256 + kImCol;
-              const uint32_t h_re = (ab ^ 1u) * 256 + kReCol, h_im = (ab ^ 1u) * 256 + kImCol;
+              const uint32_t c_re = ab * 256, c_im = ab * 256 + kImCol;
+              const uint32_t h_re = (ab ^ 1u) * 256, h_im = (ab ^ 1u) * 256 + kImCol;
 #pragma unroll 1
               for (int piece = first_p[j]; piece <= last_p[j]; ++piece) {
                 uint32_t vr[32], vi[32], sr[32], si[32];
@@ -2424,7 +2410,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           for (int j = 0; j < nblk; ++j) {
             const int b = cb[j];
             // TMEM columns of block j: D_re and D_im of its 128 columns.
-            const uint32_t c_re = WIDE ? j * kBlk : ab * 256 + kReCol;
+            const uint32_t c_re = WIDE ? j * kBlk : ab * 256;
             const uint32_t c_im = WIDE ? 256 + j * kBlk : ab * 256 + kImCol;
 #pragma unroll 1
             for (int piece = first_p[j]; piece <= last_p[j]; ++piece) {
