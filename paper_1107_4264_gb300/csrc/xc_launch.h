@@ -6,6 +6,7 @@
 
 #include "xc.h"
 #include "xc_internal.h"
+#include "xc_planar_plan.h"
 
 namespace xc {
 
@@ -63,30 +64,7 @@ cudaError_t launch_xengine(const CUtensorMap* tmap, const XeLaunch& p, cudaStrea
 // kPlanarPair (two blocks sharing a column block on a CTA pair, tcgen05
 // cta_group::2) or kPlanarWide (two blocks sharing a row block on one CTA,
 // N = 256 MMAs).
-enum : int { kPlanar128 = 0, kPlanarPair = 1, kPlanarWide = 2 };
 cudaError_t launch_planar(const CUtensorMap* in_map, const XeLaunch& p, int shape, cudaStream_t s);
-// The default shape for a (virtual) geometry, input type and operand format.
-int planar_default_shape(const Geometry& g, int in_dtype, int fmt);
-constexpr int kMaxRingSlots = 1024;
-// Samples per converter unit of the planar engine (8-bit input arrives by TMA
-// in 128-row x 1 x kPlanarUnitT boxes).
-constexpr int kPlanarUnitT = 64;
-// The planar engine's operand ring: a channel's K-blocks are split into nseg
-// segments of seg_kb (the last one shorter), and a slot holds one segment's
-// operand tiles.
-struct PlanarRing {
-  int seg_kb, nseg, slots;
-  int64_t slot_bytes;
-};
-PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid);
-// The same with one segment per channel (the least memory that works: one slot).
-PlanarRing planar_ring_whole(const Geometry& g, int fmt);
-// Small arrays (n = N P <= 64 inputs): k consecutive channels, k the largest
-// divisor of F with k n <= 128, are correlated as one virtual channel of k N
-// stations.  The input [T][F][n] is the same memory as [T][F / k][k n], so
-// nothing moves; one 128 x 128 block then holds the k channels' own blocks on
-// its diagonal.  Returns that virtual geometry and k (1 for larger arrays).
-Geometry planar_geometry(const Geometry& g, int* pack);
 
 // F-engine (xc_fengine.cu): in [n][T F] complex (in_dtype 0 int8, 1 fp16,
 // 2 fp32) -> out [T - ntaps + 1][F][n] complex (out_dtype 0 int8

@@ -1,7 +1,8 @@
 // xc_planar.cu -- host side of the planar tensor-core X-engine (the kernel
 // template is xc_planar_kernel.cuh): the single-CTA instantiations, the
-// float scale pre-pass, the kernel parameter block, the ring geometry and
-// the launch (single CTAs, or CTA pairs from xc_planar_pair.cu).
+// float scale pre-pass, the kernel parameter block and the launch (single CTAs,
+// or CTA pairs from xc_planar_pair.cu).  Its sizes are decided in
+// xc_planar_plan.h.
 #include "xc_planar_kernel.cuh"
 
 namespace xc {
@@ -13,6 +14,8 @@ const void* planar_wide_select(int in_dtype, int fmt, bool multi);
 
 static_assert(kShape128 == kPlanar128 && kShapePair == kPlanarPair && kShapeWide == kPlanarWide,
               "tile shape codes");
+static_assert(kFmtF16 == XC_PREC_FP16 && kFmtHiLo == XC_PREC_HILO && kFmtF8 == XC_PREC_FP8 && kBlk == kPlanarBlk,
+              "xc_planar_plan.h counts in the kernel's formats and blocks");
 
 namespace {
 
@@ -109,9 +112,6 @@ cudaError_t launch_amax(const XeLaunch& L, int n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int fmt_kt(int fmt) { return fmt == kFmtHiLo ? 2 : 1; }
-int fmt_tile_bytes(int fmt) { return fmt == kFmtF8 ? (1 << 13) : (1 << 14); }
-
 // fast_div's magic of a divisor (0 for a divisor of 0, which nothing divides by).
 unsigned div_magic(int d) {
   return d <= 0 ? 0u : d == 1 ? 0xffffffffu : static_cast<unsigned>((1ull << 32) / static_cast<unsigned>(d));
@@ -134,7 +134,7 @@ Params sub_params(const XeLaunch& L, int shape) {
   const int fmt = p.is_int ? (L.fmt == kFmtF8 ? kFmtF8 : kFmtF16) : L.fmt;
   p.seg_kb = std::max(1, L.ring_seg_kb);
   p.nseg = (p.nkb + p.seg_kb - 1) / p.seg_kb;
-  p.nkt = fmt_kt(fmt) * p.seg_kb;
+  p.nkt = (fmt == kFmtHiLo ? 2 : 1) * p.seg_kb;
   p.amax = L.amax;
   p.gains = static_cast<const float2*>(L.gains);
   p.in_amax = p.is_int ? nullptr : L.in_amax;
@@ -160,83 +160,6 @@ Params sub_params(const XeLaunch& L, int shape) {
 }
 
 }  // namespace
-
-Geometry planar_geometry(const Geometry& g, int* pack) {
-  int k = 1;
-  const int64_t n = static_cast<int64_t>(g.N) * g.P;
-  if (n <= kBlk / 2) {
-    for (int c = static_cast<int>(kBlk / n); c >= 2; --c) {
-      if (g.F % c == 0) {
-        k = c;
-        break;
-      }
-    }
-  }
-  Geometry v = g;
-  v.N = g.N * k;
-  v.F = g.F / k;
-  v.R = g.R * k;
-  v.NB = static_cast<int64_t>(v.N) * (v.N + 1) / 2;
-  if (pack) *pack = k;
-  return v;
-}
-
-namespace {
-PlanarRing ring_of(const Geometry& g, int fmt, int seg_kb) {
-  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
-  PlanarRing r;
-  r.seg_kb = seg_kb;
-  r.nseg = (g.Tp / kBK + seg_kb - 1) / seg_kb;
-  r.slots = 1;
-  r.slot_bytes = 2 * fmt_kt(fmt) * static_cast<int64_t>(seg_kb) * nib * fmt_tile_bytes(fmt);
-  return r;
-}
-}  // namespace
-
-PlanarRing planar_ring_whole(const Geometry& g, int fmt) { return ring_of(g, fmt, g.Tp / kBK); }
-
-// 128 x 256 items for large arrays with long integrations, whose channels are
-// few and big: a quarter fewer operand bytes per MAC, and no more channels in
-// flight than the ring can feed.  Measured (8-bit input, ms, 128 x 128 / 128 x
-// 256): N=1024 F=16 T=8192 1.39 / 1.23, N=512 F=64 T=4096 0.81 / 0.71, N=256
-// F=64 T=8192 0.59 / 0.60, N=384 F=256 T=2048 0.96 / 0.95, N=1024 F=32 T=1000
-// 0.41 / 0.40, N=256 F=1024 T=1000 0.98 / 1.01.  Float input, whose converters
-// set the pace, stays with 128 x 128 (N=512 F=60 T=2048 0.75 / 0.87).
-int planar_default_shape(const Geometry& g, int in_dtype, int fmt) {
-  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
-  return in_dtype == 0 && fmt == kFmtF16 && nib >= 8 && g.Tp >= 4096 ? kShapeWide : kShape128;
-}
-
-// Segments of at most 8 K-blocks (512 samples; half as many with hi/lo
-// operands, which take twice the bytes) and 60 MiB of ring, so that it stays
-// in the 129 MB L2 beside the streams.  Measured (8-bit input, ms):
-//   K-blocks per segment       16     8     4
-//     N=100 F=512  T=1000   0.243 0.207 0.203
-//     N=256 F=1024 T=1000   0.987 0.969 0.988
-//     N=200 F=256  T=512    0.144 0.144 0.150
-//   ring                   50 MiB 60 MiB 75 MiB 90 MiB 120 MiB 250 MiB
-//     N=256 F=1024 T=1000   1.028  0.977  1.044  1.100   1.144
-//     N=256 F=256  T=4096          1.104         1.004   1.061   1.099
-//     N=256 F=64   T=8192          0.671         0.604   0.605   0.602
-//     N=512 F=64   T=4096          0.809         0.822   0.830   0.824
-// So 90 MiB when the channels of a wave take more than 80 MiB (8-bit input:
-// the float converters are too slow to fill it), and 120 MiB on 128 x 256
-// items (N=512 F=64 T=4096 0.708 against 0.777 ms).
-PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid) {
-  const int seg = fmt == kFmtHiLo ? 4 : 8;
-  const int nkb = g.Tp / kBK;
-  const int parts = (nkb + seg - 1) / seg;
-  PlanarRing r = ring_of(g, fmt, (nkb + parts - 1) / parts);
-  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kBlk - 1) / kBlk;
-  const int64_t wave = std::max<int64_t>(1, grid / (nib * (nib + 1) / 2));
-  int64_t mib = 60;
-  if (in_dtype == 0 && wave * r.nseg * r.slot_bytes > (80ll << 20)) mib = 90;
-  if (planar_default_shape(g, in_dtype, fmt) == kShapeWide) mib = 120;
-  int64_t n = std::min<int64_t>((mib << 20) / r.slot_bytes, kMaxRingSlots);
-  n = std::max<int64_t>(n, std::max<int64_t>(4, r.nseg + 4));
-  r.slots = static_cast<int>(std::min<int64_t>(n, static_cast<int64_t>(g.F) * r.nseg));
-  return r;
-}
 
 cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps, int nsub,
                            PlanarKernel* k, int shape) {
@@ -306,8 +229,9 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     k->grid = static_cast<int>(std::min<long long>({items, static_cast<long long>(subs[0].grid), resident}));
   }
   // Runs of two units once every converter warp has eight or more to do (and a
-  // segment is an even number of units), of one below (2 stations x 1 pol, F=11, T=102: one CTA, 24 -> 17 us).  Then a
-  // warp's step from one run to its next, for its incremental unit numbers.
+  // segment is an even number of units), of one below (2 stations x 1 pol, F=11,
+  // T=102: one CTA, 24 -> 17 us).  Then a warp's step from one run to its next,
+  // for its incremental unit numbers.
   const long long workers = static_cast<long long>(k->grid) * conv;
   int run = b->unit_base[nsub] >= 8 * workers ? kUnitRun : 1;
   for (int i = 0; i < nsub; ++i)
@@ -321,10 +245,7 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
     p.step_gen = p.step_seg / p.ring_slots;
     p.step_slot = p.step_seg % p.ring_slots;
     const int item_step = pair ? k->grid / 2 : k->grid;
-    // Waves: as many channels as there are CTAs (clusters) for their items,
-    // and no more than half the ring's slots.  (N=256 F=64 T=8192 on a 60 MiB
-    // ring: 0.686 ms, and 1.150 ms with one channel to a wave.)
-    p.wave = std::max(1, std::min({item_step / p.ipc, p.ring_slots / 2, p.g.F}));
+    p.wave = planar_wave(item_step, p.ipc, p.ring_slots, p.g.F);
     if (p.ipc > item_step && p.ring_slots < p.nseg) return cudaErrorInvalidConfiguration;
     p.wave_segs = p.wave * p.nseg;
     p.wave_full = p.g.F / p.wave;

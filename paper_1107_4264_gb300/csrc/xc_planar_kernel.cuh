@@ -66,11 +66,15 @@
 //   done[slot] counts work items whose MMAs have read the segment; slot s may
 //     take segment G once done >= gen(G) * items_per_channel.
 // A segment waits for segments of lower number only, and a work item for
-// segments of its own channel.  All CTAs are co-resident and each has at most
-// one item of a wave, so the items of the lowest number not yet read are at
-// work or come next once the waves before are done: the ring cannot deadlock.
-// (When a channel has more items than there are CTAs, a wave is one channel
-// and the ring holds all its segments.)  Every wait is bounded regardless.
+// segments of its own channel, one after the other: the producer for each when
+// it comes to it, the MMA warp for stages and drained accumulators, and the
+// epilogue for full accumulators alone (stage_acc, acc_last), never for a
+// segment, so a drain needs nothing that the MMAs before it did not.  All CTAs
+// are co-resident and each has at most one item of a wave, so the items of the
+// lowest number not yet read are at work or come next once the waves before are
+// done: the ring cannot deadlock, however little of a wave it holds.  (When a
+// channel has more items than there are CTAs, a wave is one channel and the
+// ring holds all its segments.)  Every wait is bounded regardless.
 //
 // CTA roles (persistent, one CTA per SM, channel-major items):
 //   warp 0      producer: 3 stages x (Ar, Ai, Br, Bi) of 64 samples (bulk copies);
@@ -197,9 +201,9 @@ struct Cfg {
   static constexpr int kBarOff = kConvOff + conv_warps<FMT, DT>() * kConvBufBytes;
   // full, empty (and pfull) per stage; accf, acce x 2; drain; one per converter
   static constexpr int kNumBars = (SHAPE == kShapePair ? 3 : 2) * kStages + 5 + conv_warps<FMT, DT>();
-  // then the TMEM address, the abort flag and one word per stage (the chunk
-  // length of the item whose first step the stage holds)
-  static constexpr int kSmemBytes = kBarOff + kNumBars * 8 + 8 + 4 * kStages + 1024;
+  // then the TMEM address, the abort flag, one word per stage (stage_acc) and
+  // one per accumulator set (acc_last)
+  static constexpr int kSmemBytes = kBarOff + kNumBars * 8 + 8 + 4 * (kStages + 2) + 1024;
   static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
@@ -465,24 +469,6 @@ constexpr unsigned kExactSum = 1u << 24;
 __device__ __forceinline__ unsigned kblock_growth(const Params& p, int G) {
   const unsigned m = *reinterpret_cast<volatile const unsigned*>(p.amax + G);
   return 2u * m * m * kBK;
-}
-
-// First K-block after the exact chunk that starts at kb0 of the channel whose
-// segments are G0, G0 + width, ...: the same walk as the producer's (which
-// tells the MMA warp).  Every segment of the channel has been converted.
-__device__ __forceinline__ int exact_chunk_end(const Params& p, int G0, int width, int kb0) {
-  int seg = kb0 / p.seg_kb, left = p.seg_kb - (kb0 - seg * p.seg_kb);
-  unsigned sum = 0, grow = kblock_growth(p, G0 + seg * width);
-  for (int kb = kb0; kb < p.nkb; ++kb) {
-    if (left == 0) {
-      grow = kblock_growth(p, G0 + ++seg * width);
-      left = p.seg_kb;
-    }
-    if (kb > kb0 && sum + grow > kExactSum) return kb;
-    sum += grow;
-    --left;
-  }
-  return p.nkb;
 }
 
 // -------------------------------------------------------------- converter
@@ -1822,6 +1808,11 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   // stage's arrive, so the MMA thread reads it after its wait with no global
   // round trip of its own.
   volatile int* stage_acc = reinterpret_cast<volatile int*>(tmem_holder + 2);
+  // 8-bit input: is the group in accumulator set b the last one of its item?
+  // The MMA warp, which learns from the stages where groups end, writes it
+  // before it arrives on accf (the second arrival beside the MMAs' own); the
+  // epilogue reads it before it releases the set.
+  uint32_t* acc_last = tmem_holder + 2 + kStages;
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // (known uniform)
   const int lane = threadIdx.x & 31;
@@ -1835,7 +1826,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
       if (PAIR) ptx::mbar_init(pfull_bar(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      ptx::mbar_init(accf_bar(b), 1);
+      ptx::mbar_init(accf_bar(b), IS_INT ? 2 : 1);
       ptx::mbar_init(acce_bar(b), (PAIR ? 2 : 1) * kNumEpiWarps);
     }
     ptx::mbar_init(drain_bar, 1);
@@ -2114,8 +2105,16 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
     // K-block when the epilogue sums 64-sample fp32 blocks in TMEM (buffer 0
     // only).  The producer says where they start and, where it knows (not for
     // 8-bit chunks, whose end depends on the next segment's values), end.
-    auto commit_acc = [&](uint32_t ab) {
+    auto commit_acc = [&](uint32_t ab, bool last) {
       if (issuer) {
+        if constexpr (IS_INT) {
+          *reinterpret_cast<volatile uint32_t*>(acc_last + ab) = last ? 1u : 0u;
+          ptx::mbar_arrive(accf_bar(ab));
+          if constexpr (PAIR) {
+            ptx::st_shared_remote(ptx::mapa_shared(ptx::smem_u32(acc_last + ab), 1), last ? 1u : 0u);
+            ptx::mbar_arrive_remote(ptx::mapa_shared(accf_bar(ab), 1));
+          }
+        }
         if constexpr (PAIR) {
           ptx::mma_commit_pair_mc(accf_bar(ab), 0x3);
         } else {
@@ -2150,7 +2149,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
         }
         if (word & kAccStart) {
           if (open) {
-            commit_acc(ab);
+            commit_acc(ab, false);
             ++u;
           }
           ab = kOneSet ? 0u : (u & 1u);
@@ -2230,8 +2229,8 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           }
         }
         started = 1;
-        if (word & kAccEnd) {
-          commit_acc(ab);
+        if (word & kAccEnd) {  // (8-bit input: of the item's last group only)
+          commit_acc(ab, true);
           ++u;
           open = false;
         }
@@ -2303,38 +2302,16 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
       }
       // The last block with pieces to read releases the accumulator after them.
       const int jlast = (nblk == 2 && last_p[1] >= 0) ? 1 : (last_p[0] >= 0 ? 0 : -1);
-      // 8-bit input: does one exact chunk hold the whole integration?  (Lane l
-      // looks at segments l, l + 32, ... once they are converted.)
-      bool one_chunk = true;
-      int width;
-      const int G0 = seg_first(p, f, &width);
-      if constexpr (IS_INT) {
-        bool rdy = true;
-        unsigned sum = 0;  // capped: at most 32 lanes x 2^25
-        for (int sg = lane; sg < p.nseg; sg += 32) {
-          const int G = G0 + sg * width, gen = fast_div(G, p.ring_slots, p.mag_slots);
-          rdy = rdy && wait_counter(p.ready + G - gen * p.ring_slots,
-                                    static_cast<unsigned>(gen + 1) * static_cast<unsigned>(p.seg_units), p,
-                                    abort_flag);
-          const unsigned nk = static_cast<unsigned>(min(p.seg_kb, p.nkb - sg * p.seg_kb));
-          sum = min(sum + min(nk * kblock_growth(p, G), 2 * kExactSum), 2 * kExactSum);
-        }
-        if (!__all_sync(0xffffffffu, rdy)) {
-          ok = false;
-          break;
-        }
-        one_chunk = __reduce_add_sync(0xffffffffu, sum) <= kExactSum;
-      }
-      int ch = -1;
-      for (int kb0 = 0, kb1; ok && kb0 < p.nkb; kb0 = kb1) {
-        ++ch;
-        if (IS_INT)
-          kb1 = one_chunk ? p.nkb : exact_chunk_end(p, G0, width, kb0);
-        else
-          kb1 = min(p.nkb, kb0 + p.f_chunk_kb);
+      // The item's chunks: of f_chunk_kb K-blocks (float input), or until the
+      // MMA warp says that an accumulator holds the last one (8-bit input, one
+      // group each).
+      int kb0 = 0;
+      bool last_chunk = false;
+      for (int ch = 0; ok && !last_chunk; ++ch) {
+        const int kb1 = IS_INT ? kb0 + 1 : min(p.nkb, kb0 + p.f_chunk_kb);
+        if (!IS_INT) last_chunk = kb1 == p.nkb;
         const int gstep = kTmemSum ? 1 : (kb1 - kb0);
         const bool add = p.accumulate || ch > 0;
-        const bool last_chunk = kb1 == p.nkb;
         // FP64 block sums: chunks pair off, (0, 1), (2, 3), ...  The first
         // chunk of a pair stays in its TMEM accumulator (`hold`); the second's
         // drain adds it in fp32 (a correctly rounded sum of the two partials,
@@ -2374,6 +2351,10 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           if (!__all_sync(0xffffffffu, got)) {
             ok = false;
             break;
+          }
+          if constexpr (IS_INT) {
+            if (PAIR) ptx::mbar_acquire_cluster(accf_bar(ab), ap);  // (the peer's word comes from the leader)
+            last_chunk = *reinterpret_cast<volatile uint32_t*>(acc_last + ab) != 0;
           }
           ptx::tc_fence_after();
           if (hold) {  // drained with the next chunk
@@ -2470,6 +2451,7 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
           if (kTmemSum && !glast) ptx::tmem_wait_st();
           ++u;
         }
+        kb0 = kb1;
       }
     }
   } else {
