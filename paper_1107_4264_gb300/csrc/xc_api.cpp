@@ -84,7 +84,9 @@ struct BatchSub {
   void* ring = nullptr;
   size_t ring_bytes = 0;  // the region's size (for the 2x candidate)
   unsigned* counters = nullptr;
+  int counter_slots = 0;  // ring slots that `counters` serves
   unsigned* amax = nullptr;
+  int64_t amax_words = 0;
 };
 struct BatchState {
   int nsub = 0;
@@ -118,7 +120,9 @@ struct xc_handle {
   void* ring = nullptr;
   int ring_slots = 0;
   unsigned* counters = nullptr;
+  int counter_slots = 0;          // ring slots that `counters` serves (either engine, any format)
   unsigned* chan_amax = nullptr;  // [F][nseg] max |x| per channel segment (planar engine)
+  int64_t amax_words = 0;         // its size
   CUtensorMap ring_tmap;     // interleaved form: {Tp, R, ring_slots}
   xc::PlanarRing pring{};     // planar form
   // Planar engine geometry: small arrays pack `pack` consecutive channels into
@@ -303,7 +307,9 @@ xc_status launch_one(xc_handle* h, const void* in, void* out, cudaStream_t s) {
     X.ring_slots = h->pring.slots;
     X.ring_seg_kb = h->pring.seg_kb;
     X.counters = h->counters;
+    X.counter_slots = h->counter_slots;
     X.amax = h->chan_amax;
+    X.amax_words = h->amax_words;
     X.gains = gains;
     X.fmt = h->precision;
     X.in_amax = h->in_amax;
@@ -647,15 +653,16 @@ xc_handle* xc_create(int nstation, int npol, int nfreq, int ntime, xc_dtype in_d
   h->ring_slots = xc::xengine_ring_slots(h->g);
   h->pg = xc::planar_geometry(h->g, &h->pack);
   h->pring = xc::planar_ring(h->pg, in_dtype, XC_PREC_FP16, h->num_sms);
-  const int slots = std::max({h->ring_slots, h->pring.slots, xc::kMaxRingSlots});
+  h->counter_slots = std::max(h->ring_slots, xc::planar_max_slots(h->pg, in_dtype, h->num_sms));
+  h->amax_words = static_cast<int64_t>(nfreq) * h->pring.nseg;  // (8-bit input: the same in both its formats)
   h->ring_bytes = std::max(static_cast<size_t>(h->ring_slots) * R * Tp * 2,
                            static_cast<size_t>(h->pring.slots) * h->pring.slot_bytes);
   e = cudaMalloc(&h->ring, h->ring_bytes);
   if (e == cudaSuccess)
-    e = cudaMalloc(reinterpret_cast<void**>(&h->counters), 2 * sizeof(unsigned) * slots);
+    e = cudaMalloc(reinterpret_cast<void**>(&h->counters), 2 * sizeof(unsigned) * h->counter_slots);
   if (e == cudaSuccess)
     e = cudaMalloc(reinterpret_cast<void**>(&h->chan_amax),
-                   sizeof(unsigned) * static_cast<size_t>(nfreq) * h->pring.nseg);
+                   sizeof(unsigned) * static_cast<size_t>(h->amax_words));
   if (e == cudaSuccess && in_dtype != XC_CI8)
     e = cudaMalloc(reinterpret_cast<void**>(&h->in_amax),
                    sizeof(unsigned) * static_cast<size_t>(nfreq) * nstation * npol);
@@ -1131,10 +1138,12 @@ xc_status batch_prepare(xc_handle* h, const void* const* in, void* const* out,
     const xc::PlanarRing& pr = packed ? s.ring1 : s.ring1_unpacked;
     X.ring_slots = static_cast<int>(std::min<int64_t>(
         {static_cast<int64_t>(s.ring_bytes) / pr.slot_bytes, static_cast<int64_t>(pr.slots) * depth,
-         std::max<int64_t>(xc::kMaxRingSlots, pr.slots)}));
+         static_cast<int64_t>(s.counter_slots)}));
     X.ring_seg_kb = pr.seg_kb;
     X.counters = s.counters;
+    X.counter_slots = s.counter_slots;
     X.amax = s.amax;
+    X.amax_words = s.amax_words;
     X.gains = nullptr;
     X.grid = h->num_sms;
     X.timeout_ns = h->timeout_ns;
@@ -1218,6 +1227,8 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
     const size_t one = std::max(static_cast<size_t>(s.ring1.slots) * s.ring1.slot_bytes,
                                 static_cast<size_t>(s.ring1_unpacked.slots) * s.ring1_unpacked.slot_bytes);
     s.ring_bytes = std::max(one, std::min<size_t>(2 * one, 512u << 20));
+    s.counter_slots = std::max({xc::kMaxRingSlots, s.ring1.slots, s.ring1_unpacked.slots});
+    s.amax_words = static_cast<int64_t>(s.g.F) * s.ring1.nseg;  // (packed or not: nseg is the same)
     ring_off[i] = ring_total;
     ring_total += (s.ring_bytes + 255) / 256 * 256;
     in_total += s.in_bytes;
@@ -1226,11 +1237,8 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
   h->in_bytes = in_total;
   h->out_bytes = out_total;
   size_t ctr_words = 0;
-  auto ctr_of = [](const BatchSub& s) {  // ready and done counters of the deepest ring
-    return 2 * static_cast<size_t>(std::max({xc::kMaxRingSlots, s.ring1.slots, s.ring1_unpacked.slots}));
-  };
   for (int i = 0; i < nsub; ++i)
-    ctr_words += ctr_of(b->sub[i]) + static_cast<size_t>(b->sub[i].g.F) * b->sub[i].ring1.nseg;
+    ctr_words += 2 * static_cast<size_t>(b->sub[i].counter_slots) + static_cast<size_t>(b->sub[i].amax_words);
   cudaError_t e = cudaMalloc(&b->ring_all, ring_total);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&b->ctr_all), ctr_words * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
@@ -1244,9 +1252,9 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
     BatchSub& s = b->sub[i];
     s.ring = static_cast<char*>(b->ring_all) + ring_off[i];
     s.counters = c;
-    c += ctr_of(s);
+    c += 2 * static_cast<size_t>(s.counter_slots);
     s.amax = c;
-    c += static_cast<size_t>(s.g.F) * s.ring1.nseg;
+    c += static_cast<size_t>(s.amax_words);
     b->order[i] = i;
   }
   b->depth = 1;

@@ -42,6 +42,9 @@ struct XeLaunch {
   int ring_seg_kb = 0; // planar engine: K-blocks per ring segment
   unsigned* counters;  // 2 * ring_slots, zeroed by the launcher on `s`
   unsigned* amax;      // [F][segments] max |x| (planar engine, 8-bit input)
+  // Planar engine: what the two hold, which planar_prepare checks.
+  int counter_slots = 0;
+  int64_t amax_words = 0;
   const void* gains;   // cf32 [N][P] applied to float input (planar engine), or NULL
   // Planar engine, float input:
   int fmt = 0;              // operand format: 0 fp16, 1 split hi/lo fp16, 2 e4m3

@@ -195,7 +195,9 @@ extern "C" xc_status xc_correlate_noalloc(int nstation, int npol, int nfreq, int
   X.ring_slots = ring.slots;
   X.ring_seg_kb = ring.seg_kb;
   X.counters = reinterpret_cast<unsigned*>(s.scratch + off_ctr);
+  X.counter_slots = ring.slots;
   X.amax = reinterpret_cast<unsigned*>(s.scratch + off_amax);
+  X.amax_words = static_cast<int64_t>(pg.F) * ring.nseg;
   X.gains = nullptr;
   X.fmt = XC_PREC_FP16;
   X.in_amax = in_dtype == XC_CI8 ? nullptr : reinterpret_cast<unsigned*>(s.scratch + off_inamax);

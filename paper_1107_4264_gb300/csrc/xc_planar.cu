@@ -177,7 +177,8 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
   for (int i = 0; i < nsub; ++i) {
     if (subs[i].in_dtype != dt || fmt_of(subs[i]) != fmt) return cudaErrorInvalidValue;
     b->sub[i] = sub_params(subs[i], shape);
-    if (subs[i].ring_slots < 1) return cudaErrorInvalidValue;
+    if (subs[i].ring_slots < 1 || subs[i].ring_slots > subs[i].counter_slots) return cudaErrorInvalidValue;
+    if (dt == 0 && static_cast<int64_t>(subs[i].g.F) * b->sub[i].nseg > subs[i].amax_words) return cudaErrorInvalidValue;
     if (maps && maps[i]) {
       b->maps[i] = *maps[i];
     } else {

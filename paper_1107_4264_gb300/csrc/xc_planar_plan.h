@@ -111,6 +111,16 @@ inline PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid
   return r;
 }
 
+// Ring slots that the counters of a handle have to serve: the most that any
+// operand format of its input type asks for.  (A ring is at least nseg + 4
+// slots, whatever kMaxRingSlots says, and hi/lo segments are half as long.)
+inline int planar_max_slots(const Geometry& g, int in_dtype, int grid) {
+  int n = planar_ring(g, in_dtype, XC_PREC_FP16, grid).slots;
+  n = std::max(n, planar_ring(g, in_dtype, XC_PREC_FP8, grid).slots);
+  if (in_dtype != 0) n = std::max(n, planar_ring(g, in_dtype, XC_PREC_HILO, grid).slots);
+  return n;
+}
+
 // Channels per wave: as many as there are CTAs (clusters: `workers`) for their
 // items, and no more than half the ring's slots.  (N=256 F=64 T=8192 on a 60 MiB
 // ring: 0.686 ms, and 1.150 ms with one channel to a wave.)
