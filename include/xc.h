@@ -90,10 +90,10 @@ typedef enum {
  * Create an engine for fixed sizes on the current CUDA device.
  *   nstation N >= 1, npol P in {1, 2}, nfreq F >= 1 (at most 65535),
  *   ntime T >= 1.
- * Allocates the workspace: a ring of tensor-core operand tiles (60 to 120 MiB,
- * or the whole operand set if that is less, so that it stays in L2; at least
- * one channel),
- * plus counters and a status word.  Small arrays (N*P <= 64) have k
+ * Allocates the workspace: a ring of tensor-core operand tiles (60 or 90 MiB,
+ * so that it stays in L2; the whole operand set if that is less; always room
+ * for one channel and four segments of 512 samples), plus counters and a
+ * status word.  Small arrays (N*P <= 64) have k
  * consecutive channels correlated together in one tensor-core block (k the
  * largest divisor of F with k*N*P <= 128); this is internal and changes
  * neither layouts nor results.  Returns NULL on error; the reason is in
@@ -207,8 +207,11 @@ enum { XC_PREC_FP16 = 0, XC_PREC_HILO = 1, XC_PREC_FP8 = 2 };
  *     each SM stages its 128 rows and half of the 128 columns.
  *   XC_TILE_WIDE: two 128 x 128 blocks sharing a row block per CTA, one
  *     128 x 256 MMA per step (N = 256; one TMEM accumulator set): a quarter
- *     fewer shared-memory and L2 operand bytes per MAC than XC_TILE_128.  Not
- *     with XC_PREC_HILO (XC_ERR_UNSUPPORTED at the call).
+ *     fewer shared-memory and L2 operand bytes per MAC than XC_TILE_128.
+ *     Faster for large arrays with long integrations of quiet 8-bit samples;
+ *     several times slower once 2 * max|x|^2 * ntime passes 2^24, from where
+ *     the integration is drained in several exact chunks.  Not with
+ *     XC_PREC_HILO (XC_ERR_UNSUPPORTED at the call).
  *   XC_TILE_SMALL: the small-array engine (8-bit input, fp16 operands or,
  *     with XC_PREC_FP8, e4m3 operands for |x| <= 16 with the same range
  *     report; W = 2 * nstation * npol in {16, 32, 64, 128, 256}).  Each input is two
@@ -226,11 +229,8 @@ enum { XC_PREC_FP16 = 0, XC_PREC_HILO = 1, XC_PREC_FP8 = 2 };
  *     operand forms, and for batch handles.
  *   XC_TILE_AUTO: XC_TILE_SMALL where it applies (see
  *     xc_small_engine_channels; an input pointer that is not 16-byte aligned
- *     keeps the planar engine), else
- *     the planar shape measured fastest: XC_TILE_WIDE for 8-bit input with
- *     fp16 operands, nstation * npol > 896 and ntime > 4032, XC_TILE_128 for
- *     the rest.  A batch handle takes the shape xc_batch_tune chose
- *     (XC_TILE_AUTO restores the default). */
+ *     keeps the planar engine), else XC_TILE_128.  A batch handle takes the
+ *     shape xc_batch_tune chose (XC_TILE_AUTO restores XC_TILE_128). */
 enum { XC_TILE_AUTO = 0, XC_TILE_128 = 1, XC_TILE_PAIR = 2, XC_TILE_WIDE = 3, XC_TILE_SMALL = 4 };
 /* Engines:
  *   XC_ENGINE_TENSOR (default): one fused persistent tcgen05 kernel in

@@ -98,7 +98,6 @@ struct BatchState {
   bool packing = true;  // small subarrays' channels packed into one block (see planar_geometry)
   char cache_path[1024] = "";  // xc_batch_set_cache
   int shape = xc::kPlanar128;  // tile shape (xc::kPlanar*), tuned by xc_batch_tune
-  int shape_default = xc::kPlanar128;
   cudaStream_t cap_stream = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -173,12 +172,12 @@ xc_status encode_operand_map(CUtensorMap* map, void* base, int64_t R, int64_t Tp
 void batch_drop_graph(BatchState* b);
 
 // Planar tile shape for an XC_TILE_* option value (-1: not available).
-int planar_shape(int tile, const xc::Geometry& pg, int in_dtype, int fmt) {
+int planar_shape(int tile, int fmt) {
   switch (tile) {
     case XC_TILE_128: return xc::kPlanar128;
     case XC_TILE_PAIR: return xc::kPlanarPair;
     case XC_TILE_WIDE: return fmt == XC_PREC_HILO ? -1 : xc::kPlanarWide;
-    default: return xc::planar_default_shape(pg, in_dtype, fmt);
+    default: return xc::kPlanar128;
   }
 }
 
@@ -327,7 +326,7 @@ xc_status launch_one(xc_handle* h, const void* in, void* out, cudaStream_t s) {
       im = &in_map;
     }
     if (tm) tm->nkern = 1;
-    const int shape = planar_shape(h->tile, h->pg, X.in_dtype, h->precision);
+    const int shape = planar_shape(h->tile, h->precision);
     if (shape < 0) return fail(XC_ERR_UNSUPPORTED, "hi/lo operands do not run on XC_TILE_WIDE");
     e = xc::launch_planar(im, X, shape, s);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core X-engine launch");
@@ -745,8 +744,7 @@ xc_status xc_set_option(xc_handle* h, int key, long long value) {
       if (value == XC_TILE_SMALL && h->batch)
         return fail(XC_ERR_UNSUPPORTED, "batched launches run on the planar engine");
       if (h->batch) {
-        h->batch->shape = value == XC_TILE_AUTO ? h->batch->shape_default
-                                                : planar_shape(static_cast<int>(value), h->pg, XC_CI8, XC_PREC_FP16);
+        h->batch->shape = planar_shape(static_cast<int>(value), XC_PREC_FP16);
         batch_drop_graph(h->batch);
       }
       h->tile = static_cast<int>(value);
@@ -1258,10 +1256,6 @@ xc_handle* xc_batch_create(int nsub, const int* nstation, const int* nfreq, cons
     b->order[i] = i;
   }
   b->depth = 1;
-  // The larger shape pays when some subarray has more than one block row.
-  for (int i = 0; i < nsub; ++i)
-    b->shape_default = std::max(b->shape_default, xc::planar_default_shape(b->sub[i].pg, XC_CI8, XC_PREC_FP16));
-  b->shape = b->shape_default;
   succeed();
   return h;
 }

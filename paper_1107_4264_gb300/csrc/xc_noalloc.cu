@@ -216,7 +216,7 @@ extern "C" xc_status xc_correlate_noalloc(int nstation, int npol, int nfreq, int
   // Kernel parameter block on the stack: nothing is allocated, host or device.
   xc::PlanarKernel k;
   const CUtensorMap* maps[1] = {im};
-  cudaError_t e = xc::planar_prepare(&X, maps, 1, &k, xc::planar_default_shape(pg, in_dtype, XC_PREC_FP16));
+  cudaError_t e = xc::planar_prepare(&X, maps, 1, &k, xc::kPlanar128);
   if (e == cudaSuccess && k.grid > 0) e = xc::planar_setup(&X, 1, st);
   if (e == cudaSuccess) e = xc::planar_launch(k, st);
   if (e != cudaSuccess) {

@@ -13,6 +13,12 @@ namespace xc {
 // Tile shapes: 128 x 128 blocks on single CTAs, two blocks sharing a column
 // block on a CTA pair (tcgen05 cta_group::2), two blocks sharing a row block on
 // one CTA (N = 256 MMAs).
+// 128 x 128 is the one a call takes unless it asks for another.  128 x 256
+// items are faster for large arrays with long, quiet 8-bit integrations (512
+// stations x 2 pols, F=64, T=4096: 0.69 against 0.77 ms), but their
+// accumulators fill TMEM, so the MMAs stop for every drain of an exact chunk:
+// at |x| up to 80 there 2.89 against 0.93 ms, at full scale 5.16 against 1.14;
+// and how loud the samples are is not known at the launch.
 enum : int { kPlanar128 = 0, kPlanarPair = 1, kPlanarWide = 2 };
 constexpr int kPlanarBlk = 128;  // inputs per block
 // Samples per K-block and converter unit (8-bit input arrives by TMA in
@@ -68,18 +74,6 @@ inline PlanarRing planar_ring_whole(const Geometry& g, int fmt) {
   return planar_ring_of(g, fmt, g.Tp / kPlanarUnitT);
 }
 
-// 128 x 256 items for large arrays with long integrations, whose channels are
-// few and big: a quarter fewer operand bytes per MAC, and no more channels in
-// flight than the ring can feed.  Measured (8-bit input, ms, 128 x 128 / 128 x
-// 256): N=1024 F=16 T=8192 1.39 / 1.23, N=512 F=64 T=4096 0.81 / 0.71, N=256
-// F=64 T=8192 0.59 / 0.60, N=384 F=256 T=2048 0.96 / 0.95, N=1024 F=32 T=1000
-// 0.41 / 0.40, N=256 F=1024 T=1000 0.98 / 1.01.  Float input, whose converters
-// set the pace, stays with 128 x 128 (N=512 F=60 T=2048 0.75 / 0.87).
-inline int planar_default_shape(const Geometry& g, int in_dtype, int fmt) {
-  const int64_t nib = (static_cast<int64_t>(g.N) * g.P + kPlanarBlk - 1) / kPlanarBlk;
-  return in_dtype == 0 && fmt == XC_PREC_FP16 && nib >= 8 && g.Tp >= 4096 ? kPlanarWide : kPlanar128;
-}
-
 // Segments of at most 8 K-blocks (512 samples; half as many with hi/lo
 // operands, which take twice the bytes) and 60 MiB of ring, so that it stays
 // in the 129 MB L2 beside the streams.  Measured (8-bit input, ms):
@@ -93,8 +87,7 @@ inline int planar_default_shape(const Geometry& g, int in_dtype, int fmt) {
 //     N=256 F=64   T=8192          0.671         0.604   0.605   0.602
 //     N=512 F=64   T=4096          0.809         0.822   0.830   0.824
 // So 90 MiB when the channels of a wave take more than 80 MiB (8-bit input:
-// the float converters are too slow to fill it), and 120 MiB on 128 x 256
-// items (N=512 F=64 T=4096 0.708 against 0.777 ms).
+// the float converters are too slow to fill it).
 inline PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid) {
   const int seg = fmt == XC_PREC_HILO ? 4 : 8;
   const int nkb = g.Tp / kPlanarUnitT;
@@ -104,7 +97,6 @@ inline PlanarRing planar_ring(const Geometry& g, int in_dtype, int fmt, int grid
   const int64_t wave = std::max<int64_t>(1, grid / (nib * (nib + 1) / 2));
   int64_t mib = 60;
   if (in_dtype == 0 && wave * r.nseg * r.slot_bytes > (80ll << 20)) mib = 90;
-  if (planar_default_shape(g, in_dtype, fmt) == kPlanarWide) mib = 120;
   int64_t n = std::min<int64_t>((mib << 20) / r.slot_bytes, kMaxRingSlots);
   n = std::max<int64_t>(n, std::max<int64_t>(4, r.nseg + 4));
   r.slots = static_cast<int>(std::min<int64_t>(n, static_cast<int64_t>(g.F) * r.nseg));

@@ -85,7 +85,7 @@ int main(int argc, char** argv) {
   // grid shape fmt float_chunk rule nsub {N P F T loud slots}
   int a = 1;
   auto next = [&]() { return std::atoi(argv[a++]); };
-  int grid = next(); int shape = next(); const int fmt = next(), fchunk = next(), rule = next(), nsub = next();
+  int grid = next(); const int shape = next(), fmt = next(), fchunk = next(), rule = next(), nsub = next();
   const bool ints = fchunk == 0;
   std::vector<Sub> subs(nsub);
   for (Sub& s : subs) {
@@ -98,7 +98,6 @@ int main(int argc, char** argv) {
     s.r = planar_ring(s.g, ints ? 0 : 2, fmt, grid);
     if (slots > 0) s.r.slots = std::min(s.r.slots, std::max(slots, s.r.nseg));
     if (slots < 0) { s.r = planar_ring_whole(s.g, fmt); }
-    if (shape < 0) shape = planar_default_shape(s.g, ints ? 0 : 2, fmt);
     const int n = s.g.N * s.g.P;
     s.nib = (n + kPlanarBlk - 1) / kPlanarBlk;
     s.nkb = s.g.Tp / 64;
@@ -255,7 +254,7 @@ int main(int argc, char** argv) {
 }
 """
 FP16, HILO, FP8 = 0, 1, 2
-AUTO, S128, PAIR, WIDE = -1, 0, 1, 2
+S128, PAIR, WIDE = 0, 1, 2
 
 
 @pytest.fixture(scope="module")
@@ -270,7 +269,7 @@ def model(tmp_path_factory):
     subprocess.run([gxx, "-std=c++17", "-O2", "-I", CSRC, "-I", os.path.join(ROOT, "include"), str(src), "-o",
                     str(exe)], check=True)
 
-    def run(subs, shape=AUTO, fmt=FP16, fchunk=0, whole_channel=False, grid=152):
+    def run(subs, shape=S128, fmt=FP16, fchunk=0, whole_channel=False, grid=152):
         args = [grid, shape, fmt, fchunk, int(whole_channel), len(subs)] + [v for s in subs for v in s]
         return subprocess.run([str(exe)] + [str(v) for v in args], check=True, capture_output=True,
                               text=True).stdout.strip()
@@ -281,7 +280,7 @@ def model(tmp_path_factory):
 # exact chunks (one on 128 x 256 items) leave unread.
 STALLS = [(72, 2, 64, 3584, 128, S128), (100, 2, 64, 9216, 50, S128), (160, 2, 64, 4096, 128, S128),
           (256, 2, 64, 4608, 128, S128), (256, 2, 64, 10240, 50, PAIR), (300, 2, 64, 7168, 80, S128),
-          (512, 2, 64, 5632, 80, WIDE), (128, 2, 256, 4096, 128, AUTO), (256, 2, 64, 8192, -128, S128)]
+          (512, 2, 64, 5632, 80, WIDE), (128, 2, 256, 4096, 128, S128), (256, 2, 64, 8192, -128, S128)]
 
 
 @pytest.mark.parametrize("size", STALLS, ids=lambda s: "N%d_P%d_F%d_T%d_m%d_shape%d" % s)
@@ -296,9 +295,9 @@ def test_random_sizes_never_stall(model):
     batches; 152 SMs and fewer."""
     rng = random.Random(11)
     for i in range(60):
-        shape = rng.choice([AUTO, S128, PAIR, WIDE])
+        shape = rng.choice([S128, S128, PAIR, WIDE])
         ints = rng.random() < 0.75
-        fmt = rng.choice([FP16, FP16, FP8] if ints else ([FP16, HILO] if shape in (AUTO, S128, PAIR) else [FP16]))
+        fmt = rng.choice([FP16, FP16, FP8] if ints else ([FP16, HILO] if shape != WIDE else [FP16]))
         subs = []
         for _ in range(rng.choice([1, 1, 3]) if ints and fmt == FP16 else 1):
             N, P = rng.choice([3, 40, 65, 100, 160, 256, 449, 700]), rng.choice([1, 2])
