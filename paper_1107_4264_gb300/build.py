@@ -23,7 +23,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libxc.so")
 
-SOURCES = ["xc_api.cpp", "xc_form.cu", "xc_tc.cu", "xc_fp32.cu", "xc_noalloc.cu", "xc_xengine.cu", "xc_xengine2.cu", "xc_planar.cu", "xc_planar_pair.cu", "xc_planar_wide.cu", "xc_small.cu", "xc_adjoint.cu", "xc_adjoint_tc.cu", "xc_fengine.cu"]
+SOURCES = ["xc_api.cpp", "xc_form.cu", "xc_tc.cu", "xc_fp32.cu", "xc_noalloc.cu", "xc_xengine.cu", "xc_xengine2.cu", "xc_planar.cu", "xc_planar_pair.cu", "xc_planar_wide.cu", "xc_planar_words.cu", "xc_small.cu", "xc_adjoint.cu", "xc_adjoint_tc.cu", "xc_fengine.cu"]
 HEADERS = ["xc_internal.h", "xc_planar_plan.h", "xc_launch.h", "xc_ptx.cuh", "xc_convert.cuh", "xc_planar_kernel.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -35,12 +35,13 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def _flags(verbose: bool):
-    f = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
-                "--expt-relaxed-constexpr"]
-    if verbose:
-        f += ["-Xptxas", "-v"]
-    return f
+FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
+                "--expt-relaxed-constexpr", "-Xptxas", "-v"]
+
+
+def ptxas_log(src: str) -> str:
+    """Where build() keeps what ptxas says of a source's kernels (registers, spills, shared memory)."""
+    return os.path.join(BUILD, "obj", src + ".log")
 
 
 def _deps_mtime() -> float:
@@ -55,14 +56,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(os.path.join(BUILD, "obj"), exist_ok=True)
     cc = nvcc()
-    flags = _flags(verbose)
 
     def compile_one(src):
         obj = os.path.join(BUILD, "obj", src + ".o")
-        cmd = [cc] + flags + ["-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [cc] + FLAGS + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
+        with open(ptxas_log(src), "w") as fh:
+            fh.write(r.stderr)
         if verbose and (r.stdout or r.stderr):
             sys.stderr.write(r.stdout + r.stderr)
         return obj

@@ -11,6 +11,8 @@ namespace xc {
 // xc_planar_wide.cu (compiled in parallel with this file).
 const void* planar_pair_select(int in_dtype, int fmt, bool multi);
 const void* planar_wide_select(int in_dtype, int fmt, bool multi);
+// 8-bit rows that TMA cannot stride, every shape (xc_planar_words.cu).
+const void* planar_words_select(int shape, int fmt, bool multi);
 
 static_assert(kShape128 == kPlanar128 && kShapePair == kPlanarPair && kShapeWide == kPlanarWide,
               "tile shape codes");
@@ -21,7 +23,7 @@ namespace {
 
 template <bool IS_INT, int DT, int FMT, bool MULTI = false>
 const void* kernel_of() {
-  return reinterpret_cast<const void*>(planar_kernel<IS_INT, DT, FMT, MULTI>);
+  return reinterpret_cast<const void*>(planar_kernel<IS_INT, DT, FMT, MULTI, IS_INT ? kInTma : kInFloat>);
 }
 
 // Batches of several subarrays take 8-bit input.
@@ -191,7 +193,9 @@ cudaError_t planar_prepare(const XeLaunch* subs, const CUtensorMap* const* maps,
   for (int i = 0; i < nsub; ++i) b->sub[i].tma_in = all_tma ? 1 : 0;
   const int conv = (fmt == kFmtF8 && dt == 0) ? conv_warps<kFmtF8, 0>() : conv_warps<kFmtF16, 0>();
   const bool pair = shape == kShapePair;
-  switch (shape) {
+  const bool words = dt == 0 && !all_tma;
+  switch (words ? -1 : shape) {
+    case -1: k->func = planar_words_select(shape, fmt, nsub > 1); break;
     case kShape128: k->func = select_kernel(dt, fmt, nsub > 1); break;
     case kShapePair: k->func = planar_pair_select(dt, fmt, nsub > 1); break;
     case kShapeWide: k->func = planar_wide_select(dt, fmt, nsub > 1); break;

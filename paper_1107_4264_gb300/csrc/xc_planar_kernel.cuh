@@ -473,6 +473,12 @@ __device__ __forceinline__ unsigned kblock_growth(const Params& p, int G) {
 
 // -------------------------------------------------------------- converter
 
+// How a kernel's converters read their input: 8-bit in TMA boxes, 8-bit in words
+// (rows that TMA cannot stride), or float (either way).  One 8-bit form per
+// kernel: with both in one, the words' 64 registers spill in the kernel whose
+// input is aligned too (288 bytes of stores, none without them).
+enum : int { kInTma = 0, kInWords = 1, kInFloat = 2 };
+
 // fp16x2 of (component j of sample a, component j of sample b), 8-bit input.
 __device__ __forceinline__ uint32_t pair_i8(uint32_t a, uint32_t b, uint32_t j) {
   // Byte j of a into byte 0 and byte j of b into byte 2; 0x6400 | (x ^ 0x80)
@@ -804,6 +810,96 @@ __device__ __forceinline__ void drain_tma(uint32_t bar, uint32_t phase, bool pen
   __syncwarp();
 }
 
+// Where a converter warp's 8-bit words of one unit go, and the largest |x| among
+// them.  A word is (re, im) of the lane's inputs 2l and 2l + 1 at one sample; a
+// chunk (8 samples in fp16, 16 in e4m3) of them makes tile rows 2l and 2l + 1 of
+// both planes, 32 contiguous bytes each, so a warp store covers 1 KiB.
+template <int FMT, int SHAPE>
+struct WordSink {
+  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
+  uint8_t* tre;
+  uint8_t* tim;
+  int row;
+  // Ring tiles are read back by every block of the channel: keep them in L2.
+  uint64_t pol;
+  __half2 mx[2];  // fp16: from the converted (exact) values
+  uint32_t mb;    // e4m3: per byte
+
+  __device__ __forceinline__ WordSink(const Params& p, const Unit& x, int lane, uint64_t pol_last) {
+    tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, x.hb >> 1);
+    tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, x.hb >> 1);
+    row = (x.hb & 1) * 64 + 2 * lane;
+    pol = pol_last;
+    mx[0] = mx[1] = __float2half2_rn(0.f);
+    mb = 0;
+  }
+  // Rows 2l and 2l + 1 of one plane: bytes j and j + 2 of the words.
+  __device__ __forceinline__ void store8(uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq) {
+    uint32_t v[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
+      v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; k += 2)
+      mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
+                               __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
+    ptx::st_global_v8_hint(dst, v, pol);
+  }
+  // Component j of four consecutive samples as four e4m3 bytes: the exact fp16
+  // pair conversion, then one fp16x2 -> e4m3x2 conversion per pair (exact for
+  // |x| <= 16; a larger value sets the range status bit).
+  static __device__ __forceinline__ uint32_t cvt4(const uint32_t* W, uint32_t j) {
+    const uint32_t h01 = pair_i8(W[0], W[1], j), h23 = pair_i8(W[2], W[3], j);
+    __half2_raw r01, r23;
+    r01.x = static_cast<unsigned short>(h01 & 0xffffu);
+    r01.y = static_cast<unsigned short>(h01 >> 16);
+    r23.x = static_cast<unsigned short>(h23 & 0xffffu);
+    r23.y = static_cast<unsigned short>(h23 >> 16);
+    const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
+    const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
+    return (e01 & 0xffffu) | (e23 << 16);
+  }
+  // Chunk cc from its words.
+  __device__ __forceinline__ void put(int cc, const uint32_t* W) {
+    const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+    if constexpr (FMT == kFmtF16) {
+      store8(tre + off, W, 0u, mx[0]);
+      store8(tim + off, W, 1u, mx[1]);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
+      uint32_t vr[8], vi[8];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        vr[k] = cvt4(W + 4 * k, 0);
+        vi[k] = cvt4(W + 4 * k, 1);
+        vr[4 + k] = cvt4(W + 4 * k, 2);
+        vi[4 + k] = cvt4(W + 4 * k, 3);
+      }
+      ptx::st_global_v8_hint(tre + off, vr, pol);
+      ptx::st_global_v8_hint(tim + off, vi, pol);
+    }
+  }
+  // Record the unit's maximum (the whole warp; rows and samples past the end
+  // are zero).
+  __device__ __forceinline__ void finish(const Params& p, const Unit& x, int lane) const {
+    unsigned m;
+    if constexpr (FMT == kFmtF16) {
+      const __half2 mm = __hmax2(mx[0], mx[1]);
+      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
+    } else {
+      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) {
+      atomicMax(p.amax + x.G, m);
+      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
+    }
+  }
+};
+
 // 8-bit converter with TMA-staged input.  Each converter warp is an
 // independent worker on its own stream of units (u = global warp id + k *
 // warps, channel-major), with an 8 KiB staging buffer ([64 samples][128
@@ -817,7 +913,8 @@ __device__ __forceinline__ void drain_tma(uint32_t bar, uint32_t phase, bool pen
 template <int FMT, bool MULTI, int SHAPE>
 __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int cw, int lane,
                               volatile int* abort_flag) {
-  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
+  constexpr int kChunkT = FMT == kFmtF8 ? 16 : 8;  // samples per 16-byte chunk
+  const uint64_t pol_last = ptx::l2_policy_evict_last();
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
@@ -834,9 +931,7 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
   };
   const uint32_t* src = reinterpret_cast<const uint32_t*>(__cvta_shared_to_generic(static_cast<size_t>(buf)));
   // Lane l converts inputs 2l and 2l + 1 of the half block: word l of each
-  // 128-byte sample row holds (re, im) of both.  Per 8-sample chunk and plane
-  // the lane writes tile rows 2l and 2l + 1 (32 contiguous bytes), so a warp
-  // store covers 1 KiB.
+  // 128-byte sample row holds (re, im) of both.
   uint32_t phase = 0;
   int claimed = -1, claimed_sb = -1;
   // Converted units of a run not yet published: their subarray, slot, run, count.
@@ -883,83 +978,10 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
-    const int ib = x.hb >> 1;
-    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
-    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
-    const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
-    // Ring tiles are read back by every block of the channel: keep them in L2.
-    const uint64_t pol_last = ptx::l2_policy_evict_last();
-    unsigned m = 0;  // max |x| over the unit (zero-filled rows and samples contribute 0)
-    if constexpr (FMT == kFmtF16) {
-      // max |x| from the converted (exact) fp16 values.
-      __half2 mx[2];
+    WordSink<FMT, SHAPE> sink(p, x, lane, pol_last);
 #pragma unroll
-      for (int q = 0; q < 2; ++q) mx[q] = __float2half2_rn(0.f);
-      // Rows 2l and 2l + 1 of one plane: bytes j and j + 2 of the words.
-      auto store8 = [&](uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq) {
-        uint32_t v[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
-          v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; k += 2)
-          mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
-                                   __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
-        ptx::st_global_v8_hint(dst, v, pol_last);
-      };
-#pragma unroll
-      for (int cc = 0; cc < kUnitT / 8; ++cc) {
-        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-        store8(tre + off, w + 8 * cc, 0u, mx[0]);
-        store8(tim + off, w + 8 * cc, 1u, mx[1]);
-      }
-      const __half2 mm = __hmax2(mx[0], mx[1]);
-      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
-    } else {
-      // e4m3 operands: exact for |x| <= 16 (a larger value sets the range
-      // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
-      uint32_t mb = 0;  // per-byte |x| maximum
-#pragma unroll
-      for (int t = 0; t < kUnitT; ++t) mb = __vmaxu4(mb, __vabs4(w[t]));
-      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
-      // Component j of four consecutive samples as four e4m3 bytes: the
-      // exact fp16 pair conversion of the fp16 path, then one fp16x2 ->
-      // e4m3x2 conversion per pair (exact for |x| <= 16).
-      auto cvt4 = [](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t j) {
-        const uint32_t h01 = pair_i8(w0, w1, j), h23 = pair_i8(w2, w3, j);
-        __half2_raw r01, r23;
-        r01.x = static_cast<unsigned short>(h01 & 0xffffu);
-        r01.y = static_cast<unsigned short>(h01 >> 16);
-        r23.x = static_cast<unsigned short>(h23 & 0xffffu);
-        r23.y = static_cast<unsigned short>(h23 >> 16);
-        const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
-        const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
-        return (e01 & 0xffffu) | (e23 << 16);
-      };
-#pragma unroll
-      for (int cc = 0; cc < kUnitT / 16; ++cc) {
-        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-        const uint32_t* W = w + 16 * cc;
-        uint32_t vr[8], vi[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          vr[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 0);
-          vi[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 1);
-          vr[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 2);
-          vi[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 3);
-        }
-        ptx::st_global_v8_hint(tre + off, vr, pol_last);
-        ptx::st_global_v8_hint(tim + off, vi, pol_last);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) {
-      atomicMax(p.amax + x.G, m);
-      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
-    }
+    for (int cc = 0; cc < kUnitT / kChunkT; ++cc) sink.put(cc, w + kChunkT * cc);
+    sink.finish(p, x, lane);
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
@@ -991,12 +1013,10 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
 // segment may need that run).
 template <int FMT, bool MULTI, int SHAPE, bool EVEN>
 __device__ void converter_words(const Batch& bt, int cw, int lane, volatile int* abort_flag) {
-  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
   // The input streams through once: first in line for L2 replacement, so the
-  // operand ring it is converted into stays resident.  Ring tiles are read
-  // back by every block of the channel: keep them in L2.
+  // operand ring it is converted into stays resident.
   const uint64_t pol_first = ptx::l2_policy_evict_first(), pol_last = ptx::l2_policy_evict_last();
   // Where a unit's words come from: this lane's word of sample 0, the bytes
   // from sample to sample, and the samples to load (0: no such input).
@@ -1077,92 +1097,23 @@ __device__ void converter_words(const Batch& bt, int cw, int lane, volatile int*
       else
         load8(ns, cc + kRing - kBK / 8);
     };
-    const int ib = x.hb >> 1;
-    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
-    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
-    const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
     // A finished run is published now: its last stores have had some time.
     if (pend && pend_run != x.u / p.run) {
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
-    unsigned m = 0;  // max |x| over the unit (rows and samples past the end contribute 0)
-    if constexpr (FMT == kFmtF16) {
-      // max |x| from the converted (exact) fp16 values.
-      __half2 mx[2];
+    WordSink<FMT, SHAPE> sink(p, x, lane, pol_last);
+    constexpr int kLoads = FMT == kFmtF8 ? 2 : 1;  // 8-sample loads per 16-byte chunk
 #pragma unroll
-      for (int q = 0; q < 2; ++q) mx[q] = __float2half2_rn(0.f);
-      // Rows 2l and 2l + 1 of one plane: bytes j and j + 2 of the words.
-      auto store8 = [&](uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq) {
-        uint32_t v[8];
+    for (int cc = 0; cc < kBK / 8; cc += kLoads) {
+      uint32_t W[8 * kLoads];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
-          v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
-        }
+      for (int h = 0; h < kLoads; ++h) words8(cc + h, W + 8 * h);
+      sink.put(cc / kLoads, W);
 #pragma unroll
-        for (int k = 0; k < 8; k += 2)
-          mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
-                                   __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
-        ptx::st_global_v8_hint(dst, v, pol_last);
-      };
-#pragma unroll
-      for (int cc = 0; cc < kBK / 8; ++cc) {
-        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-        uint32_t W[8];
-        words8(cc, W);
-        store8(tre + off, W, 0u, mx[0]);
-        store8(tim + off, W, 1u, mx[1]);
-        reload(cc);
-      }
-      const __half2 mm = __hmax2(mx[0], mx[1]);
-      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
-    } else {
-      // e4m3 operands: exact for |x| <= 16 (a larger value sets the range
-      // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
-      uint32_t mb = 0;  // per-byte |x| maximum
-      // Component j of four consecutive samples as four e4m3 bytes: the
-      // exact fp16 pair conversion of the fp16 path, then one fp16x2 ->
-      // e4m3x2 conversion per pair (exact for |x| <= 16).
-      auto cvt4 = [](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t j) {
-        const uint32_t h01 = pair_i8(w0, w1, j), h23 = pair_i8(w2, w3, j);
-        __half2_raw r01, r23;
-        r01.x = static_cast<unsigned short>(h01 & 0xffffu);
-        r01.y = static_cast<unsigned short>(h01 >> 16);
-        r23.x = static_cast<unsigned short>(h23 & 0xffffu);
-        r23.y = static_cast<unsigned short>(h23 >> 16);
-        const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
-        const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
-        return (e01 & 0xffffu) | (e23 << 16);
-      };
-#pragma unroll
-      for (int cc = 0; cc < kBK / 16; ++cc) {
-        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-        uint32_t W[16];
-        words8(2 * cc, W);
-        words8(2 * cc + 1, W + 8);
-#pragma unroll
-        for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
-        uint32_t vr[8], vi[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          vr[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 0);
-          vi[k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 1);
-          vr[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 2);
-          vi[4 + k] = cvt4(W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3], 3);
-        }
-        ptx::st_global_v8_hint(tre + off, vr, pol_last);
-        ptx::st_global_v8_hint(tim + off, vi, pol_last);
-        reload(2 * cc);
-        reload(2 * cc + 1);
-      }
-      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
+      for (int h = 0; h < kLoads; ++h) reload(cc + h);
     }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) {
-      atomicMax(p.amax + x.G, m);
-      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
-    }
+    sink.finish(p, x, lane);
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
@@ -1781,7 +1732,7 @@ __device__ __forceinline__ long long item_stride() {
   return SHAPE == kShapePair ? static_cast<long long>(gridDim.x >> 1) : static_cast<long long>(gridDim.x);
 }
 
-template <bool IS_INT, int DT, int FMT, bool MULTI, int SHAPE>
+template <bool IS_INT, int DT, int FMT, bool MULTI, int SHAPE, int IN>
 __device__ __forceinline__ void planar_body(const Batch& bt) {
   constexpr bool PAIR = SHAPE == kShapePair;
   constexpr bool WIDE = SHAPE == kShapeWide;
@@ -2458,17 +2409,16 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
     // ---------------------------------------------------------- converters
     const int cw = warp - (2 + kNumEpiWarps);
     const uint32_t cbuf = sbase + C::kConvOff + cw * kConvBufBytes;
-    if constexpr (DT == 0) {
-      if (bt.sub[0].tma_in) {  // set for every subarray or for none
-        converter_tma<FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
-      } else {
-        bool even = true;
-        for (int i = 0; i < bt.nsub; ++i) even = even && bt.sub[i].n % 2 == 0;
-        if (even)
-          converter_words<FMT, MULTI, SHAPE, true>(bt, cw, lane, abort_flag);
-        else
-          converter_words<FMT, MULTI, SHAPE, false>(bt, cw, lane, abort_flag);
-      }
+    static_assert((DT == 0) == (IN != kInFloat), "input form of the type");
+    if constexpr (IN == kInTma) {
+      converter_tma<FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
+    } else if constexpr (IN == kInWords) {
+      bool even = true;
+      for (int i = 0; i < bt.nsub; ++i) even = even && bt.sub[i].n % 2 == 0;
+      if (even)
+        converter_words<FMT, MULTI, SHAPE, true>(bt, cw, lane, abort_flag);
+      else
+        converter_words<FMT, MULTI, SHAPE, false>(bt, cw, lane, abort_flag);
     } else {
       if (bt.sub[0].tma_in) {
         converter_tma_float<DT, FMT, MULTI, SHAPE>(bt, cbuf, conv_bar(cw), cw, lane, abort_flag);
@@ -2492,23 +2442,23 @@ __device__ __forceinline__ void planar_body(const Batch& bt) {
   }
 }
 
-template <bool IS_INT, int DT, int FMT, bool MULTI>
+template <bool IS_INT, int DT, int FMT, bool MULTI, int IN>
 __global__ void __launch_bounds__(threads_of<FMT, DT>(), 1) planar_kernel(const __grid_constant__ Batch bt) {
-  planar_body<IS_INT, DT, FMT, MULTI, kShape128>(bt);
+  planar_body<IS_INT, DT, FMT, MULTI, kShape128, IN>(bt);
 }
 
 // 128 x 256 items: one CTA, N = 256 MMAs.
-template <bool IS_INT, int DT, int FMT, bool MULTI>
+template <bool IS_INT, int DT, int FMT, bool MULTI, int IN>
 __global__ void __launch_bounds__(threads_of<FMT, DT>(), 1) planar_wide_kernel(const __grid_constant__ Batch bt) {
-  if constexpr (FMT != kFmtHiLo) planar_body<IS_INT, DT, FMT, MULTI, kShapeWide>(bt);
+  if constexpr (FMT != kFmtHiLo) planar_body<IS_INT, DT, FMT, MULTI, kShapeWide, IN>(bt);
 }
 
 // CTA pairs: the cluster shape is part of the kernel, so no launch can run it
 // without its peer.
-template <bool IS_INT, int DT, int FMT, bool MULTI>
+template <bool IS_INT, int DT, int FMT, bool MULTI, int IN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of<FMT, DT>(), 1)
     planar_pair_kernel(const __grid_constant__ Batch bt) {
-  planar_body<IS_INT, DT, FMT, MULTI, kShapePair>(bt);
+  planar_body<IS_INT, DT, FMT, MULTI, kShapePair, IN>(bt);
 }
 
 }  // namespace

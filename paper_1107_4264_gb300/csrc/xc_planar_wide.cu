@@ -9,7 +9,7 @@ namespace {
 
 template <bool IS_INT, int DT, int FMT, bool MULTI = false>
 const void* wide_kernel_of() {
-  return reinterpret_cast<const void*>(planar_wide_kernel<IS_INT, DT, FMT, MULTI>);
+  return reinterpret_cast<const void*>(planar_wide_kernel<IS_INT, DT, FMT, MULTI, IS_INT ? kInTma : kInFloat>);
 }
 
 }  // namespace
