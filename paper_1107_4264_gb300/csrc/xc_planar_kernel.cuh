@@ -810,95 +810,50 @@ __device__ __forceinline__ void drain_tma(uint32_t bar, uint32_t phase, bool pen
   __syncwarp();
 }
 
-// Where a converter warp's 8-bit words of one unit go, and the largest |x| among
-// them.  A word is (re, im) of the lane's inputs 2l and 2l + 1 at one sample; a
-// chunk (8 samples in fp16, 16 in e4m3) of them makes tile rows 2l and 2l + 1 of
-// both planes, 32 contiguous bytes each, so a warp store covers 1 KiB.
-template <int FMT, int SHAPE>
-struct WordSink {
-  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
-  uint8_t* tre;
-  uint8_t* tim;
-  int row;
-  // Ring tiles are read back by every block of the channel: keep them in L2.
-  uint64_t pol;
-  __half2 mx[2];  // fp16: from the converted (exact) values
-  uint32_t mb;    // e4m3: per byte
-
-  __device__ __forceinline__ WordSink(const Params& p, const Unit& x, int lane, uint64_t pol_last) {
-    tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, x.hb >> 1);
-    tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, x.hb >> 1);
-    row = (x.hb & 1) * 64 + 2 * lane;
-    pol = pol_last;
-    mx[0] = mx[1] = __float2half2_rn(0.f);
-    mb = 0;
-  }
-  // Rows 2l and 2l + 1 of one plane: bytes j and j + 2 of the words.
-  __device__ __forceinline__ void store8(uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq) {
-    uint32_t v[8];
+// 8-bit words to operands.  A word is (re, im) of a lane's two inputs, tile rows
+// 2l and 2l + 1, at one sample; the words of a 16-byte chunk (8 samples in fp16,
+// 16 in e4m3) make 32 contiguous bytes of a plane, so a warp store covers 1 KiB.
+// fp16, one plane (j: 0 re, 1 im), with the largest |x| of each half of `mq`.
+__device__ __forceinline__ void store_rows_f16(uint8_t* dst, const uint32_t* W, uint32_t j, __half2& mq, uint64_t pol) {
+  uint32_t v[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
-      v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
-    }
+  for (int k = 0; k < 4; ++k) {
+    v[k] = pair_i8(W[2 * k], W[2 * k + 1], j);
+    v[4 + k] = pair_i8(W[2 * k], W[2 * k + 1], j + 2);
+  }
 #pragma unroll
-    for (int k = 0; k < 8; k += 2)
-      mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
-                               __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
-    ptx::st_global_v8_hint(dst, v, pol);
-  }
-  // Component j of four consecutive samples as four e4m3 bytes: the exact fp16
-  // pair conversion, then one fp16x2 -> e4m3x2 conversion per pair (exact for
-  // |x| <= 16; a larger value sets the range status bit).
-  static __device__ __forceinline__ uint32_t cvt4(const uint32_t* W, uint32_t j) {
-    const uint32_t h01 = pair_i8(W[0], W[1], j), h23 = pair_i8(W[2], W[3], j);
-    __half2_raw r01, r23;
-    r01.x = static_cast<unsigned short>(h01 & 0xffffu);
-    r01.y = static_cast<unsigned short>(h01 >> 16);
-    r23.x = static_cast<unsigned short>(h23 & 0xffffu);
-    r23.y = static_cast<unsigned short>(h23 >> 16);
-    const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
-    const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
-    return (e01 & 0xffffu) | (e23 << 16);
-  }
-  // Chunk cc from its words.
-  __device__ __forceinline__ void put(int cc, const uint32_t* W) {
-    const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-    if constexpr (FMT == kFmtF16) {
-      store8(tre + off, W, 0u, mx[0]);
-      store8(tim + off, W, 1u, mx[1]);
-    } else {
+  for (int k = 0; k < 8; k += 2)
+    mq = __hmax2(mq, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&v[k])),
+                             __habs2(*reinterpret_cast<const __half2*>(&v[k + 1]))));
+  ptx::st_global_v8_hint(dst, v, pol);
+}
+// Component j of four consecutive samples as four e4m3 bytes: the exact fp16
+// pair conversion, then one fp16x2 -> e4m3x2 conversion per pair (exact for
+// |x| <= 16).
+__device__ __forceinline__ uint32_t quad_f8(const uint32_t* W, uint32_t j) {
+  const uint32_t h01 = pair_i8(W[0], W[1], j), h23 = pair_i8(W[2], W[3], j);
+  __half2_raw r01, r23;
+  r01.x = static_cast<unsigned short>(h01 & 0xffffu);
+  r01.y = static_cast<unsigned short>(h01 >> 16);
+  r23.x = static_cast<unsigned short>(h23 & 0xffffu);
+  r23.y = static_cast<unsigned short>(h23 >> 16);
+  const uint32_t e01 = __nv_cvt_halfraw2_to_fp8x2(r01, __NV_SATFINITE, __NV_E4M3);
+  const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
+  return (e01 & 0xffffu) | (e23 << 16);
+}
+// e4m3, both planes.
+__device__ __forceinline__ void store_rows_f8(uint8_t* re, uint8_t* im, const uint32_t* W, uint64_t pol) {
+  uint32_t vr[8], vi[8];
 #pragma unroll
-      for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
-      uint32_t vr[8], vi[8];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        vr[k] = cvt4(W + 4 * k, 0);
-        vi[k] = cvt4(W + 4 * k, 1);
-        vr[4 + k] = cvt4(W + 4 * k, 2);
-        vi[4 + k] = cvt4(W + 4 * k, 3);
-      }
-      ptx::st_global_v8_hint(tre + off, vr, pol);
-      ptx::st_global_v8_hint(tim + off, vi, pol);
-    }
+  for (int k = 0; k < 4; ++k) {
+    vr[k] = quad_f8(W + 4 * k, 0);
+    vi[k] = quad_f8(W + 4 * k, 1);
+    vr[4 + k] = quad_f8(W + 4 * k, 2);
+    vi[4 + k] = quad_f8(W + 4 * k, 3);
   }
-  // Record the unit's maximum (the whole warp; rows and samples past the end
-  // are zero).
-  __device__ __forceinline__ void finish(const Params& p, const Unit& x, int lane) const {
-    unsigned m;
-    if constexpr (FMT == kFmtF16) {
-      const __half2 mm = __hmax2(mx[0], mx[1]);
-      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
-    } else {
-      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) {
-      atomicMax(p.amax + x.G, m);
-      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
-    }
-  }
-};
+  ptx::st_global_v8_hint(re, vr, pol);
+  ptx::st_global_v8_hint(im, vi, pol);
+}
 
 // 8-bit converter with TMA-staged input.  Each converter warp is an
 // independent worker on its own stream of units (u = global warp id + k *
@@ -913,8 +868,7 @@ struct WordSink {
 template <int FMT, bool MULTI, int SHAPE>
 __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int cw, int lane,
                               volatile int* abort_flag) {
-  constexpr int kChunkT = FMT == kFmtF8 ? 16 : 8;  // samples per 16-byte chunk
-  const uint64_t pol_last = ptx::l2_policy_evict_last();
+  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
   const ptx::WaitCtl wc{bt.sub[0].timeout_ns, bt.sub[0].status, abort_flag};
@@ -931,7 +885,9 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
   };
   const uint32_t* src = reinterpret_cast<const uint32_t*>(__cvta_shared_to_generic(static_cast<size_t>(buf)));
   // Lane l converts inputs 2l and 2l + 1 of the half block: word l of each
-  // 128-byte sample row holds (re, im) of both.
+  // 128-byte sample row holds (re, im) of both.  Per 8-sample chunk and plane
+  // the lane writes tile rows 2l and 2l + 1 (32 contiguous bytes), so a warp
+  // store covers 1 KiB.
   uint32_t phase = 0;
   int claimed = -1, claimed_sb = -1;
   // Converted units of a run not yet published: their subarray, slot, run, count.
@@ -978,10 +934,46 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
-    WordSink<FMT, SHAPE> sink(p, x, lane, pol_last);
+    const int ib = x.hb >> 1;
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
+    const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
+    // Ring tiles are read back by every block of the channel: keep them in L2.
+    const uint64_t pol_last = ptx::l2_policy_evict_last();
+    unsigned m = 0;  // max |x| over the unit (zero-filled rows and samples contribute 0)
+    if constexpr (FMT == kFmtF16) {
+      // max |x| from the converted (exact) fp16 values.
+      __half2 mx[2];
 #pragma unroll
-    for (int cc = 0; cc < kUnitT / kChunkT; ++cc) sink.put(cc, w + kChunkT * cc);
-    sink.finish(p, x, lane);
+      for (int q = 0; q < 2; ++q) mx[q] = __float2half2_rn(0.f);
+#pragma unroll
+      for (int cc = 0; cc < kUnitT / 8; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        store_rows_f16(tre + off, w + 8 * cc, 0u, mx[0], pol_last);
+        store_rows_f16(tim + off, w + 8 * cc, 1u, mx[1], pol_last);
+      }
+      const __half2 mm = __hmax2(mx[0], mx[1]);
+      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
+    } else {
+      // e4m3 operands: exact for |x| <= 16 (a larger value sets the range
+      // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
+      uint32_t mb = 0;  // per-byte |x| maximum
+#pragma unroll
+      for (int t = 0; t < kUnitT; ++t) mb = __vmaxu4(mb, __vabs4(w[t]));
+      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
+#pragma unroll
+      for (int cc = 0; cc < kUnitT / 16; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        const uint32_t* W = w + 16 * cc;
+        store_rows_f8(tre + off, tim + off, W, pol_last);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+      atomicMax(p.amax + x.G, m);
+      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
+    }
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
@@ -1006,17 +998,19 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
 // 32), which so have that long to arrive.  (On rows that TMA can stride this is
 // the slower one: 256 stations x 2 pols, F=1024, T=1000 1.16 against 1.03 ms.)
 // Measured against converting single components by way of floats, for any row:
-// 37 stations x 2 pols, F=2048, T=1000 1742 -> 451 us; 131 stations x 1 pol,
-// F=300, T=500 270 -> 175 us.
+// 37 stations x 2 pols, F=2048, T=1000 1741 -> 440 us; 131 stations x 1 pol,
+// F=300, T=500 271 -> 140 us.
 // A warp publishes each run at the start of the run after it; a warp that would
 // have to wait for a slot publishes first (a consumer of the slot's previous
 // segment may need that run).
 template <int FMT, bool MULTI, int SHAPE, bool EVEN>
 __device__ void converter_words(const Batch& bt, int cw, int lane, volatile int* abort_flag) {
+  static_assert(FMT == kFmtF16 || FMT == kFmtF8, "8-bit input: fp16 or e4m3 operands");
   const long long total = table_end<MULTI>(bt.unit_base, bt.nsub);
   const long long nw = static_cast<long long>(gridDim.x) * conv_warps<FMT, 0>();
   // The input streams through once: first in line for L2 replacement, so the
-  // operand ring it is converted into stays resident.
+  // operand ring it is converted into stays resident.  Ring tiles are read
+  // back by every block of the channel: keep them in L2.
   const uint64_t pol_first = ptx::l2_policy_evict_first(), pol_last = ptx::l2_policy_evict_last();
   // Where a unit's words come from: this lane's word of sample 0, the bytes
   // from sample to sample, and the samples to load (0: no such input).
@@ -1097,23 +1091,55 @@ __device__ void converter_words(const Batch& bt, int cw, int lane, volatile int*
       else
         load8(ns, cc + kRing - kBK / 8);
     };
+    const int ib = x.hb >> 1;
+    uint8_t* tre = ring_tile<FMT, SHAPE>(p, x.slot, 0, x.k, ib);
+    uint8_t* tim = ring_tile<FMT, SHAPE>(p, x.slot, 1, x.k, ib);
+    const int row = (x.hb & 1) * 64 + 2 * lane;  // tile rows 2l and 2l + 1
     // A finished run is published now: its last stores have had some time.
     if (pend && pend_run != x.u / p.run) {
       publish_unit(*pend, pend_slot, lane, pend_n);
       pend = nullptr;
     }
-    WordSink<FMT, SHAPE> sink(p, x, lane, pol_last);
-    constexpr int kLoads = FMT == kFmtF8 ? 2 : 1;  // 8-sample loads per 16-byte chunk
+    unsigned m = 0;  // max |x| over the unit (rows and samples past the end contribute 0)
+    if constexpr (FMT == kFmtF16) {
+      // max |x| from the converted (exact) fp16 values.
+      __half2 mx[2];
 #pragma unroll
-    for (int cc = 0; cc < kBK / 8; cc += kLoads) {
-      uint32_t W[8 * kLoads];
+      for (int q = 0; q < 2; ++q) mx[q] = __float2half2_rn(0.f);
 #pragma unroll
-      for (int h = 0; h < kLoads; ++h) words8(cc + h, W + 8 * h);
-      sink.put(cc / kLoads, W);
+      for (int cc = 0; cc < kBK / 8; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        uint32_t W[8];
+        words8(cc, W);
+        store_rows_f16(tre + off, W, 0u, mx[0], pol_last);
+        store_rows_f16(tim + off, W, 1u, mx[1], pol_last);
+        reload(cc);
+      }
+      const __half2 mm = __hmax2(mx[0], mx[1]);
+      m = static_cast<unsigned>(fmaxf(__low2float(mm), __high2float(mm)));
+    } else {
+      // e4m3 operands: exact for |x| <= 16 (a larger value sets the range
+      // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
+      uint32_t mb = 0;  // per-byte |x| maximum
 #pragma unroll
-      for (int h = 0; h < kLoads; ++h) reload(cc + h);
+      for (int cc = 0; cc < kBK / 16; ++cc) {
+        const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
+        uint32_t W[16];
+        words8(2 * cc, W);
+        words8(2 * cc + 1, W + 8);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
+        store_rows_f8(tre + off, tim + off, W, pol_last);
+        reload(2 * cc);
+        reload(2 * cc + 1);
+      }
+      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
     }
-    sink.finish(p, x, lane);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) {
+      atomicMax(p.amax + x.G, m);
+      if (FMT == kFmtF8 && m > 16) atomicOr(p.status, kStatusRange);
+    }
     if (!pend) {
       pend = &p;
       pend_slot = x.slot;
