@@ -841,8 +841,11 @@ __device__ __forceinline__ uint32_t quad_f8(const uint32_t* W, uint32_t j) {
   const uint32_t e23 = __nv_cvt_halfraw2_to_fp8x2(r23, __NV_SATFINITE, __NV_E4M3);
   return (e01 & 0xffffu) | (e23 << 16);
 }
-// e4m3, both planes.
-__device__ __forceinline__ void store_rows_f8(uint8_t* re, uint8_t* im, const uint32_t* W, uint64_t pol) {
+// e4m3, both planes, with the largest |x| of each byte of `mb`.
+__device__ __forceinline__ void store_rows_f8(uint8_t* re, uint8_t* im, const uint32_t* W, uint32_t& mb,
+                                              uint64_t pol) {
+#pragma unroll
+  for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
   uint32_t vr[8], vi[8];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -959,14 +962,11 @@ __device__ void converter_tma(const Batch& bt, uint32_t buf, uint32_t bar, int c
       // status bit below).  16-sample chunks; rows 2l and 2l + 1 per store.
       uint32_t mb = 0;  // per-byte |x| maximum
 #pragma unroll
-      for (int t = 0; t < kUnitT; ++t) mb = __vmaxu4(mb, __vabs4(w[t]));
-      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
-#pragma unroll
       for (int cc = 0; cc < kUnitT / 16; ++cc) {
         const uint32_t off = tile_off<FMT, SHAPE>(row, cc);
-        const uint32_t* W = w + 16 * cc;
-        store_rows_f8(tre + off, tim + off, W, pol_last);
+        store_rows_f8(tre + off, tim + off, w + 16 * cc, mb, pol_last);
       }
+      m = max(max(mb & 0xffu, (mb >> 8) & 0xffu), max((mb >> 16) & 0xffu, mb >> 24));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -1127,9 +1127,7 @@ __device__ void converter_words(const Batch& bt, int cw, int lane, volatile int*
         uint32_t W[16];
         words8(2 * cc, W);
         words8(2 * cc + 1, W + 8);
-#pragma unroll
-        for (int t = 0; t < 16; ++t) mb = __vmaxu4(mb, __vabs4(W[t]));
-        store_rows_f8(tre + off, tim + off, W, pol_last);
+        store_rows_f8(tre + off, tim + off, W, mb, pol_last);
         reload(2 * cc);
         reload(2 * cc + 1);
       }
