@@ -979,9 +979,9 @@ xc_status channelize_impl(const void* in, xc_dtype in_dtype, int nstation, int n
   const int64_t n = static_cast<int64_t>(nstation) * npol;
   if (n > (1LL << 24) || static_cast<int64_t>(nblock) * nchan > (1LL << 36) / n)
     return fail(XC_ERR_UNSUPPORTED, "problem too large");
-  // One CTA transforms G consecutive inputs of one block (G = 8192 / nchan,
-  // 16384 / nchan for 8-bit output); the input groups form the grid's second
-  // dimension (at most 65535).
+  // The documented bound on the inputs.  (The launch has one CTA per block and
+  // group of 8192 / nchan inputs, or 16384 / nchan for 8-bit output of more than
+  // 512 channels: with T n F <= 2^36 fewer than 2^31.)
   const int64_t G = (out_dtype == XC_CI8 ? 16384 : 8192) / nchan;
   if ((n + G - 1) / G > 65535)
     return fail(XC_ERR_UNSUPPORTED, "nstation*npol=%lld above %lld for nchan=%d",

@@ -359,17 +359,17 @@ cudaError_t launch_fp(const void* in, int in_dt, void* out, int out_dt, int n, i
                       const float* taps, int ntaps, cudaStream_t s) {
   constexpr int F = 1 << LOGF, G = (1 << LOGP) / F;
   const size_t smem = static_cast<size_t>(G) * row_stride(F, G) * sizeof(float2);
-  if ((n + G - 1) / G > 65535) return cudaErrorInvalidConfiguration;
+  // Input groups fastest: the CTAs at work at one time write neighbouring runs
+  // of the same output rows (512 streams, 1024 channels, 500 blocks: 664 -> 640
+  // us).
+  const int64_t ctas = static_cast<int64_t>(T - ntaps + 1) * ((n + G - 1) / G);
+  if (ctas > 0x7fffffff) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(fengine_kernel<LOGF, LOGP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  // Input groups fastest: the CTAs at work at one time write neighbouring runs
-  // of the same output rows (512 streams, 1024 channels, 500 blocks: 664 -> 640
-  // us).  (31 bits hold it: T is an int, and T n F <= 2^36.)
-  const dim3 grid(static_cast<unsigned>(T - ntaps + 1) * static_cast<unsigned>((n + G - 1) / G));
-  fengine_kernel<LOGF, LOGP><<<grid, (1 << LOGP) / kPts, smem, s>>>(in, out, n, T, scale, in_dt,
-                                                                    out_dt, taps, ntaps);
+  fengine_kernel<LOGF, LOGP><<<static_cast<unsigned>(ctas), (1 << LOGP) / kPts, smem, s>>>(
+      in, out, n, T, scale, in_dt, out_dt, taps, ntaps);
   return cudaGetLastError();
 }
 
@@ -382,8 +382,7 @@ cudaError_t launch_fp(const void* in, int in_dt, void* out, int out_dt, int n, i
 template <int LOGF>
 cudaError_t launch_f(const void* in, int in_dt, void* out, int out_dt, int n, int T, float scale,
                      const float* taps, int ntaps, cudaStream_t s) {
-  const bool wide_grid = n > 65535 * ((1 << 13) >> LOGF);  // too many inputs for the smaller CTA's grid
-  if (out_dt == 0 && (LOGF > 9 || wide_grid))
+  if (out_dt == 0 && LOGF > 9)
     return launch_fp<LOGF, 14>(in, in_dt, out, out_dt, n, T, scale, taps, ntaps, s);
   return launch_fp<LOGF, 13>(in, in_dt, out, out_dt, n, T, scale, taps, ntaps, s);
 }
