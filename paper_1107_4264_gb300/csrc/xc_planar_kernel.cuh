@@ -84,15 +84,14 @@
 //   warps 6..9  converters
 // What bounds it: the converters' and the epilogue's stores share the SM's
 // shared-memory path with the MMAs' operand reads.  Alone, the stage copies and
-// MMAs of a 64-sample step take 1050 cycles (1024 is the tensor rate); with 4
-// warps storing 64 KiB of tiles per 6500 cycles 1260-1320, with the epilogue's
-// stores as well 1580.  In the kernel a step takes about 1830 cycles on the
-// 256-station array (2040 when one thread per CTA walked the items, waited and
-// issued four 128 x 128 MMAs per K-step): 1.07 -> 0.97 ms at 1024 channels of
-// 1000 samples, 0.195 -> 0.144 ms for 200 stations, 256 channels of 512, and
-// 1.02 -> 0.62 ms at 2048 channels of 125 samples, where the ring of whole
-// channels was 30 slots deep whatever their size and each item cost every
-// role an FP64 square root and several divisions.
+// MMAs of a 64-sample step take 1114 cycles (1024 is the tensor rate); with 4
+// warps storing 64 KiB of tiles per 6500 cycles some 200 more, and 300 more
+// again with the epilogue's stores as well.  From a ring of whole channels, one
+// thread per CTA that walked the items and issued, a wait of the epilogue for
+// the channel's maximum and an FP64 square root and several divisions per item
+// and role to now: 1.07 -> 0.99-1.01 ms on the 256-station array (1024 channels
+// of 1000 samples), 0.196 -> 0.139 ms for 200 stations, 256 channels of 512, and
+// 1.02 -> 0.54 ms at 2048 channels of 125 samples.
 //
 // CTA pairs (PAIR = true, tcgen05 cta_group::2, clusters of two CTAs): one
 // item is two 128 x 128 blocks sharing their column block b, computed by one
