@@ -43,7 +43,7 @@ N_INTEGRATIONS = 10
 PROFILE_DIR = os.path.join(ROOT, "profiles")
 TRAFFIC_FILE = os.path.join(PROFILE_DIR, "traffic.json")
 MAIN_KERNEL_SOURCES = ["paper_1107_4264_gb300/csrc/xc_planar.cu", "paper_1107_4264_gb300/csrc/xc_planar_kernel.cuh",
-                       "paper_1107_4264_gb300/csrc/xc_ptx.cuh"]
+                       "paper_1107_4264_gb300/csrc/xc_planar_plan.h", "paper_1107_4264_gb300/csrc/xc_ptx.cuh"]
 # Channels of one Large-N integration that the CPU oracle is timed on, in the
 # cpu_baseline leg and in every step of the reference arm alike (64 channels:
 # 64 MB of 8-bit input, 6.9e10 useful ops).
